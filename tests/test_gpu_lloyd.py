@@ -86,3 +86,16 @@ def test_codebook_fitted_to_a_matrix_beats_the_gaussian_one_on_it(orc):
     gauss = load_golden_codebook(K)
     _, mse_gauss = orc.lloyd_assign(z.astype(np.float64), gauss.astype(np.float64))
     assert fit["mse"] < mse_gauss
+
+
+@pytest.mark.parametrize("K,n", [(2, 1027), (32, 511), (512, 513), (1024, 4097), (2048, 9000)])
+def test_tiles_and_chunks_that_do_not_fill(orc, K, n):
+    """Sample counts around the edges of the spatial tiles (512) and sorting chunks (4096), every number of
+    codewords per thread, samples with far outliers, exact duplicates and ties: same codebook as the oracle."""
+    rng = np.random.default_rng(K + n)
+    z = np.round(rng.standard_normal((n, 2)) * 8) / 8 + (rng.standard_normal((n, 2)) * 1e-3) * (rng.random((n, 1)) < 0.7)
+    z[rng.integers(0, n, 5)] *= 1e4
+    ref_cb, ref_mse, ref_iters, _ = orc.train_codebook_on(z, K, 9, 1e-9)
+    out = q.train_codebook_gpu(K, max_iters=9, rel_tol=1e-9, samples=torch.from_numpy(z).to(DEV))
+    assert out["iters"] == ref_iters and np.array_equal(out["codebook"], ref_cb)
+    assert abs(out["mse"] - ref_mse) <= 1e-12 * ref_mse
