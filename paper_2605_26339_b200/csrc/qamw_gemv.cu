@@ -18,6 +18,7 @@
 
 #include "qamw_device.cuh"
 #include "qamw_internal.h"
+#include "qamw_launch.h"
 
 using namespace qamw;
 
@@ -29,6 +30,8 @@ namespace {
 __global__ void gemv_rotate_kernel(const float* x, const float* chan_scale, const int8_t* signs, const float* sigma,
                                    int d_in, int log2b, float2* out) {
     extern __shared__ float v[];
+    chain_release();
+    chain_wait();
     const int vec = blockIdx.x;
     const float* xv = x + size_t(vec) * d_in;
     for (int j = threadIdx.x; j < d_in; j += blockDim.x)
@@ -75,7 +78,9 @@ __global__ void __launch_bounds__(512, 1) gemv_kernel(const GemvArgs a) {
     const uint32_t cb = smem_addr(smem) + 8u * (threadIdx.x & ((1 << a.log2c) - 1));
     const int n_chunks = a.n_pairs >> 4;
     float2* xs = reinterpret_cast<float2*>(smem + ((size_t(a.K) * 8) << a.log2c));
+    chain_release();
     fill_codebook_copies(reinterpret_cast<float2*>(smem), a.codebook, a.K, a.log2c);
+    chain_wait();
     for (int i = threadIdx.x; i < NVEC * 16 * n_chunks; i += blockDim.x) xs[i] = a.xt[i];
     __syncthreads();
     const int words_per_chunk = B / 2;          // 16 B bits = B / 2 words when B is even ...
@@ -245,8 +250,10 @@ __global__ void __launch_bounds__(GemvGeom<NVEC>::kThreads, 1) gemv2_kernel(cons
     };
     auto rows_of = [&](int slice) { return in_group && slice < S && g < n_b ? (n_b - g + G - 1) / G : 0; };
     n_rows = rows_of(s0);
-    if (n_rows > 0) open_slice(s0);  // the first rows travel while the tables are built
+    chain_release();
     fill_codebook_copies(reinterpret_cast<float2*>(smem), a.codebook, a.K, a.log2c);
+    chain_wait();
+    if (n_rows > 0) open_slice(s0);
     __syncthreads();
 
     for (int pass = 0; pass * S_par < S; ++pass) {
@@ -397,8 +404,7 @@ __global__ void __launch_bounds__(GemvGeom<NVEC>::kThreads, 1) gemv2_kernel(cons
     }
 }
 
-int gemv_check(const char* what) {
-    cudaError_t e = cudaGetLastError();
+int gemv_check(const char* what, cudaError_t e) {
     if (e != cudaSuccess) {
         set_cuda_error(what, int(e));
         return QAMW_ERR_CUDA;
@@ -413,8 +419,7 @@ int launch_gemv(const GemvArgs& a, int blocks, size_t smem, cudaStream_t st) {
         set_cuda_error("cudaFuncSetAttribute", int(e));
         return QAMW_ERR_NOMEM;
     }
-    gemv_kernel<NVEC><<<blocks, 512, smem, st>>>(a);
-    return gemv_check("gemv_kernel");
+    return gemv_check("gemv_kernel", launch_chained(gemv_kernel<NVEC>, blocks, 512, smem, st, a));
 }
 
 // cudaFuncSetAttribute once per kernel and device
@@ -451,8 +456,7 @@ int launch_gemv2(const Gemv2Args& a, int sms, cudaStream_t st) {
     int rc = gemv_raise_smem(reinterpret_cast<const void*>(&gemv2_kernel<NVEC>));
     if (rc) return rc;
     const int blocks = std::max(1, std::min(sms, a.d_out));
-    gemv2_kernel<NVEC><<<blocks, threads, smem, st>>>(b);
-    return gemv_check("gemv2_kernel");
+    return gemv_check("gemv2_kernel", launch_chained(gemv2_kernel<NVEC>, blocks, threads, smem, st, b));
 }
 
 int gemv_slices(int d_in) { return (d_in / 32 + 31) / 32; }
@@ -518,9 +522,8 @@ extern "C" int qamw_decode_gemv(const uint8_t* packed, const float* row_norm, co
             return QAMW_ERR_NOMEM;
         }
     }
-    gemv_rotate_kernel<<<n_vec, 1024, size_t(p->d_in) * sizeof(float), st>>>(x, chan_scale, signs, sigma, p->d_in,
-                                                                           ilog2(p->block), xt);
-    rc = gemv_check("gemv_rotate_kernel");
+    rc = gemv_check("gemv_rotate_kernel", launch_chained(gemv_rotate_kernel, n_vec, 1024, size_t(p->d_in) * sizeof(float), st, x,
+                                                         chan_scale, signs, sigma, p->d_in, ilog2(p->block), xt));
     if (rc) return rc;
     GemvArgs a;
     a.packed = packed;

@@ -42,6 +42,7 @@
 
 #include "qamw_device.cuh"
 #include "qamw_internal.h"
+#include "qamw_launch.h"
 
 namespace qamw {
 
@@ -414,6 +415,8 @@ __global__ void __launch_bounds__(kMaxThreads, 1) encode_kernel(const EncodeArgs
     __shared__ double ss_part[2][32];  // per-warp partial sums of squares, two rows in flight
     const RowGeom& g = a.g;
     // dynamic shared memory: [codebook copies][table][index staging: one piece per warp]
+    chain_release();
+    chain_wait();
     const int group = threadIdx.x / g.tg;
     const int tid_g = threadIdx.x - group * g.tg;
     const int lane = threadIdx.x & 31;
@@ -656,6 +659,8 @@ __global__ void __launch_bounds__(kMaxThreads, 1) aux_kernel(const AuxArgs a) {
     const int tid_g = threadIdx.x - group * g.tg;
     double* red = red_all + group * 64;
     const int n_pairs = g.d_in >> 1;
+    chain_release();
+    chain_wait();
 
     f32x2 t[4][4];
     {
@@ -749,6 +754,8 @@ __global__ void __launch_bounds__(32 * kFinishSlices) calibrate_finish_kernel(co
                                                                             int pair_stride, int n_pairs, int d_in,
                                                                             float* sigma_out) {
     __shared__ double part_sum[kFinishSlices][32], part_used[kFinishSlices];
+    chain_release();
+    chain_wait();
     const int lane = threadIdx.x & 31, slice = threadIdx.x >> 5;
     const int k = blockIdx.x * 32 + lane;
     const int per = (total_groups + kFinishSlices - 1) / kFinishSlices;
@@ -827,6 +834,8 @@ __global__ void __launch_bounds__(kMaxThreads, 1) decode_kernel(const DecodeArgs
     const uint32_t cb = smem_addr(smem) + 8u * (threadIdx.x & ((1 << a.log2c) - 1));
     unsigned char* stage = smem + ((size_t(a.K) * 8) << a.log2c) + size_t(threadIdx.x >> 5) * 2 * a.stage_bytes;
 
+    chain_release();
+    chain_wait();
     // first row on its way before anything else
     const long long seg_off = (long long)(tid_g >> 5) * a.seg_bytes;  // of this warp's segment inside a packed row
     const int seg_len = int(max(0LL, min((long long)a.seg_bytes, (long long)a.row_bytes - seg_off)));
@@ -1171,6 +1180,8 @@ template <bool BF16>
 __global__ void __launch_bounds__(kDistThreads, 5) distortion_kernel(const void* W, long long w_row_stride,
                                                                   const __nv_bfloat16* What, const float* act_rms,
                                                                   int d_out, int d_in, int vec, double* out4) {
+    chain_release();
+    chain_wait();
     const long long n_items = dist_item_count(d_out, d_in);
     double s0 = 0, s1 = 0, s2 = 0, s3 = 0;
     dist_items<BF16>(W, w_row_stride, What, act_rms, d_out, d_in, vec, blockIdx.x, n_items, gridDim.x, s0, s1, s2, s3);
@@ -1187,6 +1198,8 @@ constexpr int kDistWideRecords = 64;
 template <bool BF16>
 __global__ void __launch_bounds__(kDistThreads, 5) distortion_batch_kernel(const MatDesc* descs, const int4* spans,
                                                                         const DistReduce red, int n_mats) {
+    chain_release();
+    chain_wait();
     const int4 span = spans[blockIdx.x];
     for (int m = span.x; m <= span.z; ++m) {
         const MatDesc& d = descs[m];
@@ -1279,8 +1292,7 @@ int grid_limit(const qamw_params* p) {
     return (p->flags & QAMW_FLAG_HALF_DEVICE) ? std::max(1, n / 2) : n;
 }
 
-int finish_launch(const char* what) {
-    cudaError_t e = cudaGetLastError();
+int finish_launch(const char* what, cudaError_t e) {
     if (e != cudaSuccess) {
         set_cuda_error(what, int(e));
         return QAMW_ERR_CUDA;
@@ -1312,22 +1324,19 @@ template <bool BF16, int LOG2B_T>
 int launch_encode(const EncodeArgs& a, int blocks, size_t smem, cudaStream_t st) {
     int rc = set_smem(encode_kernel<BF16, LOG2B_T>, smem);
     if (rc) return rc;
-    encode_kernel<BF16, LOG2B_T><<<blocks, a.g.tg * a.g.groups, smem, st>>>(a);
-    return finish_launch("encode_kernel");
+    return finish_launch("encode_kernel", launch_chained(encode_kernel<BF16, LOG2B_T>, blocks, a.g.tg * a.g.groups, smem, st, a));
 }
 
 template <bool BF16, int LOG2B_T>
 int launch_aux(const AuxArgs& a, int blocks, cudaStream_t st) {
-    aux_kernel<BF16, LOG2B_T><<<blocks, a.g.tg * a.g.groups, 0, st>>>(a);
-    return finish_launch("aux_kernel");
+    return finish_launch("aux_kernel", launch_chained(aux_kernel<BF16, LOG2B_T>, blocks, a.g.tg * a.g.groups, 0, st, a));
 }
 
 template <int LOG2B_T>
 int launch_decode(const DecodeArgs& a, int blocks, size_t smem, cudaStream_t st) {
     int rc = set_smem(decode_kernel<LOG2B_T>, smem);
     if (rc) return rc;
-    decode_kernel<LOG2B_T><<<blocks, a.g.tg * a.g.groups, smem, st>>>(a);
-    return finish_launch("decode_kernel");
+    return finish_launch("decode_kernel", launch_chained(decode_kernel<LOG2B_T>, blocks, a.g.tg * a.g.groups, smem, st, a));
 }
 
 #define QAMW_DISPATCH_LOG2B(log2b, CALL)            \
@@ -1349,9 +1358,9 @@ long long distortion_items(int d_out, int d_in) { return dist_item_count(d_out, 
 int distortion_batch_launch(const MatDesc* descs_dev, int n, const void* spans_dev, int blocks, int w_bf16,
                             const DistReduce& red, void* stream) {
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    if (w_bf16) distortion_batch_kernel<true><<<blocks, kDistThreads, 0, st>>>(descs_dev, static_cast<const int4*>(spans_dev), red, n);
-    else distortion_batch_kernel<false><<<blocks, kDistThreads, 0, st>>>(descs_dev, static_cast<const int4*>(spans_dev), red, n);
-    return finish_launch("distortion_batch_kernel");
+    return finish_launch("distortion_batch_kernel",
+                         launch_chained(w_bf16 ? distortion_batch_kernel<true> : distortion_batch_kernel<false>, blocks, kDistThreads, 0,
+                                        st, descs_dev, static_cast<const int4*>(spans_dev), red, n));
 }
 }  // namespace qamw
 
@@ -1619,9 +1628,9 @@ extern "C" int qamw_calibrate(const void* W, const qamw_params* p, const float* 
 #undef CALL
     if (rc) return rc;
     const int n_pairs = p->d_in / 2;
-    calibrate_finish_kernel<<<(n_pairs + 31) / 32, 32 * kFinishSlices, 0, st>>>(a.partial, c.total_groups, c.pair_stride, n_pairs,
-                                                                  p->d_in, sigma_out);
-    return finish_launch("calibrate_finish_kernel");
+    return finish_launch("calibrate_finish_kernel",
+                         launch_chained(calibrate_finish_kernel, (n_pairs + 31) / 32, 32 * kFinishSlices, 0, st, a.partial, c.total_groups,
+                                        c.pair_stride, n_pairs, p->d_in, sigma_out));
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1789,13 +1798,8 @@ extern "C" int qamw_distortion(const void* W, const void* w_hat_bf16, const floa
     const long long items = (long long)((p->d_in + 8 * kDistThreads - 1) / (8 * kDistThreads)) *
                             ((p->d_out + kDistRows - 1) / kDistRows);
     const int blocks = int(std::max<long long>(1, std::min<long long>(32LL * sm_count(), items)));
-    if (p->w_dtype == QAMW_DTYPE_BF16)
-        distortion_kernel<true><<<blocks, kDistThreads, 0, st>>>(W, p->w_row_stride,
-                                                                 static_cast<const __nv_bfloat16*>(w_hat_bf16), act_rms,
-                                                                 p->d_out, p->d_in, vec, out4);
-    else
-        distortion_kernel<false><<<blocks, kDistThreads, 0, st>>>(W, p->w_row_stride,
-                                                                  static_cast<const __nv_bfloat16*>(w_hat_bf16), act_rms,
-                                                                  p->d_out, p->d_in, vec, out4);
-    return finish_launch("distortion_kernel");
+    return finish_launch("distortion_kernel",
+                         launch_chained(p->w_dtype == QAMW_DTYPE_BF16 ? distortion_kernel<true> : distortion_kernel<false>, blocks,
+                                        kDistThreads, 0, st, W, p->w_row_stride, static_cast<const __nv_bfloat16*>(w_hat_bf16), act_rms,
+                                        p->d_out, p->d_in, vec, out4));
 }

@@ -40,6 +40,7 @@
 
 #include "qamw_device.cuh"
 #include "qamw_internal.h"
+#include "qamw_launch.h"
 
 using namespace qamw;
 
@@ -230,10 +231,12 @@ __global__ void __launch_bounds__(NS == 4 ? 512 : 896, 1) decode2_kernel(const D
     unsigned char* stage = smem + ((size_t(a.K) * 8) << a.log2c) + size_t(warp) * kDecodeDepth * a.stage_bytes;
     const uint32_t stage_addr = smem_addr(stage);
 
+    chain_release();
     fill_codebook_copies(reinterpret_cast<float2*>(smem), a.codebook, a.K, a.log2c, true);
     // the 16 bytes after a staged segment are read (and masked away) by the last threads: keep them defined
     if (lane < 4 * kDecodeDepth) reinterpret_cast<uint32_t*>(stage + (lane >> 2) * a.stage_bytes + a.seg_bytes)[lane & 3] = 0u;
     __syncthreads();
+    chain_wait();
 
     // where this thread's index bits sit inside a staged segment: two runs (the lower and the upper
     // physical slots), each 4 B TOP bits long
@@ -470,6 +473,7 @@ __global__ void __launch_bounds__(MAXT, 1) encode2_kernel(const Encode2Args a) {
     __shared__ MatDesc cur;            // the matrix the block is working on (re-read per row: saves registers)
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
 
+    chain_release();
     const int cb_bytes = QUANT != 0 ? 0 : (a.K * 8) << a.log2c;  // only the table search reads codewords
     if (QUANT == 0) fill_codebook_copies(reinterpret_cast<float2*>(smem), a.codebook, a.K, a.log2c);
     unsigned char* table = smem + cb_bytes;
@@ -515,6 +519,7 @@ __global__ void __launch_bounds__(MAXT, 1) encode2_kernel(const Encode2Args a) {
     const unsigned div_magic = 0xffffffffu / unsigned(B4) + 1u;  // ceil(2^32 / (4B))
     constexpr int kEsz = BF16 ? 2 : 4;
 
+    chain_wait();
     const int4 span = block_span(a.spans, a.one.d_out);
     for (int m = span.x; m <= span.z; ++m) {
         // The warps regroup when the row length changes: nobody may still be inside the previous
@@ -775,6 +780,8 @@ constexpr int kFinishSlices = 8;
 __global__ void __launch_bounds__(32 * kFinishSlices) calibrate_finish2_kernel(const MatDesc* descs,
                                                                              const unsigned char* calib_base) {
     __shared__ double part_sum[kFinishSlices][32], part_used[kFinishSlices];
+    chain_release();
+    chain_wait();
     const MatDesc& d = descs[blockIdx.y];
     const int n_pairs = d.d_in >> 1, pair_stride = (n_pairs + 3) & ~3;
     if (int(blockIdx.x) * 32 >= n_pairs) return;
@@ -815,8 +822,7 @@ int pick_copies(int K, size_t budget) {
     return log2c;
 }
 
-int launch_check(const char* what) {
-    cudaError_t e = cudaGetLastError();
+int launch_check(const char* what, cudaError_t e) {
     if (e != cudaSuccess) {
         set_cuda_error(what, int(e));
         return QAMW_ERR_CUDA;
@@ -850,8 +856,7 @@ template <int NS, int LOG2B>
 int launch_decode2(const Decode2Args& a, int blocks, int threads, size_t smem, cudaStream_t st) {
     int rc = raise_smem_limit(reinterpret_cast<const void*>(&decode2_kernel<NS, LOG2B>));
     if (rc) return rc;
-    decode2_kernel<NS, LOG2B><<<blocks, threads, smem, st>>>(a);
-    return launch_check("decode2_kernel");
+    return launch_check("decode2_kernel", launch_chained(decode2_kernel<NS, LOG2B>, blocks, threads, smem, st, a));
 }
 
 template <bool BF16, int LOG2B, int NS, int MAXT>
@@ -859,19 +864,18 @@ int launch_encode2(const Encode2Args& a, int blocks, int threads, size_t smem, c
     if (a.calib_base) {
         int rc = raise_smem_limit(reinterpret_cast<const void*>(&encode2_kernel<BF16, LOG2B, NS, MAXT, 2>));
         if (rc) return rc;
-        encode2_kernel<BF16, LOG2B, NS, MAXT, 2><<<blocks, threads, smem, st>>>(a);
-        return launch_check("encode2_kernel (calibrate)");
+        return launch_check("encode2_kernel (calibrate)",
+                            launch_chained(encode2_kernel<BF16, LOG2B, NS, MAXT, 2>, blocks, threads, smem, st, a));
     }
     if (a.polar_ba >= 0) {
         int rc = raise_smem_limit(reinterpret_cast<const void*>(&encode2_kernel<BF16, LOG2B, NS, MAXT, 1>));
         if (rc) return rc;
-        encode2_kernel<BF16, LOG2B, NS, MAXT, 1><<<blocks, threads, smem, st>>>(a);
-        return launch_check("encode2_kernel (polar)");
+        return launch_check("encode2_kernel (polar)",
+                            launch_chained(encode2_kernel<BF16, LOG2B, NS, MAXT, 1>, blocks, threads, smem, st, a));
     }
     int rc = raise_smem_limit(reinterpret_cast<const void*>(&encode2_kernel<BF16, LOG2B, NS, MAXT, 0>));
     if (rc) return rc;
-    encode2_kernel<BF16, LOG2B, NS, MAXT, 0><<<blocks, threads, smem, st>>>(a);
-    return launch_check("encode2_kernel");
+    return launch_check("encode2_kernel", launch_chained(encode2_kernel<BF16, LOG2B, NS, MAXT, 0>, blocks, threads, smem, st, a));
 }
 
 constexpr size_t kEncode2StaticSmem = 1024;  // ss_part and the current matrix descriptor, rounded up
@@ -1318,18 +1322,18 @@ extern "C" int qamw_calibrate_batch(const qamw_batch* b, void* workspace, size_t
         if (rc) return rc;
     }
     if (!any_general && (fast[0] || fast[1] || fast[2])) {
-        calibrate_finish2_kernel<<<dim3(unsigned((b->cal_all_max_pairs + 31) / 32), unsigned(b->cal_all_n)), 32 * kFinishSlices, 0,
-                                   st>>>(b->d_cal_all, ws);
-        return launch_check("calibrate_finish2_kernel");
+        return launch_check("calibrate_finish2_kernel",
+                            launch_chained(calibrate_finish2_kernel, dim3(unsigned((b->cal_all_max_pairs + 31) / 32), unsigned(b->cal_all_n)),
+                                           32 * kFinishSlices, 0, st, b->d_cal_all, ws));
     }
     for (int c = 0; c < 3; ++c) {
         if (!fast[c]) continue;
         const RowSet& set = b->cal[c];
         int max_pairs = 0;
         for (const MatDesc& d : set.descs) max_pairs = std::max(max_pairs, d.d_in / 2);
-        calibrate_finish2_kernel<<<dim3(unsigned((max_pairs + 31) / 32), unsigned(set.descs.size())), 32 * kFinishSlices, 0,
-                                   st>>>(set.d_descs, ws);
-        const int rc = launch_check("calibrate_finish2_kernel");
+        const int rc = launch_check("calibrate_finish2_kernel",
+                                    launch_chained(calibrate_finish2_kernel, dim3(unsigned((max_pairs + 31) / 32), unsigned(set.descs.size())),
+                                                   32 * kFinishSlices, 0, st, set.d_descs, ws));
         if (rc) return rc;
     }
     return QAMW_OK;
