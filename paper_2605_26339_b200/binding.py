@@ -1,4 +1,5 @@
-"""Thin ctypes binding of libqamw.so (same names as the C ABI in include/qamw.h).
+"""Thin binding of libqamw.so (same names as the C ABI in include/qamw.h): the calls made per matrix or per step go
+through the extension module _qamw, everything else through ctypes.
 
 Only argument marshalling happens here: torch supplies device memory and the
 stream, every step of the codec runs inside the library's CUDA kernels.  There
@@ -118,8 +119,21 @@ def lib() -> C.CDLL:
     return _lib
 
 
+_ext = None
+
+
+def ext():
+    """The extension module of the per-call entry points, on the same libqamw.so as lib()."""
+    global _ext
+    if _ext is None:
+        lib()
+        from . import _qamw
+        _ext = _qamw
+    return _ext
+
+
 def _check(fn: str, rc: int):
-    if rc != QAMW_OK:
+    if rc:
         detail = lib().qamw_last_cuda_error().decode() if rc == ERR_CUDA else ""
         raise QamwError(fn, rc, detail)
 
@@ -314,9 +328,7 @@ def calibrate_workspace_bytes(p: Params) -> int:
 
 def calibrate(W: torch.Tensor, p: Params, chan_scale, signs, sigma_out: torch.Tensor, workspace: torch.Tensor,
               status: Optional[torch.Tensor] = None, stream=None):
-    _check("qamw_calibrate", lib().qamw_calibrate(_dp(W), C.byref(p), _dp(chan_scale), _dp(signs), _dp(sigma_out),
-                                                 _dp(workspace), workspace.numel() * workspace.element_size(),
-                                                 _dp(status), _stream(stream)))
+    _check("qamw_calibrate", ext().calibrate(W, p, chan_scale, signs, sigma_out, workspace, status, stream))
 
 
 STATIC_SCRATCH_BYTES = 16 << 20
@@ -336,19 +348,17 @@ def calibrate_static(W: torch.Tensor, p: Params, chan_scale, signs, sigma_out: t
 
 def encode(W: torch.Tensor, p: Params, chan_scale, signs, sigma, cb: Codebook, packed_out: torch.Tensor,
            row_norm_out: torch.Tensor, status: Optional[torch.Tensor] = None, stream=None):
-    _check("qamw_encode", lib().qamw_encode(_dp(W), C.byref(p), _dp(chan_scale), _dp(signs), _dp(sigma), cb.handle,
-                                           _dp(packed_out), _dp(row_norm_out), _dp(status), _stream(stream)))
+    _check("qamw_encode", ext().encode(W, p, chan_scale, signs, sigma, cb._h, packed_out, row_norm_out, status, stream))
 
 
 def quantize(W: torch.Tensor, p: Params, act_rms, alpha: float, sign_seed: int, cb: Codebook, chan_scale_out,
              signs_out: torch.Tensor, sigma_out: torch.Tensor, packed_out: torch.Tensor, row_norm_out: torch.Tensor,
              workspace: torch.Tensor, status: Optional[torch.Tensor] = None, stream=None):
     """qamw_quantize: channel scales -> signs -> calibrate -> encode in one call (act_rms: host array or None)."""
-    r = None if act_rms is None else _np(act_rms, np.float32)
-    _check("qamw_quantize", lib().qamw_quantize(
-        _dp(W), C.byref(p), None if r is None else r.ctypes.data, alpha, sign_seed, cb.handle, _dp(chan_scale_out),
-        _dp(signs_out), _dp(sigma_out), _dp(packed_out), _dp(row_norm_out), _dp(workspace),
-        workspace.numel() * workspace.element_size(), _dp(status), _stream(stream)))
+    if act_rms is not None and not (type(act_rms) is np.ndarray and act_rms.dtype == np.float32 and act_rms.flags.c_contiguous):
+        act_rms = _np(act_rms, np.float32)
+    _check("qamw_quantize", ext().quantize(W, p, act_rms, alpha, sign_seed, cb._h, chan_scale_out, signs_out, sigma_out, packed_out,
+                                           row_norm_out, workspace, status, stream))
 
 
 def rotate(W: torch.Tensor, p: Params, chan_scale, signs, y_out: torch.Tensor, row_norm_out: torch.Tensor,
@@ -359,19 +369,15 @@ def rotate(W: torch.Tensor, p: Params, chan_scale, signs, y_out: torch.Tensor, r
 
 def decode(packed: torch.Tensor, row_norm: torch.Tensor, chan_scale, signs, sigma, cb: Codebook, p: Params,
            w_hat_out: torch.Tensor, stream=None):
-    _check("qamw_decode", lib().qamw_decode(_dp(packed), _dp(row_norm), _dp(chan_scale), _dp(signs), _dp(sigma),
-                                           cb.handle, C.byref(p), _dp(w_hat_out), _stream(stream)))
+    _check("qamw_decode", ext().decode(packed, row_norm, chan_scale, signs, sigma, cb._h, p, w_hat_out, stream))
 
 
 def decode_gemv(packed: torch.Tensor, row_norm: torch.Tensor, chan_scale, signs, sigma, cb: Codebook, p: Params,
                 x: torch.Tensor, y_out: torch.Tensor, workspace: Optional[torch.Tensor] = None, stream=None):
     """y = W_hat x straight from the packed stream (x: float32 [n_vec, d_in], y_out: float32 [d_out, n_vec])."""
-    n_vec = x.shape[0]
     if workspace is None:
-        workspace = torch.empty(int(lib().qamw_gemv_workspace_bytes(C.byref(p), n_vec)), dtype=torch.uint8, device=x.device)
-    _check("qamw_decode_gemv", lib().qamw_decode_gemv(
-        _dp(packed), _dp(row_norm), _dp(chan_scale), _dp(signs), _dp(sigma), cb.handle, C.byref(p), _dp(x), n_vec,
-        _dp(y_out), _dp(workspace), workspace.numel(), _stream(stream)))
+        workspace = torch.empty(int(lib().qamw_gemv_workspace_bytes(C.byref(p), x.shape[0])), dtype=torch.uint8, device=x.device)
+    _check("qamw_decode_gemv", ext().decode_gemv(packed, row_norm, chan_scale, signs, sigma, cb._h, p, x, y_out, workspace, stream))
 
 
 def measure_fp32_peak() -> float:
@@ -427,17 +433,16 @@ class Batch:
         return int(lib().qamw_batch_workspace_bytes(self._h))
 
     def calibrate(self, workspace: torch.Tensor, status: Optional[torch.Tensor] = None, stream=None):
-        _check("qamw_calibrate_batch", lib().qamw_calibrate_batch(
-            self._h, _dp(workspace), workspace.numel() * workspace.element_size(), _dp(status), _stream(stream)))
+        _check("qamw_calibrate_batch", ext().calibrate_batch(self._h, workspace, status, stream))
 
     def encode(self, status: Optional[torch.Tensor] = None, stream=None):
-        _check("qamw_encode_batch", lib().qamw_encode_batch(self._h, _dp(status), _stream(stream)))
+        _check("qamw_encode_batch", ext().encode_batch(self._h, status, stream))
 
     def decode(self, stream=None):
-        _check("qamw_decode_batch", lib().qamw_decode_batch(self._h, _stream(stream)))
+        _check("qamw_decode_batch", ext().decode_batch(self._h, stream))
 
     def distortion(self, stream=None):
-        _check("qamw_distortion_batch", lib().qamw_distortion_batch(self._h, _stream(stream)))
+        _check("qamw_distortion_batch", ext().distortion_batch(self._h, stream))
 
     def close(self):
         if getattr(self, "_h", None):
