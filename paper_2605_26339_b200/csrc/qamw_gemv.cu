@@ -139,18 +139,24 @@ __device__ __forceinline__ uint32_t lds_word(uint32_t addr) {
 }
 
 // ---------------------------------------------------------------------------------------------
-// Fast path (packed rows 16-byte aligned): column slices in registers.
+// Fast path: column slices in registers.
 //
 // Block b owns rows b, b + gridDim, b + 2 gridDim, ...  Its warps form G row groups of S_par warps; a
-// warp owns one *slice* of 512 pairs (1024 columns) and walks every G-th row of the block.  Lane l
-// holds the rotated, scaled activations of chunk 32 slice + l (16 pairs, 32 floats per vector) in
-// registers -- computed by the warp itself, since a slice is a whole number of Hadamard blocks -- so a
-// pair costs one codeword gather and two fused multiply-adds per vector and nothing else on the
-// shared-memory pipe.  The 64 B bytes of a row's slice arrive through a ring of 16-byte asynchronous
-// copies, several rows ahead (one row in flight per warp leaves the memory system idle).  The slices'
+// warp owns one *slice* of 512 pairs (1024 columns) and walks every G-th row of the block, two at a time.
+// Lane l holds the rotated, scaled activations of chunk 32 slice + l (16 pairs, 32 floats per vector) in
+// registers -- a slice is a whole number of Hadamard blocks, so a warp can rotate its own -- and a
+// pair costs one codeword gather and one packed fused multiply-add per vector.  The 64 B bytes of a
+// row's slice arrive through a ring of 16-byte asynchronous copies, several rows ahead; a row that starts off
+// a 16-byte boundary is copied from the boundary below it and read at an offset.  The slices'
 // partial sums of a tile of rows meet in shared memory behind one block barrier per tile and are
 // added in ascending slice order, so the result does not depend on timing.  Rows longer than the
 // block has warps for are walked in several passes, each adding into y.
+//
+// Bound by the shared-memory pipe: a gather of 32 codewords takes 4 wavefronts from eight copies (K = 2048), the
+// index words 0.75, copies, sums and staging 1, which is 20 us for the 35.4 M pairs of 13824 x 5120 on 148 SMs.  The
+// width B of an index is a template parameter for the bitrates in use, so that every index is cut out at a fixed
+// position, and the two rows of a step share the activations, which keeps 32 gathers in flight with the few warps
+// that 32 registers per vector leave room for.
 // ---------------------------------------------------------------------------------------------
 struct Gemv2Args {
     const uint8_t* packed;
@@ -161,6 +167,7 @@ struct Gemv2Args {
     const float* sigma;
     const float2* codebook;
     const float* row_norm;
+    float4* xt;               // four vectors: rotated activations, see xt_index
     float* y;                 // [d_out][n_vec]
     int d_out, d_in, n_chunks, n_slices, K, B, log2c, log2b;
     int s_par;                // slices walked side by side: ceil(n_slices / passes)
@@ -171,37 +178,150 @@ struct Gemv2Args {
 template <int NVEC>
 struct GemvGeom {
     static constexpr int kThreads = NVEC == 4 ? 320 : NVEC == 2 ? 384 : 512;  // 32 activation registers per thread and vector; warps per scheduler set the register cap
-    static constexpr int kRowBatch = 4 / NVEC;              // rows whose sums are reduced together (four values)
-    static constexpr int kDepth = NVEC == 4 ? 10 : NVEC == 2 ? 8 : 6;  // staged rows per warp: about 45 KB in flight per SM
-    static constexpr int kTileRows = 32;                    // rows per warp between two block barriers
+    static constexpr int kDepth = 6;       // staged rows per warp, in pairs: about 40 KB in flight per SM
+    static constexpr int kTileRows = 32;   // rows per warp between two block barriers
 };
+constexpr int kRotateStage = 32 * 144;     // shared memory of rotate_slice: 32 chunks of 128 bytes, 16 apart
 
-// Sums of four per-lane values over the warp with 6 shuffles instead of 20: the first two steps halve
-// the number of values a lane carries.  Afterwards every lane holds the total of value
-// 2 * bit4(lane) + bit3(lane).
-__device__ __forceinline__ float warp_sum4(const float (&v)[4], int lane) {
-    const bool hi = lane & 16;
-    const float b0 = (hi ? v[2] : v[0]) + __shfl_xor_sync(kFull, hi ? v[0] : v[2], 16);
-    const float b1 = (hi ? v[3] : v[1]) + __shfl_xor_sync(kFull, hi ? v[1] : v[3], 16);
-    const bool h = lane & 8;
-    float c = (h ? b1 : b0) + __shfl_xor_sync(kFull, h ? b0 : b1, 8);
-    c += __shfl_xor_sync(kFull, c, 4);
-    c += __shfl_xor_sync(kFull, c, 2);
-    c += __shfl_xor_sync(kFull, c, 1);
-    return c;
+// Sums of N per-lane values over the warp: while more than one value is left, a step halves the number that a lane
+// carries.  Afterwards the lanes with (lane & (32 / N - 1)) == 0 hold value lane / (32 / N).
+template <int N>
+__device__ __forceinline__ float warp_sums(float (&v)[N], int lane) {
+    int m = 16;
+#pragma unroll
+    for (int n = N / 2; n >= 1; n /= 2, m /= 2) {
+        const bool up = lane & m;
+#pragma unroll
+        for (int i = 0; i < n; ++i) {
+            const float keep = up ? v[i + n] : v[i], send = up ? v[i] : v[i + n];
+            v[i] = keep + __shfl_xor_sync(kFull, send, m);
+        }
+    }
+    for (; m >= 1; m /= 2) v[0] += __shfl_xor_sync(kFull, v[0], m);
+    return v[0];
 }
 
 template <int N>
 __device__ __forceinline__ void cp_async_wait_pending() {
     asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
+// 16 bytes of shared memory, of which the first n come from global memory (nothing else is read) and the rest is zero
+__device__ __forceinline__ void cp_async_upto16(unsigned char* dst, const unsigned char* src, int n) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_addr(dst)), "l"(src), "r"(n) : "memory");
+}
 
+// Rotated activations of one slice, by one warp: lane l gets chunk 32 slice + l of each vector,
+// xr[v][i] = sigma_k (F S D_s^-1 x_v) at pair k = 16 chunk + i; zero beyond the row.  The columns are read
+// lane by lane along the row and handed to their chunks through `stage` (read at a chunk per lane they
+// took 32 wavefronts a load and 5 of the 30 us of 13824 x 5120).
 template <int NVEC>
+__device__ __forceinline__ void rotate_slice(const Gemv2Args& a, int slice, int v0, unsigned char* stage, int lane, f32x2 (&xr)[NVEC][16]) {
+    const int col0 = 1024 * slice, chunk = 32 * slice + lane;
+    float tj[32];  // sign_j / s_j of columns col0 + 128 e + 4 lane + i
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+        const int col = col0 + 128 * e + 4 * lane;
+        const bool in = col < a.d_in;
+        const uint32_t sw = in ? __ldg(reinterpret_cast<const uint32_t*>(a.signs + col)) : 0u;
+        float4 q = make_float4(1.f, 1.f, 1.f, 1.f);
+        if (in && a.chan_scale) q = __ldg(reinterpret_cast<const float4*>(a.chan_scale + col));
+        tj[4 * e] = __fdividef(float(int(int8_t(sw & 0xffu))), q.x);
+        tj[4 * e + 1] = __fdividef(float(int(int8_t((sw >> 8) & 0xffu))), q.y);
+        tj[4 * e + 2] = __fdividef(float(int(int8_t((sw >> 16) & 0xffu))), q.z);
+        tj[4 * e + 3] = __fdividef(float(int(int8_t(sw >> 24))), q.w);
+    }
+    float4 sg4[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+        sg4[e] = chunk < a.n_chunks ? __ldg(reinterpret_cast<const float4*>(a.sigma + 16 * chunk) + e) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int v = 0; v < NVEC; ++v) {
+        const float* x = a.x + size_t(v0 + v) * a.d_in;
+        __syncwarp();  // the staging memory is free
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            const int col = col0 + 128 * e + 4 * lane;
+            float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (col < a.d_in) q = __ldg(reinterpret_cast<const float4*>(x + col));
+            *reinterpret_cast<float4*>(stage + (4 * e + (lane >> 3)) * 144 + (lane & 7) * 16) =
+                make_float4(q.x * tj[4 * e], q.y * tj[4 * e + 1], q.z * tj[4 * e + 2], q.w * tj[4 * e + 3]);
+        }
+        __syncwarp();
+        float t[32];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            const float4 q = *reinterpret_cast<const float4*>(stage + lane * 144 + 16 * e);
+            t[4 * e] = q.x;
+            t[4 * e + 1] = q.y;
+            t[4 * e + 2] = q.z;
+            t[4 * e + 3] = q.w;
+        }
+#pragma unroll
+        for (int st = 0; st < 5; ++st) {  // butterflies inside the lane's 32 columns
+            if (st < a.log2b) {
+                const int h = 1 << st;
+#pragma unroll
+                for (int e = 0; e < 32; ++e)
+                    if (!(e & h)) {
+                        const float lo = t[e], up = t[e + h];
+                        t[e] = lo + up;
+                        t[e + h] = lo - up;
+                    }
+            }
+        }
+        for (int st = 5; st < a.log2b; ++st) {  // blocks wider than a chunk: lanes 2^(st-5) apart
+            const int m = 1 << (st - 5);
+            const bool upper = lane & m;
+#pragma unroll
+            for (int e = 0; e < 32; ++e) {
+                const float o = __shfl_xor_sync(kFull, t[e], m);
+                t[e] = upper ? o - t[e] : t[e] + o;
+            }
+        }
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const float sg[4] = {sg4[e].x * a.inv_sqrt_b, sg4[e].y * a.inv_sqrt_b, sg4[e].z * a.inv_sqrt_b, sg4[e].w * a.inv_sqrt_b};
+#pragma unroll
+            for (int i = 0; i < 4; ++i) xr[v][4 * e + i] = pack2(t[8 * e + 2 * i] * sg[i], t[8 * e + 2 * i + 1] * sg[i]);
+        }
+    }
+    __syncwarp();
+}
+
+// Where the rotated activations of four vectors lie: by slice, vector and group of two pairs, one float4 per live
+// lane, so that a warp reads whole lines and the whole takes no more than the vectors themselves.
+__device__ __forceinline__ size_t xt_index(const Gemv2Args& a, int slice, int v, int j, int lane) {
+    return size_t(slice) * 1024 + (v * 8 + j) * min(32, a.n_chunks - 32 * slice) + lane;
+}
+constexpr int kRotateWarps = 4;
+__global__ void __launch_bounds__(32 * kRotateWarps) gemv_rotate4_kernel(const Gemv2Args a) {
+    __shared__ __align__(16) unsigned char stage[kRotateWarps][kRotateStage];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;  // a warp per vector, a block per slice
+    chain_release();
+    chain_wait();
+    f32x2 xr[1][16];
+    rotate_slice<1>(a, blockIdx.x, warp, stage[warp], lane, xr);
+    if (32 * int(blockIdx.x) + lane >= a.n_chunks) return;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        float4 o;
+        unpack2(xr[0][2 * j], o.x, o.y);
+        unpack2(xr[0][2 * j + 1], o.z, o.w);
+        a.xt[xt_index(a, blockIdx.x, warp, j, lane)] = o;
+    }
+}
+
+// BT: bits of an index, or 0 for the widths below 6, read from the arguments
+template <int NVEC, int BT>
 __global__ void __launch_bounds__(GemvGeom<NVEC>::kThreads, 1) gemv2_kernel(const Gemv2Args a) {
-    constexpr int RB = GemvGeom<NVEC>::kRowBatch, D = GemvGeom<NVEC>::kDepth;
+    constexpr int R = 2, D = GemvGeom<NVEC>::kDepth;
+    constexpr int BMAX = BT ? BT : 5;
+    constexpr bool ODD = BT == 0 || BT % 2;                         // a chunk may start in the middle of a word
+    constexpr int NB = (16 * BMAX + 31) / 32;                      // words of a lane's 16 indices,
+    constexpr int NW = (16 * BMAX + (ODD ? 16 : 0) + 31) / 32;     // and of what they are cut from
     extern __shared__ __align__(16) unsigned char smem[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
-    const int B = a.B;
+    const int B = BT ? BT : a.B;
     const uint32_t mask = (1u << B) - 1u;
     const uint32_t cb_stride = 8u << a.log2c;
     const uint32_t cb = smem_addr(smem) + 8u * (threadIdx.x & ((1 << a.log2c) - 1));
@@ -211,7 +331,6 @@ __global__ void __launch_bounds__(GemvGeom<NVEC>::kThreads, 1) gemv2_kernel(cons
     const int S = a.n_slices;
     const int S_par = a.s_par;                // slices walked side by side
     const int G = n_warps / S_par;            // row groups
-    const bool in_group = warp < S_par * G;
     const int s0 = warp % S_par, g = warp / S_par;
     constexpr int JT = GemvGeom<NVEC>::kTileRows;
     const int TI = JT * G;                    // rows of the block per tile
@@ -221,169 +340,123 @@ __global__ void __launch_bounds__(GemvGeom<NVEC>::kThreads, 1) gemv2_kernel(cons
     float* ps_base = reinterpret_cast<float*>(smem + ((size_t(a.K) * 8) << a.log2c) + size_t(n_warps) * D * a.stage_bytes);
     // where the lane's 16 B index bits start inside a staged segment
     const uint32_t w_off = 4u * ((uint32_t(B) * uint32_t(lane)) >> 1), sh = ((uint32_t(B) * uint32_t(lane)) & 1u) * 16u;
-    const int row_bytes = int(((((long long)(a.d_in >> 1)) * B + 7) / 8 + 15) & ~15LL);  // <= stride (a multiple of 16)
+    const int row_bytes = int((((long long)(a.d_in >> 1)) * B + 7) / 8 + 3) & ~3;  // <= stride (a multiple of 4)
     const long long src_step = (long long)G * int(gridDim.x) * a.stride;
-    int n_rows = 0;  // rows of the current pass for this warp
 
-    // the ring of a warp: D staged rows of its slice, one commit group per row (empty past the end)
-    const unsigned char* src = nullptr;
-    bool copy0 = false, copy1 = false;
-    int issued = 0;
-    auto issue_row = [&]() {
-        if (issued < n_rows) {
-            unsigned char* dst = stage + (issued % D) * a.stage_bytes;
-            if (copy0) cp_async(dst + (lane << 4), src + (lane << 4), 4);
-            if (copy1) cp_async(dst + ((lane + 32) << 4), src + ((lane + 32) << 4), 4);
-            src += src_step;
-        }
-        ++issued;
-        cp_async_commit();
-    };
-    auto open_slice = [&](int slice) {
-        const long long seg_off = (long long)slice * a.seg_bytes;
-        const int n16 = max(0, min(a.seg_bytes, row_bytes - int(seg_off))) >> 4;  // at most 48 pieces of 16 bytes
-        copy0 = lane < n16;
-        copy1 = lane + 32 < n16;
-        src = a.packed + ((long long)blockIdx.x + (long long)gridDim.x * g) * a.stride + seg_off;
-        issued = 0;
-        for (int i = 0; i < D - 1; ++i) issue_row();
-    };
-    auto rows_of = [&](int slice) { return in_group && slice < S && g < n_b ? (n_b - g + G - 1) / G : 0; };
-    n_rows = rows_of(s0);
     chain_release();
     fill_codebook_copies(reinterpret_cast<float2*>(smem), a.codebook, a.K, a.log2c);
     chain_wait();
-    if (n_rows > 0) open_slice(s0);
     __syncthreads();
 
     for (int pass = 0; pass * S_par < S; ++pass) {
         const int slice = pass * S_par + s0;
         const int n_live = min(S_par, S - pass * S_par);
-        if (pass > 0) {
-            __syncthreads();  // the previous pass's sums have been read; its last rows too
-            n_rows = rows_of(slice);
-            if (n_rows > 0) open_slice(slice);
-        }
-        const int chunk = slice * 32 + lane;
-        const bool valid = n_rows > 0 && chunk < a.n_chunks;
-        // rotated activations of this lane's chunk: xr[v][2 i], xr[v][2 i + 1] = sigma_k (F S D_s^-1 x_v) at pair k = 16 chunk + i
-        float xr[NVEC][32];
-        if (valid) {
-            const int col0 = 32 * chunk;
-            const uint4* sp = reinterpret_cast<const uint4*>(a.signs + col0);
-            const uint4 s0 = __ldg(sp), s1 = __ldg(sp + 1);
-            const uint32_t sw[8] = {s0.x, s0.y, s0.z, s0.w, s1.x, s1.y, s1.z, s1.w};  // one sign byte per column
-#pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                float tj[4];  // sign_j / s_j
-#pragma unroll
-                for (int i = 0; i < 4; ++i) tj[i] = float(int(int8_t((sw[e] >> (8 * i)) & 0xffu)));
-                if (a.chan_scale) {
-                    const float4 q = __ldg(reinterpret_cast<const float4*>(a.chan_scale + col0) + e);
-                    tj[0] = __fdividef(tj[0], q.x);
-                    tj[1] = __fdividef(tj[1], q.y);
-                    tj[2] = __fdividef(tj[2], q.z);
-                    tj[3] = __fdividef(tj[3], q.w);
-                }
-#pragma unroll
-                for (int v = 0; v < NVEC; ++v) {
-                    const float4 q = __ldg(reinterpret_cast<const float4*>(a.x + size_t(v) * a.d_in + col0) + e);
-                    xr[v][4 * e] = q.x * tj[0];
-                    xr[v][4 * e + 1] = q.y * tj[1];
-                    xr[v][4 * e + 2] = q.z * tj[2];
-                    xr[v][4 * e + 3] = q.w * tj[3];
-                }
-            }
-        } else {
-#pragma unroll
-            for (int v = 0; v < NVEC; ++v)
-#pragma unroll
-                for (int e = 0; e < 32; ++e) xr[v][e] = 0.f;
-        }
-#pragma unroll
-        for (int v = 0; v < NVEC; ++v) {
-            float* t = xr[v];
-#pragma unroll
-            for (int st = 0; st < 5; ++st) {  // butterflies inside the lane's 32 columns
-                if (st < a.log2b) {
-                    const int h = 1 << st;
-#pragma unroll
-                    for (int e = 0; e < 32; ++e)
-                        if (!(e & h)) {
-                            const float lo = t[e], up = t[e + h];
-                            t[e] = lo + up;
-                            t[e + h] = lo - up;
-                        }
-                }
-            }
-            for (int st = 5; st < a.log2b; ++st) {  // blocks wider than a chunk: lanes 2^(st-5) apart
-                const int m = 1 << (st - 5);
-                const bool upper = lane & m;
-#pragma unroll
-                for (int e = 0; e < 32; ++e) {
-                    const float o = __shfl_xor_sync(kFull, t[e], m);
-                    t[e] = upper ? o - t[e] : t[e] + o;
-                }
-            }
-        }
-        if (valid) {
-            const float4* gp = reinterpret_cast<const float4*>(a.sigma + 16 * chunk);
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const float4 q = __ldg(gp + e);
-                const float sg[4] = {q.x * a.inv_sqrt_b, q.y * a.inv_sqrt_b, q.z * a.inv_sqrt_b, q.w * a.inv_sqrt_b};
+        const int n_rows = slice < S && g < n_b ? (n_b - g + G - 1) / G : 0;  // of this warp
+        if (pass > 0) __syncthreads();  // the previous pass's sums have been read
+        const long long seg_off = (long long)slice * a.seg_bytes;
+        const int seg_len = max(0, min(a.seg_bytes, row_bytes - int(seg_off)));
+        const unsigned char* src = a.packed + ((long long)blockIdx.x + (long long)gridDim.x * g) * a.stride + seg_off;
+        int off = int(reinterpret_cast<uintptr_t>(src) & 15);  // of the current row from the 16-byte boundary below it
+        f32x2 xr[NVEC][16];
+        if (n_rows > 0) {
+            if constexpr (NVEC == 4) {
+                const bool valid = 32 * slice + lane < a.n_chunks;
 #pragma unroll
                 for (int v = 0; v < NVEC; ++v)
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        xr[v][8 * e + 2 * i] *= sg[i];
-                        xr[v][8 * e + 2 * i + 1] *= sg[i];
+                    for (int j = 0; j < 8; ++j) {
+                        const float4 q = valid ? __ldcg(a.xt + xt_index(a, slice, v, j, lane)) : make_float4(0.f, 0.f, 0.f, 0.f);
+                        xr[v][2 * j] = pack2(q.x, q.y);
+                        xr[v][2 * j + 1] = pack2(q.z, q.w);
                     }
+            } else {
+                // the first rows come to the L2 while the ring's memory serves the rotation
+                for (int i = 0; i < min(n_rows, D) && lane * 128 < seg_len + 15; ++i)
+                    asm volatile("prefetch.global.L2 [%0];" ::"l"(src + i * src_step + min(lane * 128, seg_len - 1)));
+                rotate_slice<NVEC>(a, slice, 0, stage, lane, xr);
             }
         }
+        // the ring of a warp: D staged rows of its slice, one commit group per R rows (empty past the end)
+        int issued = 0;
+        auto issue = [&]() {
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                if (issued < n_rows) {
+                    unsigned char* dst = stage + (issued % D) * a.stage_bytes + (lane << 4);
+                    const int mis = int(reinterpret_cast<uintptr_t>(src) & 15);
+                    const unsigned char* from = src - mis + (lane << 4);
+                    const int left = mis + seg_len - (lane << 4);  // at most 49 pieces: two per lane
+                    if (left > 0) cp_async_upto16(dst, from, min(16, left));
+                    if (left > 512) cp_async_upto16(dst + 512, from + 512, min(16, left - 512));
+                    src += src_step;
+                }
+                ++issued;
+            }
+            cp_async_commit();
+        };
+        for (int i = 0; i < D / R - 1; ++i) issue();
 
         for (int tile = 0; tile < n_tiles; ++tile) {
             float* ps = ps_base + (tile & 1) * (S_par * TI * NVEC);  // [slice][row of the tile][vector]
-            for (int jj = 0; jj < JT; jj += RB) {
+            for (int jj = 0; jj < JT; jj += R) {
                 const int it = tile * JT + jj;  // this warp's row counter
                 if (it >= n_rows) break;
-                float acc[4] = {0.f, 0.f, 0.f, 0.f};  // RB rows x NVEC vectors
+                cp_async_wait_pending<D / R - 2>();
+                __syncwarp();  // every lane's part of these rows has landed; the buffers refilled next are no longer read
+                issue();
+                // R rows at once; past the last row of the warp the sums of stale bytes are computed and not stored
+                uint32_t win[R][NB + 1];
 #pragma unroll
-                for (int r = 0; r < RB; ++r) {
-                    if (it + r >= n_rows) break;
-                    cp_async_wait_pending<D - 2>();
-                    __syncwarp();  // every lane's part of this row has landed; the buffer refilled next is no longer read
-                    issue_row();
-                    const uint32_t in = stage_addr + uint32_t(((it + r) % D) * a.stage_bytes) + w_off;
-                    uint32_t word[6], win[6];
+                for (int r = 0; r < R; ++r) {
+                    const uint32_t in = stage_addr + uint32_t(((it + r) % D) * a.stage_bytes) + w_off + uint32_t(off);
+                    off = (off + int(src_step & 15)) & 15;
+                    uint32_t word[NW + 1];
 #pragma unroll
-                    for (int i = 0; i < 6; ++i) word[i] = lds_word(in + 4u * i);
+                    for (int i = 0; i < NW; ++i) word[i] = lds_word(in + 4u * i);
+                    word[NW] = 0u;
 #pragma unroll
-                    for (int i = 0; i < 5; ++i) win[i] = __funnelshift_r(word[i], word[i + 1], sh);
-                    win[5] = word[5] >> sh;
+                    for (int i = 0; i < NB; ++i) win[r][i] = ODD ? __funnelshift_r(word[i], word[i + 1], sh) : word[i];
+                    win[r][NB] = 0u;
+                }
+                f32x2 acc[R][NVEC];
 #pragma unroll
-                    for (int t = 0; t < 8; ++t) {  // two indices per step of 2 B bits
-                        const uint32_t i0 = win[0] & mask, i1 = (win[0] >> B) & mask;
-                        const float2 c0 = lds_f32x2(cb + i0 * cb_stride), c1 = lds_f32x2(cb + i1 * cb_stride);
+                for (int r = 0; r < R; ++r)
 #pragma unroll
-                        for (int v = 0; v < NVEC; ++v) {
-                            float sum = acc[r * NVEC + v];
-                            sum = fmaf(c0.x, xr[v][4 * t], sum);
-                            sum = fmaf(c0.y, xr[v][4 * t + 1], sum);
-                            sum = fmaf(c1.x, xr[v][4 * t + 2], sum);
-                            sum = fmaf(c1.y, xr[v][4 * t + 3], sum);
-                            acc[r * NVEC + v] = sum;
+                    for (int v = 0; v < NVEC; ++v) acc[r][v] = 0ull;
+#pragma unroll
+                for (int t = 0; t < 16; ++t) {
+#pragma unroll
+                    for (int r = 0; r < R; ++r) {
+                        uint32_t id;
+                        if (BT) {
+                            constexpr int W = BT ? BT : 1;
+                            const int w = t * W / 32, s = t * W % 32;
+                            id = (s + W <= 32 ? win[r][w] >> s : __funnelshift_r(win[r][w], win[r][w + 1 <= NB ? w + 1 : NB], s)) & mask;
+                        } else {
+                            const unsigned bit = unsigned(t * B);
+                            const uint32_t lo = bit < 32u ? win[r][0] : bit < 64u ? win[r][1] : win[r][2];
+                            const uint32_t hi = bit < 32u ? win[r][1] : bit < 64u ? win[r][2] : win[r][3 <= NB ? 3 : NB];
+                            id = __funnelshift_r(lo, hi, bit & 31u) & mask;
                         }
-                        if (t < 7) {
+                        const float2 c = lds_f32x2(cb + id * cb_stride);
+                        const f32x2 c2 = pack2(c.x, c.y);
 #pragma unroll
-                            for (int i = 0; i < 5; ++i) win[i] = __funnelshift_r(win[i], win[i + 1], 2 * B);
-                            win[5] >>= 2 * B;
-                        }
+                        for (int v = 0; v < NVEC; ++v) acc[r][v] = fma2(c2, xr[v][t], acc[r][v]);
                     }
                 }
-                const float total = warp_sum4(acc, lane);
-                if ((lane & 7) == 0) {  // lanes 0, 8, 16, 24 hold values 0, 1, 2, 3
-                    const int id = lane >> 3, r = id / NVEC, v = id - r * NVEC;
+                float sums[R * NVEC];
+#pragma unroll
+                for (int r = 0; r < R; ++r)
+#pragma unroll
+                    for (int v = 0; v < NVEC; ++v) {
+                        float p, q;
+                        unpack2(acc[r][v], p, q);
+                        sums[r * NVEC + v] = p + q;
+                    }
+                const float total = warp_sums<R * NVEC>(sums, lane);
+                constexpr int W = 32 / (R * NVEC);
+                if (lane % W == 0) {
+                    const int id = lane / W, r = id / NVEC, v = id - r * NVEC;
                     if (it + r < n_rows) ps[(s0 * TI + (jj + r) * G + g) * NVEC + v] = total;
                 }
             }
@@ -441,22 +514,39 @@ int gemv_raise_smem(const void* kernel) {
     return QAMW_OK;
 }
 
+template <int NVEC, int BT>
+int launch_gemv2_b(const Gemv2Args& a, int blocks, int threads, size_t smem, cudaStream_t st) {
+    int rc = gemv_raise_smem(reinterpret_cast<const void*>(&gemv2_kernel<NVEC, BT>));
+    if (rc) return rc;
+    return gemv_check("gemv2_kernel", launch_chained(gemv2_kernel<NVEC, BT>, blocks, threads, smem, st, a));
+}
+
 template <int NVEC>
 int launch_gemv2(const Gemv2Args& a, int sms, cudaStream_t st) {
     constexpr int kThreads = GemvGeom<NVEC>::kThreads, kWarps = kThreads / 32;
     // as many passes as the warps of a block require, the slices spread evenly over them
     const int passes = (a.n_slices + kWarps - 1) / kWarps;
-    const int S_par = (a.n_slices + passes - 1) / passes, G = kWarps / S_par;
+    const int S_par = (a.n_slices + passes - 1) / passes;
+    const int blocks = std::max(1, std::min(sms, a.d_out));
+    const int n_b = (a.d_out + blocks - 1) / blocks;  // rows of a block
+    const int G = std::max(1, std::min(kWarps / S_par, n_b));
     Gemv2Args b = a;
     b.s_par = S_par;
+    b.log2c = pick_copies(a.K, (long long)n_b * (a.d_in / 64), size_t(128) * 1024);
     const int threads = 32 * S_par * G;
     const size_t sums = size_t(2) * S_par * GemvGeom<NVEC>::kTileRows * G * NVEC * sizeof(float);
-    const size_t smem = (size_t(a.K) * 8 << a.log2c) + size_t(S_par * G) * GemvGeom<NVEC>::kDepth * a.stage_bytes + sums;
+    const size_t smem = (size_t(a.K) * 8 << b.log2c) + size_t(S_par * G) * GemvGeom<NVEC>::kDepth * a.stage_bytes + sums;
     if (smem > kSmemLimit) return QAMW_ERR_NOMEM;
-    int rc = gemv_raise_smem(reinterpret_cast<const void*>(&gemv2_kernel<NVEC>));
-    if (rc) return rc;
-    const int blocks = std::max(1, std::min(sms, a.d_out));
-    return gemv_check("gemv2_kernel", launch_chained(gemv2_kernel<NVEC>, blocks, threads, smem, st, b));
+    switch (a.B) {
+        case 6: return launch_gemv2_b<NVEC, 6>(b, blocks, threads, smem, st);
+        case 7: return launch_gemv2_b<NVEC, 7>(b, blocks, threads, smem, st);
+        case 8: return launch_gemv2_b<NVEC, 8>(b, blocks, threads, smem, st);
+        case 9: return launch_gemv2_b<NVEC, 9>(b, blocks, threads, smem, st);
+        case 10: return launch_gemv2_b<NVEC, 10>(b, blocks, threads, smem, st);
+        case 11: return launch_gemv2_b<NVEC, 11>(b, blocks, threads, smem, st);
+        case 12: return launch_gemv2_b<NVEC, 12>(b, blocks, threads, smem, st);
+        default: return launch_gemv2_b<NVEC, 0>(b, blocks, threads, smem, st);
+    }
 }
 
 int gemv_slices(int d_in) { return (d_in / 32 + 31) / 32; }
@@ -465,7 +555,7 @@ int gemv_slices(int d_in) { return (d_in / 32 + 31) / 32; }
 
 extern "C" size_t qamw_gemv_workspace_bytes(const qamw_params* p, int n_vec) {
     if (check_matrix_params(p) || n_vec < 1) return 0;
-    return size_t(n_vec) * size_t(p->d_in) * sizeof(float);  // the layout-agnostic kernel's rotated activations
+    return size_t(n_vec) * size_t(p->d_in) * sizeof(float);  // rotated activations
 }
 
 extern "C" int qamw_decode_gemv(const uint8_t* packed, const float* row_norm, const float* chan_scale,
@@ -485,9 +575,9 @@ extern "C" int qamw_decode_gemv(const uint8_t* packed, const float* row_norm, co
     if (p->d_out == 0) return QAMW_OK;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const bool general = (p->flags & QAMW_FLAG_GENERAL_KERNELS) != 0;
-    if (!general && reinterpret_cast<uintptr_t>(packed) % 16 == 0 && p->packed_row_stride % 16 == 0 &&
-        reinterpret_cast<uintptr_t>(x) % 16 == 0) {
-        Gemv2Args g;
+    auto aligned16 = [](const void* v) { return reinterpret_cast<uintptr_t>(v) % 16 == 0; };
+    if (!general && aligned16(packed) && aligned16(workspace) && aligned16(x) && aligned16(chan_scale) && aligned16(signs) && aligned16(sigma)) {
+        Gemv2Args g{};
         g.packed = packed;
         g.stride = p->packed_row_stride;
         g.x = x;
@@ -504,13 +594,18 @@ extern "C" int qamw_decode_gemv(const uint8_t* packed, const float* row_norm, co
         g.K = p->K;
         g.B = ilog2(p->K);
         g.log2b = ilog2(p->block);
-        g.log2c = 4;
-        while (g.log2c > 0 && (size_t(p->K) * 8 << g.log2c) > size_t(128) * 1024) --g.log2c;
         g.seg_bytes = 64 * g.B;
-        g.stage_bytes = (g.seg_bytes + 32 + 127) & ~127;  // a lane reads six words from its first one
+        // 12 bytes before a row off its boundary, 4 read past the last lane's indices; the ring also serves rotate_slice
+        g.stage_bytes = std::max((g.seg_bytes + 32 + 127) & ~127, kRotateStage / GemvGeom<1>::kDepth);
+        g.xt = static_cast<float4*>(workspace);
         g.inv_sqrt_b = 1.0f / std::sqrt(float(p->block));
         const int sms = sm_count();
-        return n_vec == 1 ? launch_gemv2<1>(g, sms, st) : n_vec == 2 ? launch_gemv2<2>(g, sms, st) : launch_gemv2<4>(g, sms, st);
+        if (n_vec == 1) return launch_gemv2<1>(g, sms, st);
+        if (n_vec == 2) return launch_gemv2<2>(g, sms, st);
+        // Four vectors are rotated once by a small kernel of its own: done by every block, as for one or two, it
+        // costs 650 wavefronts per warp and the registers that the rows need.
+        rc = gemv_check("gemv_rotate4_kernel", launch_chained(gemv_rotate4_kernel, g.n_slices, 32 * kRotateWarps, 0, st, g));
+        return rc ? rc : launch_gemv2<4>(g, sms, st);
     }
     const size_t x_bytes = size_t(n_vec) * p->d_in * sizeof(float);
     if (x_bytes + size_t(p->K) * 8 > kSmemLimit || size_t(p->d_in) * sizeof(float) > kSmemLimit) return QAMW_ERR_NOMEM;

@@ -106,6 +106,11 @@ int rows_encode(const MatDesc* descs_dev, const MatDesc* descs_host, int n, cons
                 int block, int K, int w_bf16, const ::qamw_codebook* cb, uint32_t flags, int32_t* status, void* stream,
                 void* calib_base = nullptr);  // calib_base: run the calibration pass instead (cb may be NULL)
 int sm_count();
+// log2 of the number of bank-separated codebook copies a block keeps in shared memory (at most 16, and at most
+// `budget` bytes) when it makes `gathers` warp-wide codeword reads in all.  A copy costs its stores (one wavefront per 128
+// bytes), more copies save wavefronts per read: with 16 copies a read takes 2 wavefronts, with 8, 4, 2 and 1
+// about 4, 5.4, 5.9 and 6.2 (16 random lanes on 16 pairs of banks, twice).
+int pick_copies(int K, long long gathers, size_t budget);
 int check_matrix_params(const qamw_params* p);
 long long distortion_items(int d_out, int d_in);  // work items of the distortion kernel for one matrix
 // zeroes every matrix's four sums, then one launch over all matrices (spans of the concatenated item list)

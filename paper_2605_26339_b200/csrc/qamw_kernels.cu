@@ -64,6 +64,20 @@ int sm_count() {
     return cached > 0 ? cached : 148;
 }
 
+int pick_copies(int K, long long gathers, size_t budget) {
+    static const double per_read[5] = {6.2, 5.9, 5.4, 4.0, 2.0};
+    int best = 0;
+    double best_cost = 0.0;
+    for (int c = 0; c <= 4 && (c == 0 || (size_t(K) * 8 << c) <= budget); ++c) {
+        const double cost = double(size_t(K) * 8 << c) / 128.0 + double(gathers) * per_read[c];
+        if (c == 0 || cost < best_cost) {
+            best = c;
+            best_cost = cost;
+        }
+    }
+    return best;
+}
+
 }  // namespace qamw
 
 using namespace qamw;

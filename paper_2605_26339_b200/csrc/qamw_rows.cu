@@ -816,12 +816,6 @@ __global__ void __launch_bounds__(32 * kFinishSlices) calibrate_finish2_kernel(c
 // ---------------------------------------------------------------------------------------------
 inline bool aligned(const void* p, uintptr_t a) { return reinterpret_cast<uintptr_t>(p) % a == 0; }
 
-int pick_copies(int K, size_t budget) {
-    int log2c = 4;
-    while (log2c > 0 && (size_t(K) * 8 << log2c) > budget) --log2c;
-    return log2c;
-}
-
 int launch_check(const char* what, cudaError_t e) {
     if (e != cudaSuccess) {
         set_cuda_error(what, int(e));
@@ -940,7 +934,7 @@ int rows_decode(const MatDesc* descs_dev, const MatDesc* descs_host, int n, cons
     a.stage_bytes = (a.seg_bytes + 16 + 127) & ~127;  // 128-byte aligned ring buffers
     a.inv_sqrt_b = float(1.0 / std::sqrt(double(block)));
     const size_t stage_total = size_t(kWarps) * kDecodeDepth * a.stage_bytes;
-    a.log2c = pick_copies(K, std::min(size_t(128) * 1024, kSmemLimit - stage_total));
+    a.log2c = pick_copies(K, 1 << 20, std::min(size_t(128) * 1024, kSmemLimit - stage_total));
     const size_t smem = (size_t(K) * 8 << a.log2c) + stage_total;
     int grid = sm_count();
     if (flags & QAMW_FLAG_HALF_DEVICE) grid = std::max(1, grid / 2);
@@ -1026,7 +1020,7 @@ int rows_encode(const MatDesc* descs_dev, const MatDesc* descs_host, int n, cons
     const size_t fixed = ((size_t(a.table_bytes) + 15) & ~size_t(15)) + size_t(warps) * Stage2<NS>::kSlots * 8;
     if (!calib && fixed + size_t(K) * 8 > kSmemLimit - kEncode2StaticSmem) return QAMW_ERR_SHAPE;
     const bool tables = !calib && !polar;
-    a.log2c = tables ? pick_copies(K, kSmemLimit - kEncode2StaticSmem - fixed) : 0;
+    a.log2c = tables ? pick_copies(K, 1 << 20, kSmemLimit - kEncode2StaticSmem - fixed) : 0;
     const size_t smem = fixed + (tables ? (size_t(K) * 8 << a.log2c) : 0);
     int grid = sm_count();
     if (flags & QAMW_FLAG_HALF_DEVICE) grid = std::max(1, grid / 2);

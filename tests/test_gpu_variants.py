@@ -192,3 +192,25 @@ def test_step_replayed_as_a_cuda_graph_gives_the_same_bytes():
         assert torch.equal(s.packed, p) and torch.equal(s.row_norm, r)
         assert torch.equal(s.w_hat.view(torch.int16), w.view(torch.int16)) and torch.equal(s.dist, d)
     assert int(mc.status.cpu()[0]) == 0
+
+
+@pytest.mark.parametrize("K", [2, 32, 64, 128, 512, 1024, 2048, 4096])
+@pytest.mark.parametrize("d_out,d_in,n_vec", [(1, 32, 1), (150, 544, 2), (301, 1056, 1), (37, 2080, 4)])
+def test_fused_gemv_rows_off_16_byte_boundaries(orc, K, d_out, d_in, n_vec):
+    """Every index width, with packed rows that start anywhere on 4 bytes and end inside a 16-byte piece."""
+    W, act = _problem(K + n_vec, d_out, d_in)
+    g = torch.Generator().manual_seed(d_in)
+    cbh = orc.train_codebook(K, 1 << 13, 7, 2, 1e-6)[0]
+    cb = q.Codebook(cbh)
+    p = q.make_params(None, d_out, d_in, 32, K)
+    packed = torch.randint(0, 256, (d_out, p.packed_row_stride), generator=g, dtype=torch.uint8)
+    norm, sigma = torch.rand(d_out, generator=g) + 0.5, torch.rand(d_in // 2, generator=g) + 0.5
+    s = torch.from_numpy(q.channel_scales(act, 0.3))
+    signs = torch.from_numpy(q.make_signs(q.DEFAULT_SIGN_SEED, d_in))
+    x = torch.randn((n_vec, d_in), generator=g)
+    y = torch.full((d_out, n_vec), float("nan"), dtype=torch.float32, device=DEV)
+    q.decode_gemv(packed.to(DEV), norm.to(DEV), s.to(DEV), signs.to(DEV), sigma.to(DEV), cb, p, x.to(DEV), y)
+    _, w64 = orc.decode(packed.numpy(), norm.numpy(), 32, cbh, s.numpy(), signs.numpy(), sigma.numpy(), d_in, want_f64=True)
+    ref = w64 @ x.numpy().astype(np.float64).T
+    bound = 1e-5 * np.sqrt((w64 ** 2).sum(1))[:, None] * np.sqrt((x.numpy().astype(np.float64) ** 2).sum(1))[None, :]
+    assert np.all(np.abs(y.cpu().numpy() - ref) <= bound + 1e-30)
