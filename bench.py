@@ -293,7 +293,7 @@ def run_ours(args):
         return
 
     peak, peak_kind = measured_peaks()
-    enc_launches = len({mc._encoder_class(s.d_in) for s in mc.slots}) if mc.use_batch else len(mc.slots)
+    enc_launches = len({mc._encoder_class(s.d_in, mc.spec.block) for s in mc.slots}) if mc.use_batch else len(mc.slots)
     dec_launches = 1 if mc.use_batch else len(mc.slots)
     fp32_peak = q.measure_fp32_peak()
     pipe = load_pipe_note()

@@ -71,9 +71,12 @@ bool build_cell_lists(const double* cb, int K, int grid, CellLists* out);  // de
 double overflow_cost(const CellLists& cl);
 bool pack_search_table(const CellLists& cl, SearchTable* out);
 
-// grid > 0 (odd): exactly that grid (fails if it does not fit); grid == 0: the default grid for K,
-// shrunk until the table fits in budget_bytes.
-bool choose_search_table(const float* codebook, int K, int grid, size_t budget_bytes, SearchTable* out);
+// grid > 0 (odd): exactly that grid (fails if it does not fit); grid == 0: `first` columns (0: the default for
+// K), shrunk until the table fits in budget_bytes.
+bool choose_search_table(const float* codebook, int K, int grid, size_t budget_bytes, SearchTable* out, int first = 0);
+// The records as the kernels read them (SearchSmem in qamw_device.cuh), for codebook entries of 2^log2_entry bytes:
+// grid * grid * 2 words, then the overflow lists.  False if the lists do not fit their fields.
+bool pack_device_table(const SearchTable& t, int K, int log2_entry, std::vector<uint32_t>* words, std::vector<uint16_t>* lists);
 
 void set_cuda_error(const char* what, int code);
 void set_error_text(const char* text);
@@ -93,7 +96,7 @@ struct MatDesc {
     long long packed_row_stride;  // bytes
     long long calib_offset;       // batched calibration: byte offset of this matrix's partial sums in the workspace,
     int calib_first_block;        //   the first block whose span touches it, and the number of slots it has
-    int calib_slots;              //   ((blocks touching it) x (row groups per block)), each [pair_stride] doubles
+    int calib_slots;              //   (blocks touching it), each [pair_stride] doubles
     int d_out, d_in;
 };
 
@@ -105,6 +108,9 @@ int rows_decode(const MatDesc* descs_dev, const MatDesc* descs_host, int n, cons
 int rows_encode(const MatDesc* descs_dev, const MatDesc* descs_host, int n, const void* spans_dev, int span_blocks,
                 int block, int K, int w_bf16, const ::qamw_codebook* cb, uint32_t flags, int32_t* status, void* stream,
                 void* calib_base = nullptr);  // calib_base: run the calibration pass instead (cb may be NULL)
+// The calibration pass and its finish for one matrix; QAMW_ERR_SHAPE as above.
+int rows_calibrate(MatDesc d, int block, int w_bf16, uint32_t flags, void* workspace, size_t workspace_bytes, int32_t* status,
+                   void* stream);
 int sm_count();
 // log2 of the number of bank-separated codebook copies a block keeps in shared memory (at most 16, and at most
 // `budget` bytes) when it makes `gathers` warp-wide codeword reads in all.  A copy costs its stores (one wavefront per 128
@@ -139,6 +145,7 @@ struct qamw_codebook {
     void* d_blob = nullptr;
     size_t blob_bytes = 0;
     size_t off_cells = 0, off_overflow = 0;
+    int log2c = 0;  // log2 of the codebook copies that the cell records assume
     qamw::CellMap map;
     int n_candidates = 0, max_list = 0, n_overflow_cells = 0;
     std::vector<float> h_codebook;  // host copy (decode only needs the device codebook)

@@ -86,7 +86,7 @@ namespace {
 
 constexpr int kMaxThreads = 512;   // threads per block (register budget: 128 per thread)
 constexpr int kMaxGroups = 15;     // named barriers 1..15
-constexpr size_t kEncodeStaticSmem = 512;  // the encoder's statically allocated partial sums
+constexpr size_t kEncodeStaticSmem = 1024;  // the encoder's statically allocated partial sums, rounded up
 
 struct RowGeom {
     int d_out, d_in;
@@ -406,6 +406,7 @@ struct EncodeArgs {
     int K, log2K, grid;
     float map_zmax, map_c0, map_c1, map_c2, map_bias;  // the cell map of the table
     int log2c;               // log2 of the number of codebook copies in shared memory
+    int table_entry;         // log2 of the entry size that the cell records assume
     int brute;
     float inv_sqrt_b;        // c_b = f32(1 / sqrt(b))
     uint8_t* packed;
@@ -486,12 +487,10 @@ __global__ void __launch_bounds__(kMaxThreads, 1) encode_kernel(const EncodeArgs
     const int any_risky = __syncthreads_or(risky ? 1 : 0);  // also the prologue's barrier
 
     SearchSmem s;
-    s.cb = smem_addr(smem) + 8u * (threadIdx.x & ((1 << a.log2c) - 1));
-    s.cb_stride = 8u << a.log2c;
+    search_fields(s, smem, a.K, a.log2K, a.log2c, a.table_entry);
     s.cells = smem_addr(table) - 8u * kMagicBits * uint32_t(a.grid + 1);
     s.overflow = smem_addr(table + a.off_overflow);
     s.grid = uint32_t(a.grid);
-    s.K = a.K;
     s.zlo = pack2(-a.map_zmax, -a.map_zmax);
     s.c0 = pack2(a.map_c0, a.map_c0);
     s.c1 = pack2(a.map_c1, a.map_c1);
@@ -578,25 +577,26 @@ __global__ void __launch_bounds__(kMaxThreads, 1) encode_kernel(const EncodeArgs
                 const int k0 = 4 * Layout<LOG2B_T>::octet_after(tid_g, rr);
                 uint32_t v[4];
                 if (MODE == 0) {
-                    uint2 rec[4];
+                    uint32_t word1[4];
                     float2 z[4];
 #pragma unroll
                     for (int p = 0; p < 4; ++p) {
                         unpack2(P[rr][p], z[p].x, z[p].y);
-                        v[p] = uint32_t(search_cell(s, z[p].x, z[p].y, rec[p]));
+                        v[p] = search_cell<true>(s, z[p].x, z[p].y, word1[p]);
                     }
-                    // rare: one of the four cells has more than four candidates
-                    if (cell_overflows(rec[0]) || cell_overflows(rec[1]) || cell_overflows(rec[2]) || cell_overflows(rec[3])) {
+                    if (cell_overflows(word1[0] | word1[1] | word1[2] | word1[3])) {
 #pragma unroll
                         for (int p = 0; p < 4; ++p)
-                            if (cell_overflows(rec[p])) v[p] = uint32_t(search_overflow(s, rec[p], z[p].x, z[p].y));
+                            if (cell_overflows(word1[p])) v[p] = search_overflow(s, word1[p], v[p], z[p].x, z[p].y);
                     }
+#pragma unroll
+                    for (int p = 0; p < 4; ++p) v[p] >>= s.log2_entry;
                 } else {
 #pragma unroll
                     for (int p = 0; p < 4; ++p) {
                         float2 z;
                         unpack2(P[rr][p], z.x, z.y);
-                        v[p] = uint32_t(MODE == 2 ? search_exhaustive(s, z.x, z.y) : search_table(s, z.x, z.y));
+                        v[p] = (MODE == 2 ? search_exhaustive(s, z.x, z.y) : search_table<true>(s, z.x, z.y)) >> s.log2_entry;
                     }
                 }
                 // two indices fit a 32-bit word (B <= 12)
@@ -1399,12 +1399,17 @@ extern "C" int qamw_codebook_create(const float* codebook_host, int K, int grid,
     if (grid < 0 || grid > 255 || (grid > 0 && grid % 2 == 0)) return QAMW_ERR_ARG;
     *out = nullptr;
     SearchTable t;
-    // The encoder's shared memory also holds 20 KB of per-warp index staging (16 warps x 1.25 KB)
-    // and the codebook in eight bank-separated copies (two for K = 4096): the table gets what is left
-    // of the 227 KB of one SM.  The grid side is odd.
-    const size_t copies = K <= 2048 ? 8 : 2;
-    const size_t budget = kSmemLimit - kEncodeStaticSmem - size_t(16) * (kStageSlotsPerWarp * 8) - size_t(K) * 8 * copies;
-    if (!choose_search_table(codebook_host, K, grid, budget, &t)) return QAMW_ERR_NOMEM;
+    // A block of the encoder holds the table and as many bank-separated copies of the codebook as fit beside it:
+    // sixteen up to K = 1024, eight at 2048, two at 4096.  The table gets what is left of the 227 KB of an SM, up to
+    // 3.1 sqrt(K) columns: at K = 1024 that leaves 0.1 % of the points in cells with more than four candidates (0.9 %
+    // with 2.2 sqrt(K)) and 6 % in cells with four (13 %); more columns would take longer to copy than they save.
+    const int log2c = K <= 1024 ? 4 : K <= 2048 ? 3 : 1;
+    const size_t budget = kSmemLimit - kEncodeStaticSmem - (size_t(K) * 8 << log2c);
+    const int first = 2 * std::max(15, std::min(int(1.55 * std::sqrt(double(K))), 127)) + 1;
+    if (!choose_search_table(codebook_host, K, grid, budget, &t, first)) return QAMW_ERR_NOMEM;
+    std::vector<uint32_t> words;
+    std::vector<uint16_t> lists;
+    if (!pack_device_table(t, K, 3 + log2c, &words, &lists)) return QAMW_ERR_NOMEM;
     qamw_codebook* cb = new (std::nothrow) qamw_codebook();
     if (!cb) return QAMW_ERR_NOMEM;
     cb->K = K;
@@ -1414,12 +1419,13 @@ extern "C" int qamw_codebook_create(const float* codebook_host, int K, int grid,
     cb->n_overflow_cells = t.n_overflow_cells;
     cb->h_codebook.assign(codebook_host, codebook_host + 2 * K);
     cb->off_cells = size_t(K) * 8;
-    cb->off_overflow = cb->off_cells + t.cells.size() * 2;
-    cb->blob_bytes = cb->off_overflow + t.overflow.size() * 2;
+    cb->off_overflow = cb->off_cells + words.size() * 4;
+    cb->blob_bytes = cb->off_overflow + lists.size() * 2;
+    cb->log2c = log2c;
     std::vector<unsigned char> blob(cb->blob_bytes, 0);
     std::memcpy(blob.data(), codebook_host, size_t(K) * 8);
-    std::memcpy(blob.data() + cb->off_cells, t.cells.data(), t.cells.size() * 2);
-    if (!t.overflow.empty()) std::memcpy(blob.data() + cb->off_overflow, t.overflow.data(), t.overflow.size() * 2);
+    std::memcpy(blob.data() + cb->off_cells, words.data(), words.size() * 4);
+    std::memcpy(blob.data() + cb->off_overflow, lists.data(), lists.size() * 2);
     cudaError_t e = cudaGetDevice(&cb->device);
     if (e == cudaSuccess) e = cudaMalloc(&cb->d_blob, cb->blob_bytes);
     if (e == cudaSuccess) e = cudaMemcpy(cb->d_blob, blob.data(), cb->blob_bytes, cudaMemcpyHostToDevice);
@@ -1558,7 +1564,8 @@ extern "C" int qamw_encode(const void* W, const qamw_params* p, const float* cha
     const size_t fixed = ((size_t(a.table_bytes) + 15) & ~size_t(15)) +
                          size_t(a.g.groups) * (a.g.tg / 32) * (kStageSlotsPerWarp * 8);
     if (fixed + size_t(p->K) * 8 > kSmemLimit - kEncodeStaticSmem) return QAMW_ERR_NOMEM;
-    a.log2c = pick_log2_copies(p->K, kSmemLimit - kEncodeStaticSmem - fixed);
+    a.log2c = std::min(cb->log2c, pick_log2_copies(p->K, kSmemLimit - kEncodeStaticSmem - fixed));
+    a.table_entry = 3 + cb->log2c;
     const size_t smem = fixed + (size_t(p->K) * 8 << a.log2c);
     const int blocks = std::max(1, std::min(grid_limit(p), (p->d_out + a.g.groups - 1) / a.g.groups));
     cudaStream_t st = static_cast<cudaStream_t>(stream);
@@ -1628,6 +1635,18 @@ extern "C" int qamw_calibrate(const void* W, const qamw_params* p, const float* 
     a.g.cvec = const_vec_ok(p, chan_scale, signs, nullptr);
     const CalibPlan c = calib_plan(p, a.g);
     if (workspace_bytes < c.bytes) return QAMW_ERR_NOMEM;
+    if (!(p->flags & QAMW_FLAG_GENERAL_KERNELS)) {  // common layouts: the encoder's kernel
+        MatDesc d{};
+        d.W = W;
+        d.chan_scale = chan_scale;
+        d.signs = signs;
+        d.sigma = sigma_out;
+        d.w_row_stride = p->w_row_stride;
+        d.d_out = p->d_out;
+        d.d_in = p->d_in;
+        rc = rows_calibrate(d, p->block, a.g.w_bf16, p->flags, workspace, workspace_bytes, status_out, stream);
+        if (rc != QAMW_ERR_SHAPE) return rc;
+    }
     a.W = W;
     a.chan_scale = chan_scale;
     a.signs = signs;

@@ -32,6 +32,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
+#include <cstring>
 #include <mutex>
 #include <new>
 #include <type_traits>
@@ -49,12 +50,13 @@ namespace {
 // ---------------------------------------------------------------------------------------------
 // layout of a Hadamard block over NS slots and L = 2^S lanes
 // ---------------------------------------------------------------------------------------------
+// LOG2B = 0: blocks of 2 to 16 elements, whose size is a run-time value; they never leave the thread.
 template <int NS, int LOG2B>
 struct Lay2 {
     static_assert(NS == 2 || NS == 4, "two or four octets per thread");
     static constexpr int LS = NS == 4 ? 2 : 1;          // slot bits
     static constexpr int TOP = NS / 2;                  // value of the top slot bit
-    static constexpr int S = LOG2B - 3 - LS;            // cross-lane stages
+    static constexpr int S = LOG2B ? LOG2B - 3 - LS : 0;  // cross-lane stages
     static_assert(S >= 0 && S <= 5, "block size out of range for this geometry");
     static constexpr int L = 1 << S;
     // octet (units of 8 elements, relative to the warp's segment) in physical slot p before the
@@ -90,7 +92,7 @@ struct Lay2 {
 // the L lanes of the block.  P[p][i] holds elements (2i, 2i+1) of the octet in physical slot p.
 // FIRST_STAGE_DONE: the caller's inputs already went through stage h = 1.
 template <int NS, int LOG2B, bool FIRST_STAGE_DONE>
-__device__ __forceinline__ void fwht2(f32x2 (&P)[NS][4], int lane) {
+__device__ __forceinline__ void fwht2(f32x2 (&P)[NS][4], int lane, int log2b_small) {
     typedef Lay2<NS, LOG2B> Lay;
     constexpr int TOP = Lay::TOP;
     if (!FIRST_STAGE_DONE) {
@@ -103,6 +105,25 @@ __device__ __forceinline__ void fwht2(f32x2 (&P)[NS][4], int lane) {
                 P[p][i] = pack2(__fadd_rn(a, c), __fsub_rn(a, c));
             }
     }
+    if constexpr (LOG2B == 0) {
+#pragma unroll
+        for (int p = 0; p < NS; ++p) {
+            if (log2b_small >= 2) {
+                bfly2(P[p][0], P[p][1]);
+                bfly2(P[p][2], P[p][3]);
+            }
+            if (log2b_small >= 3) {
+                bfly2(P[p][0], P[p][2]);
+                bfly2(P[p][1], P[p][3]);
+            }
+        }
+        if (log2b_small >= 4) {
+#pragma unroll
+            for (int p = 0; p < NS; p += 2)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) bfly2(P[p][i], P[p + 1][i]);
+        }
+    } else {
 #pragma unroll
     for (int p = 0; p < NS; ++p) {  // h = 2, 4
         bfly2(P[p][0], P[p][1]);
@@ -164,6 +185,7 @@ __device__ __forceinline__ void fwht2(f32x2 (&P)[NS][4], int lane) {
                 }
         }
     }
+    }  // LOG2B != 0
 }
 
 __device__ __forceinline__ void st_global_256(void* p, const uint32_t (&w)[8]) {
@@ -360,7 +382,7 @@ __global__ void __launch_bounds__(NS == 4 ? 512 : 896, 1) decode2_kernel(const D
                     }
                 }
             }
-            fwht2<NS, LOG2B, true>(P, lane);
+            fwht2<NS, LOG2B, true>(P, lane, LOG2B);
             const f32x2 rn2 = pack2(rn, rn);
 #pragma unroll
             for (int p = 0; p < NS; p += (NS == 4 ? 2 : 1)) {
@@ -400,9 +422,12 @@ struct Encode2Args {
     int table_bytes;         // a multiple of 16
     int off_overflow;        // byte offset inside the table
     int K, log2K, grid;
-    float map_zmax, map_c0, map_c1, map_c2, map_bias;  // the cell map of the table
+    f32x2 map_zlo, map_c0, map_c1, map_c2, map_bias;  // the cell map of the table, each value twice
     int log2c;               // log2 of the number of codebook copies in shared memory
-    int brute;
+    int log2b;               // log2 of the Hadamard block
+    int wide;                // rows of W start on 32 bytes and d_in is a multiple of 8 NS
+    int brute;               // every point is compared with the whole codebook
+    float reach;             // |z| from which on a point is: 16000, or -1 with `brute`
     float inv_sqrt_b;        // c_b = f32(1 / sqrt(b))
     int32_t* status;         // out (optional): bit 0 set when a row norm is not finite
     unsigned char* calib_base;  // calibration mode: base of the partial-sum workspace (MatDesc::calib_offset)
@@ -445,24 +470,95 @@ __device__ __forceinline__ int search_polar(const PolarSmem& s, float zx, float 
     return (p << s.Ba) | a;
 }
 
-// Index staging of a warp: its 64 octets as one 64-bit value each (index p of the octet at bits
-// [p B, (p+1) B)); 8 slots of padding after every 16 keep the two stores of a warp on distinct banks
-// for the common block sizes.
-template <int NS>
-struct Stage2 {
-    static constexpr int kSlots = NS == 2 ? 96 : 160;  // 32 NS octets plus their padding
-    __device__ static __forceinline__ int slot(int o) { return NS == 2 ? o + ((o >> 4) << 3) : o + ((o >> 4) << 2); }
-};
+// Sum of v over the warp, in every lane, by two 8x8x4 double matrix products with a matrix of ones: the first
+// adds the four lanes of a quad, the second the eight quads (two of them added by hand in between).  Ten
+// shuffles and five additions, the alternative, load the pipe that binds the encoder.
+__device__ __forceinline__ double warp_total(double v) {
+    auto quads = [](double b, double& d0, double& d1) {
+        asm("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0, %1}, {%2}, {%3}, {%4, %4};"
+            : "=d"(d0), "=d"(d1)
+            : "d"(1.0), "d"(b), "d"(0.0));
+    };
+    double d0, d1, e0, e1;
+    quads(v, d0, d1);          // this lane: totals of quads 2 (lane mod 4) and 2 (lane mod 4) + 1
+    quads(d0 + d1, e0, e1);
+    return e0;
+}
 
-// Encoder, two octets per thread.  A warp owns 512 consecutive elements of a row: it scales them,
-// adds up its part of the row norm, rotates (shuffles only), and after the one meeting point of the
-// row's warps -- a named barrier for the norm -- searches its 256 pairs, stages the indices and
-// writes its 32 B bytes of the packed row.  W is read once.
+// For every unit of a thread the unit that follows it in the row: units u0 and u1 of a lane lie L units apart, at q
+// and q + L of the block (q: lane inside the block).  A lane that is read for its u1 by the last lane of its block is
+// not read for its u0, so one shuffle per 32 bits serves both.
+template <int L>
+__device__ __forceinline__ void next_units(uint32_t u0, uint32_t u1, int lane, uint32_t& n0, uint32_t& n1) {
+    const int q = lane & (L - 1);
+    const bool first = q == 0, last = q == L - 1;
+    n0 = __shfl_sync(kFull, first ? u1 : u0, last ? lane - (L - 1) : lane + 1);
+    n1 = __shfl_sync(kFull, first ? u0 : u1, lane + 1);
+}
+
+// The words of the packed row that start inside an octet of this thread.  u[p]: the 4 B bits of the octet in
+// slot p; first[p]: the first such word (relative to the warp's segment) and, from bit 16 on, its distance from
+// the octet's first bit; limit: words of the row's payload from the segment's first on.  The bits past an octet come
+// from the lanes that hold the next ones.
+template <int NS, int LOG2B>
+__device__ __forceinline__ void store_indices(const uint2 (&u)[NS], const uint32_t (&first)[NS], int B, uint32_t* out, int limit, int lane) {
+    constexpr int L = Lay2<NS, LOG2B>::L, X = NS / 2;  // the octets that change lanes: slots 0 and X hand over to X - 1 and NS - 1
+    const int U = 4 * B;
+    if (U > 32) {
+        uint2 nxt[NS];
+        next_units<L>(u[0].x, u[X].x, lane, nxt[X - 1].x, nxt[NS - 1].x);
+        next_units<L>(u[0].y, u[X].y, lane, nxt[X - 1].y, nxt[NS - 1].y);
+        if (NS == 4) {
+            nxt[0] = u[1 % NS];
+            nxt[2 % NS] = u[3 % NS];
+        }
+#pragma unroll
+        for (int p = 0; p < NS; ++p) {
+            const int w = int(first[p] & 0xffffu), off = int(first[p] >> 16);
+            const uint32_t x1 = u[p].y | (nxt[p].x << (U - 32));
+            const uint32_t x2 = __funnelshift_r(nxt[p].x, nxt[p].y, 64 - U);
+            if (w < limit) out[w] = __funnelshift_r(u[p].x, x1, off);
+            if (off + 32 < U && w + 1 < limit) out[w + 1] = __funnelshift_r(x1, x2, off);
+        }
+    } else {
+        uint32_t cur[NS];
+        unsigned long long acc[NS];
+#pragma unroll
+        for (int p = 0; p < NS; ++p) acc[p] = cur[p] = u[p].x;
+        for (int at = U; at < U + 31; at += U) {  // a word that starts in the octet's last bit ends 31 bits later
+            uint32_t nxt[NS];
+            next_units<L>(cur[0], cur[X], lane, nxt[X - 1], nxt[NS - 1]);
+            if (NS == 4) {
+                nxt[0] = cur[1 % NS];
+                nxt[2 % NS] = cur[3 % NS];
+            }
+#pragma unroll
+            for (int p = 0; p < NS; ++p) {
+                cur[p] = nxt[p];
+                acc[p] |= (unsigned long long)cur[p] << at;
+            }
+        }
+#pragma unroll
+        for (int p = 0; p < NS; ++p) {
+            const int w = int(first[p] & 0xffffu), off = int(first[p] >> 16);
+            if (off < U && w < limit) out[w] = uint32_t(acc[p] >> off);
+        }
+    }
+}
+
+// Encoder.  A warp owns 256 NS consecutive elements of a row (NS = 2; blocks of 1024 elements take NS = 4): it scales
+// them, adds up its part of the row norm, rotates (shuffles only), and after the one meeting point of the
+// row's warps -- a named barrier for the norm -- searches its pairs and writes its 16 NS B bytes of the packed
+// row.  W is read once.
+//
+// Bound by the shared-memory pipe: of 26 wavefronts per 32 points a cell record (8 random bytes) takes 5.6, the candidate
+// codewords 14 (4 per read from eight copies; the fourth candidate only where there is one), rotation shuffles 3.
 // QUANT: 0 = nearest codeword through the cell table, 1 = polar quantiser, 2 = no quantiser at all:
 // the kernel then is the calibration pass of Section 3.4, which visits n = min(d_out, 1024) rows
-// floor(t d_out / n) and adds up the pair moduli |(y_2k, y_2k+1)| per pair position.  Every row group
-// of every block owns one slot of partial sums in the workspace; calibrate_finish2_kernel adds the
-// slots in ascending order, so the result does not depend on timing.
+// floor(t d_out / n) and adds up the pair moduli |(y_2k, y_2k+1)| per pair position.  The row groups of a
+// block add their sums up in shared memory, in ascending order, and every block leaves one slot of partial sums per
+// matrix in the workspace; calibrate_finish2_kernel adds the slots in ascending order, so the result does not
+// depend on timing.
 template <bool BF16, int LOG2B, int NS, int MAXT, int QUANT>
 __global__ void __launch_bounds__(MAXT, 1) encode2_kernel(const Encode2Args a) {
     constexpr bool POLAR = QUANT == 1, CALIB = QUANT == 2;
@@ -471,6 +567,8 @@ __global__ void __launch_bounds__(MAXT, 1) encode2_kernel(const Encode2Args a) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ double ss_part[2][32];  // per-warp partial sums of squares, two rows in flight
     __shared__ MatDesc cur;            // the matrix the block is working on (re-read per row: saves registers)
+    __shared__ int used_rows[16];      // calibration: rows that each group has added up
+    __shared__ int row_words[2];       // words of a packed row of the matrix: with payload, and up to its stride
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
 
     chain_release();
@@ -494,39 +592,44 @@ __global__ void __launch_bounds__(MAXT, 1) encode2_kernel(const Encode2Args a) {
             }
         }
     }
-    const int table_pad = (a.table_bytes + 15) & ~15;
-    unsigned long long* oct_s = reinterpret_cast<unsigned long long*>(table + table_pad) + size_t(warp) * Stage2<NS>::kSlots;
 
     SearchSmem s;
-    s.cb = smem_addr(smem) + 8u * (threadIdx.x & ((1 << a.log2c) - 1));
-    s.cb_stride = 8u << a.log2c;
+    search_fields(s, smem, a.K, a.log2K, a.log2c, 3 + a.log2c);
     s.cells = smem_addr(table) - 8u * kMagicBits * uint32_t(a.grid + 1);
     s.overflow = smem_addr(table + a.off_overflow);
     s.grid = uint32_t(a.grid);
-    s.K = a.K;
-    s.zlo = pack2(-a.map_zmax, -a.map_zmax);
-    s.c0 = pack2(a.map_c0, a.map_c0);
-    s.c1 = pack2(a.map_c1, a.map_c1);
-    s.c2 = pack2(a.map_c2, a.map_c2);
-    s.bias = pack2(a.map_bias, a.map_bias);
+    s.zlo = a.map_zlo;
+    s.c0 = a.map_c0;
+    s.c1 = a.map_c1;
+    s.c2 = a.map_c2;
+    s.bias = a.map_bias;
     PolarSmem ps;
     ps.thr2 = smem_addr(table);
     ps.bnd = smem_addr(table + a.off_overflow);
     ps.Ba = a.polar_ba;
     ps.Bp = a.polar_bp;
 
-    const int B = a.log2K, B4 = 4 * a.log2K;
-    const unsigned div_magic = 0xffffffffu / unsigned(B4) + 1u;  // ceil(2^32 / (4B))
+    const int B = a.log2K;
     constexpr int kEsz = BF16 ? 2 : 4;
+    uint32_t first[NS];  // see store_indices
+#pragma unroll
+    for (int p = 0; p < NS; ++p) {
+        const uint32_t bit0 = uint32_t(4 * B * Lay::octet_after(lane, p)), w = (bit0 + 31) >> 5;
+        first[p] = w | ((32 * w - bit0) << 16);
+    }
 
     chain_wait();
-    const int4 span = block_span(a.spans, a.one.d_out);
+    const int4 span = block_span(a.spans, CALIB ? min(a.one.d_out, QAMW_CALIB_MAX_ROWS) : a.one.d_out);
     for (int m = span.x; m <= span.z; ++m) {
         // The warps regroup when the row length changes: nobody may still be inside the previous
         // matrix (its named barriers and partial sums) when the first warp enters the next one.  The
         // first pass also waits for the tables.
         __syncthreads();
-        if (threadIdx.x == 0) cur = a.descs ? a.descs[m] : a.one;
+        if (threadIdx.x == 0) {
+            cur = a.descs ? a.descs[m] : a.one;
+            row_words[0] = int((((long long)(cur.d_in >> 1) * B + 7) / 8 + 3) / 4);
+            row_words[1] = int(cur.packed_row_stride >> 2);
+        }
         __syncthreads();
         const MatDesc& d = cur;
         const int d_in = d.d_in, n_pairs = d_in >> 1;
@@ -536,8 +639,8 @@ __global__ void __launch_bounds__(MAXT, 1) encode2_kernel(const Encode2Args a) {
         const int n_seg = (d_in + WE - 1) / WE;
         const int groups = min(15, n_warps / n_seg);  // named barriers 1..15
         const int group = warp / n_seg, seg = warp - group * n_seg;
-        const int row0 = row_begin + group;
-        if (group >= groups || row0 >= row_end) continue;
+        const int row0 = group < groups ? row_begin + group : row_end;
+        if (!CALIB && row0 >= row_end) continue;
         const int row_step = groups;
         const int tg = n_seg * 32;
         const int oct0 = seg * (WE / 8);
@@ -546,7 +649,7 @@ __global__ void __launch_bounds__(MAXT, 1) encode2_kernel(const Encode2Args a) {
         // (with the butterfly's sign pattern folded in) of the pairs it holds after the rotation
         f32x2 t[NS][4];
         float q[NS][4];
-        bool live[NS];
+        uint32_t live = 0;  // bit p: the octet that ends up in slot p lies inside the row
         bool risky = false;
 #pragma unroll
         for (int p = 0; p < NS; ++p) {
@@ -562,123 +665,131 @@ __global__ void __launch_bounds__(MAXT, 1) encode2_kernel(const Encode2Args a) {
 #pragma unroll
             for (int i = 0; i < 4; ++i) t[p][i] = pack2(cs[2 * i] * sgn[2 * i], cs[2 * i + 1] * sgn[2 * i + 1]);
             const int k0 = 4 * (oct0 + Lay::octet_after(lane, p));
-            live[p] = k0 < n_pairs;
+            const bool in = k0 < n_pairs;
+            live |= in ? 1u << p : 0u;
             if (!CALIB) {
                 load4f(d.sigma, k0, n_pairs, 1, 1.0f, q[p]);
-            } else {
+                const float fl = Lay::negated(lane, p) ? -1.0f : 1.0f;
 #pragma unroll
-                for (int i = 0; i < 4; ++i) q[p][i] = 1.0f;
-            }
-            const float fl = Lay::negated(lane, p) ? -1.0f : 1.0f;
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                // q_k = f32(1 / (double)sigma_k): the correctly rounded f32 reciprocal is the same number
-                const float r = live[p] ? __frcp_rn(q[p][i]) : 0.f;
-                // |z| <= q (1 + eps) because |y| <= 1 for a unit row: only a huge reciprocal pair scale can
-                // carry a point beyond the table's reach
-                risky |= !(r < 15000.0f);
-                q[p][i] = fl * r;
+                for (int i = 0; i < 4; ++i) {
+                    // q_k = f32(1 / (double)sigma_k): the correctly rounded f32 reciprocal is the same number
+                    const float r = in ? __frcp_rn(q[p][i]) : 0.f;
+                    // |z| <= q (1 + eps) because |y| <= 1 for a unit row: only a huge reciprocal pair scale can
+                    // carry a point beyond the table's reach
+                    risky |= !(r < 15000.0f);
+                    q[p][i] = fl * r;
+                }
             }
         }
-        const bool any_risky = __any_sync(kFull, risky);
+        const uint32_t careful = a.brute || __any_sync(kFull, risky) ? 1u : 0u;
 
         const int col0 = seg * WE + 8 * NS * lane;  // first column of this thread
-        const bool have_w = col0 < d_in;            // the fast path needs d_in to be a multiple of 8 NS: all or none
         const int seg_word0 = 4 * NS * B * seg;     // first packed word of this warp's segment (16 NS B bytes per segment)
         const bool last_seg = seg == n_seg - 1;
         double* part_base = &ss_part[0][group * n_seg];
 
-        auto rows = [&](auto mode_tag) {
-            constexpr int MODE = decltype(mode_tag)::value;  // 0 = table, 1 = table with reach check, 2 = exhaustive, 3 = polar, 4 = calibrate
-            int parity = 0;
-            double acc[NS][4];
-            int used = 0;
+        int parity = 0;
+        double acc[NS][4];
+        int used = 0;
 #pragma unroll
-            for (int p = 0; p < NS; ++p)
+        for (int p = 0; p < NS; ++p)
 #pragma unroll
-                for (int i = 0; i < 4; ++i) acc[p][i] = 0.0;
-            // raw bits of the thread's elements of one row; the next row is fetched as soon as this one
-            // has been converted, so its latency hides behind the rotation and the search
-            constexpr int kRaw = BF16 ? 4 * NS : 8 * NS;
-            uint32_t raw[kRaw];
-            auto fetch = [&](int t) {
-                const long long row = CALIB ? (long long)t * cur.d_out / n_cal : t;
-                const char* wp = static_cast<const char*>(cur.W) + (row * cur.w_row_stride + col0) * kEsz;
+            for (int i = 0; i < 4; ++i) acc[p][i] = 0.0;
+        // Raw bits of the thread's elements of one row.  The next row is fetched between the searches of the thread's
+        // octets: early enough for its latency to hide, and late enough that its registers are those of the points
+        // searched already (with both alive, 72 and 80 registers a thread spilled into the row loop: 58
+        // against 46 cycles per 32 points).  Columns beyond the row stay zero.
+        constexpr int kRaw = BF16 ? 4 * NS : 8 * NS;
+        uint32_t raw[kRaw];
+        auto fetch = [&](int t) {
+            const long long row = CALIB ? (long long)t * cur.d_out / n_cal : t;
+            const char* wp = static_cast<const char*>(cur.W) + (row * cur.w_row_stride + col0) * kEsz;
+            if (a.wide) {
+                if (col0 < d_in) {
 #pragma unroll
-                for (int h = 0; h < kRaw / 8; ++h) {
-                    uint32_t w[8];
-                    ld_global_256(wp + 32 * h, w);
+                    for (int h = 0; h < kRaw / 8; ++h) {
+                        uint32_t w[8];
+                        ld_global_256(wp + 32 * h, w);
 #pragma unroll
-                    for (int i = 0; i < 8; ++i) raw[8 * h + i] = w[i];
+                        for (int i = 0; i < 8; ++i) raw[8 * h + i] = w[i];
+                    }
                 }
-            };
+            } else {
 #pragma unroll
-            for (int i = 0; i < kRaw; ++i) raw[i] = 0u;
-            if (have_w) fetch(row0);
-            for (int row = row0; row < row_end; row += row_step, parity ^= 1) {
-                f32x2 P[NS][4];
-                if (BF16) {
+                for (int h = 0; h < kRaw / 4; ++h)  // 16 bytes: an octet of bf16, half of one of f32
+                    if (col0 + 16 * h / kEsz < d_in) {
+                        const uint4 w = __ldg(reinterpret_cast<const uint4*>(wp + 16 * h));
+                        raw[4 * h] = w.x;
+                        raw[4 * h + 1] = w.y;
+                        raw[4 * h + 2] = w.z;
+                        raw[4 * h + 3] = w.w;
+                    }
+            }
+        };
 #pragma unroll
-                    for (int i = 0; i < 4 * NS; ++i)
-                        P[i >> 2][i & 3] = mul2(pack2(__uint_as_float(raw[i] << 16), __uint_as_float(raw[i] & 0xffff0000u)),
-                                                t[i >> 2][i & 3]);
-                } else {
+        for (int i = 0; i < kRaw; ++i) raw[i] = 0u;
+        if (row0 < row_end) fetch(row0);
+        for (int row = row0; row < row_end; row += row_step, parity ^= 1) {
+            f32x2 P[NS][4];
+            if (BF16) {
 #pragma unroll
-                    for (int i = 0; i < 4 * NS; ++i)
-                        P[i >> 2][i & 3] = mul2(pack2(__uint_as_float(raw[2 * i]), __uint_as_float(raw[2 * i + 1])), t[i >> 2][i & 3]);
-                }
-                if (have_w && row + row_step < row_end) fetch(row + row_step);
-                // sum of squares of the row: ss = sum_j (double)x_j^2, per thread, per warp, then per row
-                double* part = part_base + parity * 32;
-                {
-                    double ss = 0.0;
+                for (int i = 0; i < 4 * NS; ++i)
+                    P[i >> 2][i & 3] = mul2(pack2(__uint_as_float(raw[i] << 16), __uint_as_float(raw[i] & 0xffff0000u)),
+                                            t[i >> 2][i & 3]);
+            } else {
+#pragma unroll
+                for (int i = 0; i < 4 * NS; ++i)
+                    P[i >> 2][i & 3] = mul2(pack2(__uint_as_float(raw[2 * i]), __uint_as_float(raw[2 * i + 1])), t[i >> 2][i & 3]);
+            }
+            if (CALIB && row + row_step < row_end) fetch(row + row_step);
+            // sum of squares of the row: ss = sum_j (double)x_j^2, per thread, per warp, then per row
+            double* part = part_base + parity * 32;
+            {
+                double s0 = 0.0, s1 = 0.0;
+#pragma unroll
+                for (int p = 0; p < NS; ++p)
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        float x0, x1;
+                        unpack2(P[p][i], x0, x1);
+                        const double d0 = double(x0), d1 = double(x1);
+                        s0 = fma(d0, d0, s0);
+                        s1 = fma(d1, d1, s1);
+                    }
+                s0 = warp_total(s0 + s1);
+                if (lane == 0) part[seg] = s0;
+            }
+            // The rotation does not need the norm, so the warps of the row meet only after it.  A
+            // warp can be one row ahead of another at most, hence the two sets of partial sums.
+            fwht2<NS, LOG2B, false>(P, lane, a.log2b);
+            group_barrier(group, tg);
+            // every warp adds the same numbers in the same order
+            const float r = float(sqrt(warp_total(lane < n_seg ? part[lane] : 0.0)));
+            // g = f32(c_b / r); 0 for a zero row (all its pairs become the origin) and for a non-finite
+            // row (its indices are unspecified; the searches accept any input)
+            const float gn = isfinite(r) && r > 0.f ? __fdiv_rn(a.inv_sqrt_b, r) : 0.f;
+            if (lane == 0 && seg == 0) {
+                if (!CALIB) cur.row_norm[row] = r;
+                if (!isfinite(r) && a.status) atomicOr(a.status, 1);
+            }
+            const f32x2 gn2 = pack2(gn, gn);
+            if constexpr (CALIB) {  // calibration: rows of zero (or non-finite) norm are skipped
+                if (gn != 0.f) {
+                    ++used;
 #pragma unroll
                     for (int p = 0; p < NS; ++p)
 #pragma unroll
                         for (int i = 0; i < 4; ++i) {
-                            float x0, x1;
-                            unpack2(P[p][i], x0, x1);
-                            const double d0 = double(x0), d1 = double(x1);
-                            ss = fma(d0, d0, ss);
-                            ss = fma(d1, d1, ss);
+                            float y0, y1;
+                            unpack2(mul2(P[p][i], gn2), y0, y1);
+                            acc[p][i] += double(sqrtf(__fmaf_rn(y1, y1, __fmul_rn(y0, y0))));
                         }
-                    ss = warp_sum(ss);
-                    if (lane == 0) part[seg] = ss;
                 }
-                // The rotation does not need the norm, so the warps of the row meet only after it.  A
-                // warp can be one row ahead of another at most, hence the two sets of partial sums.
-                fwht2<NS, LOG2B, false>(P, lane);
-                group_barrier(group, tg);
-                float gn = 0.f;
-                if (lane == 0) {  // every warp adds the same numbers in the same order
-                    double total = 0.0;
-                    for (int w = 0; w < n_seg; ++w) total += part[w];
-                    const float r = float(sqrt(total));
-                    // g = f32(c_b / r); 0 for a zero row (all its pairs become the origin) and for a non-finite
-                    // row (its indices are unspecified; the searches accept any input)
-                    if (isfinite(r) && r > 0.f) gn = __fdiv_rn(a.inv_sqrt_b, r);
-                    if (seg == 0) {
-                        if (!CALIB) cur.row_norm[row] = r;
-                        if (!isfinite(r) && a.status) atomicOr(a.status, 1);
-                    }
-                }
-                gn = __shfl_sync(kFull, gn, 0);
-                const f32x2 gn2 = pack2(gn, gn);
-                if constexpr (MODE == 4) {  // calibration: rows of zero (or non-finite) norm are skipped
-                    if (gn != 0.f) {
-                        ++used;
-#pragma unroll
-                        for (int p = 0; p < NS; ++p)
-#pragma unroll
-                            for (int i = 0; i < 4; ++i) {
-                                float y0, y1;
-                                unpack2(mul2(P[p][i], gn2), y0, y1);
-                                acc[p][i] += double(sqrtf(__fmaf_rn(y1, y1, __fmul_rn(y0, y0))));
-                            }
-                    }
-                } else {
+            } else {
+                uint2 octet[NS];  // 4 B bits
 #pragma unroll
                 for (int p = 0; p < NS; ++p) {
+                    if (p == NS / 2 && row + row_step < row_end) fetch(row + row_step);
                     uint32_t v[4];
                     float2 z[4];
 #pragma unroll
@@ -687,102 +798,79 @@ __global__ void __launch_bounds__(MAXT, 1) encode2_kernel(const Encode2Args a) {
                         unpack2(mul2(P[p][i], gn2), yx, yy);
                         z[i] = make_float2(__fmul_rn(yx, q[p][i]), __fmul_rn(yy, q[p][i]));
                     }
-                    if (MODE == 3) {
+                    if (POLAR) {
 #pragma unroll
                         for (int i = 0; i < 4; ++i) v[i] = uint32_t(search_polar(ps, z[i].x, z[i].y));
-                    } else if (MODE == 0) {
-                        uint2 rec[4];
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) v[i] = uint32_t(search_cell(s, z[i].x, z[i].y, rec[i]));
-                        // rare: one of the four cells has more than four candidates
-                        if (int(cell_overflows(rec[0])) | int(cell_overflows(rec[1])) | int(cell_overflows(rec[2])) | int(cell_overflows(rec[3]))) {
-#pragma unroll
-                            for (int i = 0; i < 4; ++i)
-                                if (cell_overflows(rec[i])) v[i] = uint32_t(search_overflow(s, rec[i], z[i].x, z[i].y));
-                        }
                     } else {
+                        uint32_t word1[4];
 #pragma unroll
-                        for (int i = 0; i < 4; ++i)
-                            v[i] = uint32_t(MODE == 2 ? search_exhaustive(s, z[i].x, z[i].y) : search_table(s, z[i].x, z[i].y));
-                    }
-                    // two indices fit a 32-bit word (B <= 12); octets beyond the row are staged as zero
-                    unsigned long long packed4 =
-                        (unsigned long long)(v[0] | (v[1] << B)) | ((unsigned long long)(v[2] | (v[3] << B)) << (2 * B));
-                    if (!live[p]) packed4 = 0ull;
-                    oct_s[Stage2<NS>::slot(Lay::octet_after(lane, p))] = packed4;
-                }
-                __syncwarp();
-                // bit packing of the warp's segment: octet o occupies bits [o*4B, (o+1)*4B) (LSB first)
-                const long long pstride = cur.packed_row_stride;
-                uint32_t* out = reinterpret_cast<uint32_t*>(cur.packed + (long long)row * pstride);
-                const int row_words = int(pstride >> 2);
-                const int payload_words = int((((long long)(cur.d_in >> 1) * B + 7) / 8 + 3) / 4);
-                for (int j = lane; j < 4 * NS * B; j += 32) {
-                    const int gw = seg_word0 + j;
-                    if (gw >= payload_words) break;
-                    const unsigned bit0 = unsigned(j) * 32u;
-                    int o = int(__umulhi(bit0, div_magic));  // floor(bit0 / (4B)), octet inside the segment
-                    uint32_t word;
-                    if (B4 >= 32) {
-                        // an octet is at least as wide as a word: bits from octet o and, past its end, from o + 1
-                        const int sh = int(bit0) - o * B4;  // 0 <= sh < 4B
-                        const unsigned long long v0 = oct_s[Stage2<NS>::slot(o)];
-                        const unsigned long long v1 = o + 1 < WE / 8 ? oct_s[Stage2<NS>::slot(o + 1)] : 0ull;
-                        word = uint32_t(v0 >> sh) | uint32_t((v1 << (B4 - sh)) & 0xffffffffull);
-                    } else {
-                        word = 0;
-                        for (; o < WE / 8; ++o) {
-                            const int sh = o * B4 - int(bit0);
-                            if (sh >= 32) break;
-                            const unsigned long long v = oct_s[Stage2<NS>::slot(o)];
-                            word |= sh >= 0 ? uint32_t(v << sh) : uint32_t(v >> (-sh));
+                        for (int i = 0; i < 4; ++i) v[i] = search_cell<false>(s, z[i].x, z[i].y, word1[i]);
+                        // one of the four cells has more than four candidates, or points may lie beyond the table
+                        if (cell_overflows(word1[0] | word1[1] | word1[2] | word1[3] | careful)) {
+#pragma unroll
+                            for (int i = 0; i < 4; ++i) {
+                                if (careful && !(fmaxf(fabsf(z[i].x), fabsf(z[i].y)) < a.reach))
+                                    v[i] = search_exhaustive(s, z[i].x, z[i].y);
+                                else if (cell_overflows(word1[i]))
+                                    v[i] = search_overflow(s, word1[i], v[i], z[i].x, z[i].y);
+                            }
                         }
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) v[i] >>= s.log2_entry;
                     }
-                    out[gw] = word;
+                    // two indices fit a 32-bit word (B <= 12); octets beyond the row are packed as zero
+                    const uint32_t lo = v[0] | (v[1] << B), hi = v[2] | (v[3] << B);
+                    const bool in = live & (1u << p);
+                    octet[p].x = in ? lo | (2 * B < 32 ? hi << (2 * B) : 0u) : 0u;
+                    octet[p].y = in ? hi >> (32 - 2 * B) : 0u;
                 }
+                uint32_t* out = reinterpret_cast<uint32_t*>(cur.packed + (long long)row * cur.packed_row_stride) + seg_word0;
+                const int payload = row_words[0] - seg_word0;
+                store_indices<NS, LOG2B>(octet, first, B, out, payload, lane);
                 if (last_seg)  // padding up to the row stride is written as zero
-                    for (int gw = payload_words + lane; gw < row_words; gw += 32) out[gw] = 0u;
-                __syncwarp();  // the staging piece is free again
-                }  // MODE != 4
-            }
-            if constexpr (MODE == 4) {  // this row group's sums go to its own slot of the matrix's workspace
-                const int pair_stride = (n_pairs + 3) & ~3;
-                const int slot = (int(blockIdx.x) - cur.calib_first_block) * groups + group;
-                double* ws = reinterpret_cast<double*>(a.calib_base + cur.calib_offset);
-                double* mine = ws + size_t(slot) * pair_stride;
+                    for (int w = payload + lane; w < row_words[1] - seg_word0; w += 32) out[w] = 0u;
+            }  // !CALIB
+        }
+        if constexpr (CALIB) {
+            double* sums = reinterpret_cast<double*>(smem);  // [group][n_pairs]
+            if (group < groups) {
 #pragma unroll
                 for (int p = 0; p < NS; ++p)
-                    if (live[p]) {
+                    if (live & (1u << p)) {
                         const int k0 = 4 * (oct0 + Lay::octet_after(lane, p));
 #pragma unroll
-                        for (int i = 0; i < 4; ++i) mine[k0 + i] = acc[p][i];
+                        for (int i = 0; i < 4; ++i) sums[group * n_pairs + k0 + i] = acc[p][i];
                     }
-                if (lane == 0 && seg == 0) ws[size_t(cur.calib_slots) * pair_stride + slot] = double(used);
+                if (lane == 0 && seg == 0) used_rows[group] = used;
             }
-        };
-        if constexpr (CALIB) {
-            rows(std::integral_constant<int, 4>{});
-        } else if constexpr (POLAR) {
-            rows(std::integral_constant<int, 3>{});
-        } else {
-            if (a.brute) rows(std::integral_constant<int, 2>{});
-            else if (any_risky) rows(std::integral_constant<int, 1>{});
-            else rows(std::integral_constant<int, 0>{});
+            __syncthreads();
+            const int pair_stride = (n_pairs + 3) & ~3;
+            const int slot = int(blockIdx.x) - cur.calib_first_block;
+            double* ws = reinterpret_cast<double*>(a.calib_base + cur.calib_offset);
+            for (int k = threadIdx.x; k < n_pairs; k += blockDim.x) {
+                double v = 0.0;
+                for (int g = 0; g < groups; ++g) v += sums[g * n_pairs + k];
+                ws[size_t(slot) * pair_stride + k] = v;
+            }
+            if (threadIdx.x == 0) {
+                int n = 0;
+                for (int g = 0; g < groups; ++g) n += used_rows[g];
+                ws[size_t(cur.calib_slots) * pair_stride + slot] = double(n);
+            }
         }
     }
 }
 
-// sigma_k of every matrix from the slots of partial sums (zeroed before the calibration pass, so a
-// slot nobody wrote counts as empty).  A block owns 32 pair positions of one matrix; its eight
-// warps each add a contiguous slice of the slots in ascending order, and the eight slice sums are
-// then added in ascending order: the result does not depend on timing.
+// sigma_k of every matrix from the slots of partial sums, one per block that the matrix was spread over.  A block
+// owns 32 pair positions of one matrix; its eight warps each add a contiguous slice of the slots in ascending
+// order, and the eight slice sums are then added in ascending order: the result does not depend on timing.
 constexpr int kFinishSlices = 8;
-__global__ void __launch_bounds__(32 * kFinishSlices) calibrate_finish2_kernel(const MatDesc* descs,
+__global__ void __launch_bounds__(32 * kFinishSlices) calibrate_finish2_kernel(const MatDesc* descs, const MatDesc one,
                                                                              const unsigned char* calib_base) {
     __shared__ double part_sum[kFinishSlices][32], part_used[kFinishSlices];
     chain_release();
     chain_wait();
-    const MatDesc& d = descs[blockIdx.y];
+    const MatDesc& d = descs ? descs[blockIdx.y] : one;
     const int n_pairs = d.d_in >> 1, pair_stride = (n_pairs + 3) & ~3;
     if (int(blockIdx.x) * 32 >= n_pairs) return;
     const int lane = threadIdx.x & 31, slice = threadIdx.x >> 5;
@@ -791,10 +879,19 @@ __global__ void __launch_bounds__(32 * kFinishSlices) calibrate_finish2_kernel(c
     const int per = (d.calib_slots + kFinishSlices - 1) / kFinishSlices;
     const int s0 = min(d.calib_slots, slice * per), s1 = min(d.calib_slots, s0 + per);
     double sum = 0.0, used = 0.0;
-    for (int slot = s0; slot < s1; ++slot) {
-        if (k < n_pairs) sum += ws[size_t(slot) * pair_stride + k];
-        if (lane == 0) used += ws[size_t(d.calib_slots) * pair_stride + slot];
+    for (int slot = s0 + lane; slot < s1; slot += 32) used += ws[size_t(d.calib_slots) * pair_stride + slot];  // whole numbers: any order
+    if (k < n_pairs) {
+        int slot = s0;
+        for (; slot + 8 <= s1; slot += 8) {
+            double v[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) v[u] = ws[size_t(slot + u) * pair_stride + k];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) sum += v[u];
+        }
+        for (; slot < s1; ++slot) sum += ws[size_t(slot) * pair_stride + k];
     }
+    used = warp_total(used);
     part_sum[slice][lane] = sum;
     if (lane == 0) part_used[slice] = used;
     __syncthreads();
@@ -861,7 +958,7 @@ int launch_encode2(const Encode2Args& a, int blocks, int threads, size_t smem, c
         return launch_check("encode2_kernel (calibrate)",
                             launch_chained(encode2_kernel<BF16, LOG2B, NS, MAXT, 2>, blocks, threads, smem, st, a));
     }
-    if (a.polar_ba >= 0) {
+    if constexpr (LOG2B >= 5 && LOG2B <= 9) if (a.polar_ba >= 0) {
         int rc = raise_smem_limit(reinterpret_cast<const void*>(&encode2_kernel<BF16, LOG2B, NS, MAXT, 1>));
         if (rc) return rc;
         return launch_check("encode2_kernel (polar)",
@@ -953,21 +1050,33 @@ int rows_decode(const MatDesc* descs_dev, const MatDesc* descs_host, int n, cons
     return rc;
 }
 
-// Block sizes of the encoder: 20, 24 or 28 warps.  The register file is split over the four
-// schedulers of an SM, 16384 registers each, so 5, 6 or 7 warps per scheduler leave 96, 80 or 72
-// registers per thread.  A row of n_seg segments takes the size that keeps most warps busy (whole
-// groups of n_seg warps, at most 15 groups), and among equals the smallest: 0 if the row is too long.
+// Block sizes of the encoder: 16, 20, 24 or 28 warps.  The register file is split over the four
+// schedulers of an SM, 16384 registers each, so 4, 5, 6 or 7 warps per scheduler leave 128, 96, 80 or 72
+// registers per thread.  With all warps busy the sizes take 45.9, 47.6, 51.2 and 49.4 us for 8192 rows of 2048 (fewer
+// registers, less of a row's search in flight; the last two spill a little), and time grows with the share of warps
+// that a row length leaves idle (whole groups of n_seg warps, at most 15 groups): the size with the
+// largest product of the two is taken; 0 if the row is too long.
+// Hadamard blocks of 1024 elements need all 32 lanes with four octets each: 16 warps.
 int encode_groups(int warps, int n_seg) { return std::min(15, warps / n_seg); }
-int encode_warps(int n_seg) {
-    int best = 0, best_busy = 0;
-    for (int w = 20; w <= 28; w += 4) {
-        const int busy = encode_groups(w, n_seg) * n_seg;
-        if (busy > best_busy) {
-            best = w;
-            best_busy = busy;
+int encode_segment(int block) { return block == 1024 ? 1024 : 512; }
+constexpr int kEncodeClasses = 4;
+constexpr int kEncodeWarps[kEncodeClasses] = {16, 20, 24, 28};
+int encode_warps(int n_seg, int block) {
+    if (block == 1024) return n_seg <= 16 ? 16 : 0;
+    const double full[kEncodeClasses] = {1.0, 45.9 / 47.6, 45.9 / 51.2, 45.9 / 49.4};
+    int best = 0;
+    double best_rate = 0.0;
+    for (int c = 0; c < kEncodeClasses; ++c) {
+        const double rate = full[c] * encode_groups(kEncodeWarps[c], n_seg) * n_seg / kEncodeWarps[c];
+        if (rate > best_rate) {
+            best = kEncodeWarps[c];
+            best_rate = rate;
         }
     }
     return best;
+}
+int encode_class(int warps) {  // rows too long for any size end up in the last class and fall back later
+    return warps ? (warps - 16) / 4 : kEncodeClasses - 1;
 }
 int decode_groups(int n_seg) { return 16 / n_seg; }
 constexpr int kCostUnit = 360360;  // divisible by every group count 1..15
@@ -975,23 +1084,27 @@ constexpr int kCostUnit = 360360;  // divisible by every group count 1..15
 int rows_encode(const MatDesc* descs_dev, const MatDesc* descs_host, int n, const void* spans_dev, int span_blocks,
                 int block, int K, int w_bf16, const ::qamw_codebook* cb, uint32_t flags, int32_t* status, void* stream,
                 void* calib_base) {
-    constexpr int NS = 2, WE = 256 * NS;
-    const int log2b = ilog2(block);
-    if (log2b < 5 || log2b > 9 || n <= 0) return QAMW_ERR_SHAPE;
+    const int log2b = ilog2(block), WE = encode_segment(block), NS = WE / 256;
+    if (n <= 0) return QAMW_ERR_SHAPE;
     const size_t esz = w_bf16 ? 2 : 4;
     int max_seg = 1, warps = 0;
     long long rows = 0;
+    bool wide = true;
     for (int i = 0; i < n; ++i) {
         const MatDesc& d = descs_host[i];
-        if (d.d_in % (8 * NS)) return QAMW_ERR_SHAPE;
-        if (!aligned(d.W, 32) || (size_t(d.w_row_stride) * esz) % 32) return QAMW_ERR_SHAPE;
+        if (d.d_in % 8) return QAMW_ERR_SHAPE;
+        const size_t row_bytes = size_t(d.w_row_stride) * esz;
+        if (!aligned(d.W, 16) || row_bytes % 16) return QAMW_ERR_SHAPE;
+        wide = wide && aligned(d.W, 32) && row_bytes % 32 == 0 && d.d_in % (8 * NS) == 0;
         if (!aligned(d.chan_scale, 16) || !aligned(d.signs, 8) || (!calib_base && !aligned(d.sigma, 16))) return QAMW_ERR_SHAPE;
         const int n_seg = (d.d_in + WE - 1) / WE;
         max_seg = std::max(max_seg, n_seg);
-        warps = std::max(warps, encode_warps(n_seg));
-        rows += d.d_out;
+        warps = std::max(warps, encode_warps(n_seg, block));
+        rows += calib_base ? std::min(d.d_out, QAMW_CALIB_MAX_ROWS) : d.d_out;
     }
     if (max_seg > warps) return QAMW_ERR_SHAPE;  // also: a row too long for any block size
+    // the polar quantiser is built for the layouts of the models it is compared on
+    if (!calib_base && cb->polar && (log2b < 5 || log2b > 9 || !wide)) return QAMW_ERR_SHAPE;
     if (rows == 0) return QAMW_OK;
     Encode2Args a;
     a.descs = descs_dev;
@@ -1006,49 +1119,90 @@ int rows_encode(const MatDesc* descs_dev, const MatDesc* descs_host, int n, cons
     a.K = K;
     a.log2K = ilog2(K);
     a.grid = calib ? 1 : cb->map.grid;
-    a.map_zmax = calib ? 0.f : cb->map.zmax;
-    a.map_c0 = calib ? 0.f : cb->map.c0;
-    a.map_c1 = calib ? 0.f : cb->map.c1;
-    a.map_c2 = calib ? 0.f : cb->map.c2;
-    a.map_bias = calib ? 0.f : 12582912.0f + float(cb->map.half);
+    auto twice = [](float v) {
+        uint32_t bits;
+        std::memcpy(&bits, &v, 4);
+        return (f32x2(bits) << 32) | bits;
+    };
+    a.map_zlo = twice(calib ? 0.f : -cb->map.zmax);
+    a.map_c0 = twice(calib ? 0.f : cb->map.c0);
+    a.map_c1 = twice(calib ? 0.f : cb->map.c1);
+    a.map_c2 = twice(calib ? 0.f : cb->map.c2);
+    a.map_bias = twice(calib ? 0.f : 12582912.0f + float(cb->map.half));
+    a.log2b = log2b;
+    a.wide = wide;
     a.brute = (flags & QAMW_FLAG_BRUTE_FORCE) ? 1 : 0;
+    a.reach = a.brute ? -1.0f : 16000.0f;
     a.inv_sqrt_b = float(1.0 / std::sqrt(double(block)));
     a.status = status;
     const bool polar = !calib && cb->polar;
     a.polar_ba = polar ? cb->polar_ba : -1;
     a.polar_bp = polar ? cb->polar_bp : -1;
-    const size_t fixed = ((size_t(a.table_bytes) + 15) & ~size_t(15)) + size_t(warps) * Stage2<NS>::kSlots * 8;
-    if (!calib && fixed + size_t(K) * 8 > kSmemLimit - kEncode2StaticSmem) return QAMW_ERR_SHAPE;
     const bool tables = !calib && !polar;
-    a.log2c = tables ? pick_copies(K, 1 << 20, kSmemLimit - kEncode2StaticSmem - fixed) : 0;
-    const size_t smem = fixed + (tables ? (size_t(K) * 8 << a.log2c) : 0);
+    a.log2c = tables ? cb->log2c : 0;
+    // calibration: the block's groups meet in shared memory, a double per pair of every warp's segment
+    const size_t smem = calib ? size_t(warps) * (WE / 2) * sizeof(double)
+                              : ((size_t(a.table_bytes) + 15) & ~size_t(15)) + (tables ? size_t(K) * 8 << a.log2c : 0);
+    if (smem > kSmemLimit - kEncode2StaticSmem) return QAMW_ERR_SHAPE;
     int grid = sm_count();
     if (flags & QAMW_FLAG_HALF_DEVICE) grid = std::max(1, grid / 2);
-    const int blocks = spans_dev ? span_blocks : int(std::max<long long>(1, std::min<long long>(grid, rows)));
+    int blocks = spans_dev ? span_blocks : int(std::max<long long>(1, std::min<long long>(grid, rows)));
+    if (!spans_dev && calib) blocks = descs_host[0].calib_slots;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     int rc = QAMW_ERR_SHAPE;
 #define QAMW_ENC2(LB)                                                                          \
     case LB:                                                                                   \
         if (warps == 28)                                                                       \
-            rc = w_bf16 ? launch_encode2<true, LB, NS, 896>(a, blocks, 896, smem, st)          \
-                        : launch_encode2<false, LB, NS, 896>(a, blocks, 896, smem, st);        \
+            rc = w_bf16 ? launch_encode2<true, LB, 2, 896>(a, blocks, 896, smem, st)           \
+                        : launch_encode2<false, LB, 2, 896>(a, blocks, 896, smem, st);         \
         else if (warps == 24)                                                                  \
-            rc = w_bf16 ? launch_encode2<true, LB, NS, 768>(a, blocks, 768, smem, st)          \
-                        : launch_encode2<false, LB, NS, 768>(a, blocks, 768, smem, st);        \
+            rc = w_bf16 ? launch_encode2<true, LB, 2, 768>(a, blocks, 768, smem, st)           \
+                        : launch_encode2<false, LB, 2, 768>(a, blocks, 768, smem, st);         \
+        else if (warps == 20)                                                                  \
+            rc = w_bf16 ? launch_encode2<true, LB, 2, 640>(a, blocks, 640, smem, st)           \
+                        : launch_encode2<false, LB, 2, 640>(a, blocks, 640, smem, st);         \
         else                                                                                   \
-            rc = w_bf16 ? launch_encode2<true, LB, NS, 640>(a, blocks, 640, smem, st)          \
-                        : launch_encode2<false, LB, NS, 640>(a, blocks, 640, smem, st);        \
+            rc = w_bf16 ? launch_encode2<true, LB, 2, 512>(a, blocks, 512, smem, st)           \
+                        : launch_encode2<false, LB, 2, 512>(a, blocks, 512, smem, st);         \
         break;
-    switch (log2b) {
+    switch (log2b >= 5 ? log2b : 0) {
+        QAMW_ENC2(0)
         QAMW_ENC2(5)
         QAMW_ENC2(6)
         QAMW_ENC2(7)
         QAMW_ENC2(8)
         QAMW_ENC2(9)
+        case 10:
+            rc = w_bf16 ? launch_encode2<true, 10, 4, 512>(a, blocks, 512, smem, st)
+                        : launch_encode2<false, 10, 4, 512>(a, blocks, 512, smem, st);
+            break;
         default: break;
     }
 #undef QAMW_ENC2
     return rc;
+}
+
+int rows_calibrate(MatDesc d, int block, int w_bf16, uint32_t flags, void* workspace, size_t workspace_bytes, int32_t* status,
+                   void* stream) {
+    const int n_rows = std::min(d.d_out, QAMW_CALIB_MAX_ROWS);
+    if (n_rows == 0) return QAMW_ERR_SHAPE;
+    // as many blocks as have a row for each of their groups: every one leaves a slot for the finish to add up
+    const int WE = encode_segment(block), n_seg = (d.d_in + WE - 1) / WE, warps = encode_warps(n_seg, block);
+    if (!warps) return QAMW_ERR_SHAPE;
+    int grid = sm_count();
+    if (flags & QAMW_FLAG_HALF_DEVICE) grid = std::max(1, grid / 2);
+    const int groups = encode_groups(warps, n_seg);
+    const size_t slot = (size_t((d.d_in / 2 + 3) & ~3) + 1) * sizeof(double);
+    d.calib_offset = 0;
+    d.calib_first_block = 0;
+    d.calib_slots = int(std::min<size_t>(size_t(std::min(grid, (n_rows + groups - 1) / groups)), workspace_bytes / slot));
+    if (d.calib_slots < 1) return QAMW_ERR_SHAPE;
+    const int rc = rows_encode(nullptr, &d, 1, nullptr, 0, block, 2, w_bf16, nullptr, flags, status, stream, workspace);
+    if (rc) return rc;
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    return launch_check("calibrate_finish2_kernel",
+                        launch_chained(calibrate_finish2_kernel, dim3(unsigned((d.d_in / 2 + 31) / 32)), 32 * kFinishSlices, 0, st,
+                                       nullptr, d, static_cast<unsigned char*>(workspace)));
 }
 
 }  // namespace qamw
@@ -1073,7 +1227,7 @@ struct qamw_batch {
     std::vector<qamw_matrix> items;
     int n_blocks = 0;
     RowSet dec;                     // all matrices, spans weighted for the decoder's geometry
-    RowSet enc[3];                  // encoder: one set per block size (20, 24, 28 warps)
+    RowSet enc[kEncodeClasses];     // encoder: one set per block size
     int4* d_spans_dist = nullptr;   // distortion: spans of the concatenated work-item list, over dec.d_descs
     int n_blocks_dist = 0;
     double* d_dist_partial = nullptr;   // one record of four sums per (block, matrix of its span)
@@ -1081,7 +1235,7 @@ struct qamw_batch {
     unsigned int* d_dist_counter = nullptr;  // ticket of the blocks; zero between launches
     MatDesc* d_cal_all = nullptr;       // calibration descriptors of all block-size classes, for the one finish launch
     int cal_all_n = 0, cal_all_max_pairs = 0;
-    RowSet cal[3];                  // calibration: the encoder's sets again, spans over the calibration rows
+    RowSet cal[kEncodeClasses];     // calibration: the encoder's sets again, spans over the calibration rows
     size_t cal_bytes = 0;           // partial-sum slots of all matrices (front of the caller's workspace)
     std::vector<size_t> ws_offset;  // calibration scratch of item i inside the caller's workspace
     size_t ws_bytes = 0;
@@ -1156,24 +1310,24 @@ extern "C" int qamw_batch_create(const qamw_matrix* items, int n, const qamw_cod
     b->cb = cb;
     b->items.assign(items, items + n);
     b->n_blocks = sm_count();
-    std::vector<int> dec_cost, enc_cost[3];
+    std::vector<int> dec_cost, enc_cost[kEncodeClasses];
     for (int i = 0; i < n; ++i) {
         const MatDesc d = make_desc(items[i]);
         b->ws_offset.push_back(b->ws_bytes);
         b->ws_bytes += (qamw_calibrate_workspace_bytes(&items[i].p) + 255) & ~size_t(255);
-        const int seg4 = (d.d_in + 1023) / 1024, seg2 = (d.d_in + 511) / 512;
+        const int seg4 = (d.d_in + 1023) / 1024, seg2 = (d.d_in + encode_segment(b->block) - 1) / encode_segment(b->block);
         b->dec.index.push_back(i);
         b->dec.descs.push_back(d);
         dec_cost.push_back(kCostUnit / std::max(1, decode_groups(std::min(seg4, 16))));
-        const int warps = encode_warps(seg2);
-        const int c = warps == 20 ? 0 : (warps == 24 ? 1 : 2);  // rows too long for any size end up in the last set and fall back later
+        const int warps = encode_warps(seg2, b->block);
+        const int c = encode_class(warps);
         b->enc[c].index.push_back(i);
         b->enc[c].descs.push_back(d);
         enc_cost[c].push_back(kCostUnit / std::max(1, encode_groups(warps ? warps : 28, std::min(seg2, 28))));
     }
     e = upload_row_set(b->dec, b->n_blocks, dec_cost);
-    for (int c = 0; c < 3 && e == cudaSuccess; ++c) e = upload_row_set(b->enc[c], b->n_blocks, enc_cost[c]);
-    for (int c = 0; c < 3 && e == cudaSuccess; ++c) {  // calibration: min(d_out, 1024) rows per matrix
+    for (int c = 0; c < kEncodeClasses && e == cudaSuccess; ++c) e = upload_row_set(b->enc[c], b->n_blocks, enc_cost[c]);
+    for (int c = 0; c < kEncodeClasses && e == cudaSuccess; ++c) {  // calibration: min(d_out, 1024) rows per matrix
         RowSet& r = b->cal[c];
         r.index = b->enc[c].index;
         r.descs = b->enc[c].descs;
@@ -1191,9 +1345,8 @@ extern "C" int qamw_batch_create(const qamw_matrix* items, int n, const qamw_cod
             }
         for (int i = 0; i < m; ++i) {
             MatDesc& d = r.descs[size_t(i)];
-            const int groups = kCostUnit / enc_cost[c][size_t(i)];
             d.calib_first_block = first[size_t(i)];
-            d.calib_slots = std::max(0, last[size_t(i)] - first[size_t(i)] + 1) * groups;
+            d.calib_slots = std::max(0, last[size_t(i)] - first[size_t(i)] + 1);
             d.calib_offset = (long long)b->cal_bytes;
             const size_t pair_stride = (size_t(d.d_in / 2) + 3) & ~size_t(3);
             b->cal_bytes += ((size_t(d.calib_slots) * (pair_stride + 1)) * sizeof(double) + 255) & ~size_t(255);
@@ -1205,7 +1358,7 @@ extern "C" int qamw_batch_create(const qamw_matrix* items, int n, const qamw_cod
     }
     if (e == cudaSuccess) {  // all calibration descriptors in one array: one finish launch for every class
         std::vector<MatDesc> all;
-        for (int c = 0; c < 3; ++c) all.insert(all.end(), b->cal[c].descs.begin(), b->cal[c].descs.end());
+        for (int c = 0; c < kEncodeClasses; ++c) all.insert(all.end(), b->cal[c].descs.begin(), b->cal[c].descs.end());
         b->cal_all_n = int(all.size());
         for (const MatDesc& d : all) b->cal_all_max_pairs = std::max(b->cal_all_max_pairs, d.d_in / 2);
         if (!all.empty()) {
@@ -1256,7 +1409,7 @@ extern "C" int qamw_batch_create(const qamw_matrix* items, int n, const qamw_cod
 extern "C" void qamw_batch_destroy(qamw_batch* b) {
     if (!b) return;
     free_row_set(b->dec);
-    for (int c = 0; c < 3; ++c) {
+    for (int c = 0; c < kEncodeClasses; ++c) {
         free_row_set(b->enc[c]);
         free_row_set(b->cal[c]);
     }
@@ -1282,26 +1435,18 @@ extern "C" int qamw_calibrate_batch(const qamw_batch* b, void* workspace, size_t
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const uint32_t flags = b->items[0].p.flags;
     unsigned char* ws = static_cast<unsigned char*>(workspace);
-    bool zeroed = false;
     // One pass per block size; the partial sums of all of them are finished by one launch, unless a class
     // had to go through the single-matrix kernels (then the classes that did not are finished one by one).
-    bool fast[3] = {false, false, false}, any_general = false;
-    for (int c = 0; c < 3; ++c) {
+    bool fast[kEncodeClasses] = {}, any_fast = false, any_general = false;
+    for (int c = 0; c < kEncodeClasses; ++c) {
         const RowSet& set = b->cal[c];
         if (set.descs.empty()) continue;
         int rc = QAMW_ERR_SHAPE;
         if (!(flags & QAMW_FLAG_GENERAL_KERNELS)) {
-            if (!zeroed) {  // a slot that no row group writes must read as empty
-                cudaError_t e = cudaMemsetAsync(ws, 0, b->cal_bytes, st);
-                if (e != cudaSuccess) {
-                    set_cuda_error("cudaMemsetAsync", int(e));
-                    return QAMW_ERR_CUDA;
-                }
-                zeroed = true;
-            }
             rc = rows_encode(set.d_descs, set.descs.data(), int(set.descs.size()), set.d_spans, b->n_blocks, b->block, b->K,
                              b->w_dtype == QAMW_DTYPE_BF16, nullptr, flags, status_out, stream, ws);
             fast[c] = rc == QAMW_OK;
+            any_fast = any_fast || fast[c];
         }
         if (rc == QAMW_ERR_SHAPE) {  // some matrix of the set needs the general kernel: one call per matrix
             any_general = true;
@@ -1315,19 +1460,19 @@ extern "C" int qamw_calibrate_batch(const qamw_batch* b, void* workspace, size_t
         }
         if (rc) return rc;
     }
-    if (!any_general && (fast[0] || fast[1] || fast[2])) {
+    if (!any_general && any_fast) {
         return launch_check("calibrate_finish2_kernel",
                             launch_chained(calibrate_finish2_kernel, dim3(unsigned((b->cal_all_max_pairs + 31) / 32), unsigned(b->cal_all_n)),
-                                           32 * kFinishSlices, 0, st, b->d_cal_all, ws));
+                                           32 * kFinishSlices, 0, st, b->d_cal_all, MatDesc{}, ws));
     }
-    for (int c = 0; c < 3; ++c) {
+    for (int c = 0; c < kEncodeClasses; ++c) {
         if (!fast[c]) continue;
         const RowSet& set = b->cal[c];
         int max_pairs = 0;
         for (const MatDesc& d : set.descs) max_pairs = std::max(max_pairs, d.d_in / 2);
         const int rc = launch_check("calibrate_finish2_kernel",
                                     launch_chained(calibrate_finish2_kernel, dim3(unsigned((max_pairs + 31) / 32), unsigned(set.descs.size())),
-                                                   32 * kFinishSlices, 0, st, set.d_descs, ws));
+                                                   32 * kFinishSlices, 0, st, set.d_descs, MatDesc{}, ws));
         if (rc) return rc;
     }
     return QAMW_OK;
@@ -1340,7 +1485,7 @@ extern "C" int qamw_encode_batch(const qamw_batch* b, int32_t* status_out, void*
         if (!it.W || !it.sigma || !it.packed || !it.row_norm) return QAMW_ERR_ARG;
     }
     const uint32_t flags = b->items[0].p.flags;
-    for (int c = 0; c < 3; ++c) {  // one launch per block size
+    for (int c = 0; c < kEncodeClasses; ++c) {  // one launch per block size
         const RowSet& set = b->enc[c];
         if (set.descs.empty()) continue;
         int rc = QAMW_ERR_SHAPE;

@@ -272,7 +272,37 @@ bool pack_search_table(const CellLists& cl, SearchTable* out) {
     return true;
 }
 
-bool choose_search_table(const float* codebook, int K, int grid, size_t budget_bytes, SearchTable* out) {
+bool pack_device_table(const SearchTable& t, int K, int log2_entry, std::vector<uint32_t>* words, std::vector<uint16_t>* lists) {
+    const int B = ilog2(K), list_shift = log2_entry + B;
+    const size_t n_cells = t.cells.size() / 4;
+    words->assign(2 * n_cells, 0);
+    lists->clear();
+    std::vector<uint16_t> entries;
+    auto word = [&](uint32_t lo, uint32_t hi) { return (lo << log2_entry) | (hi << (32 - B)); };
+    const size_t base = size_t(t.n_overflow_cells) + 1;  // the lists come after their starts
+    for (size_t c = 0; c < n_cells; ++c) {
+        const uint16_t* rec = &t.cells[4 * c];
+        uint32_t* w = &(*words)[2 * c];
+        if (rec[0] != 0xFFFF) {
+            w[0] = word(rec[0], rec[1]);
+            w[1] = word(rec[2], rec[3]) | (rec[3] != rec[2] ? 2u : 0u);
+            continue;
+        }
+        const uint16_t* list = &t.overflow[rec[1]];
+        if ((lists->size() >> (32 - list_shift)) != 0 || base + entries.size() > 0xFFFF) return false;
+        w[0] = word(list[0], list[1]);
+        w[1] = (uint32_t(list[2]) << log2_entry) | (uint32_t(lists->size()) << list_shift) | 1u;
+        lists->push_back(uint16_t(base + entries.size()));
+        entries.insert(entries.end(), list + 3, list + rec[2]);
+    }
+    if (base + entries.size() > 0xFFFF) return false;
+    lists->push_back(uint16_t(base + entries.size()));
+    lists->insert(lists->end(), entries.begin(), entries.end());
+    while ((words->size() * 4 + lists->size() * 2) % 16) lists->push_back(0);  // copied in 16-byte pieces
+    return true;
+}
+
+bool choose_search_table(const float* codebook, int K, int grid, size_t budget_bytes, SearchTable* out, int first) {
     std::vector<double> cb(static_cast<size_t>(2 * K), 0.0);
     for (int i = 0; i < 2 * K; ++i) cb[size_t(i)] = double(codebook[i]);
     VoronoiSet vs;
@@ -283,7 +313,7 @@ bool choose_search_table(const float* codebook, int K, int grid, size_t budget_b
     for (double T : {17.0, 18.0, 19.0})
         for (double eps : {0.015, 0.02})
             for (double rho : {1.22, 1.27}) shapes.push_back(MapShape{T, eps, rho});
-    for (int g = grid > 0 ? grid : default_grid(K); g >= 1; g -= 2) {
+    for (int g = grid > 0 ? grid : first > 0 ? first : default_grid(K); g >= 1; g -= 2) {
         if (size_t(g) * g * 8 <= budget_bytes) {
             bool found = false;
             double best = INFINITY;

@@ -273,19 +273,18 @@ class ModelCodec:
         if self.use_batch and self.batch is not None:
             # one encoder block size per class of row lengths: a calibration pass and an encode launch per
             # class; one finish launch, one decode launch, one distortion launch
-            classes = len({self._encoder_class(s.d_in) for s in self.slots})
+            classes = len({self._encoder_class(s.d_in, self.spec.block) for s in self.slots})
             return 2 * classes + 3
         return 5 * n
 
     @staticmethod
-    def _encoder_class(d_in: int) -> int:
+    def _encoder_class(d_in: int, block: int) -> int:
+        """Warps of the encoder's block for this row length (the rule of the library)."""
+        if block == 1024:
+            return 16
         n_seg = (d_in + 511) // 512
-        best, busy = 0, 0
-        for w in (20, 24, 28):
-            b = min(15, w // n_seg) * n_seg
-            if b > busy:
-                best, busy = w, b
-        return best
+        full = {16: 1.0, 20: 45.9 / 47.6, 24: 45.9 / 51.2, 28: 45.9 / 49.4}
+        return max(full, key=lambda w: full[w] * (min(15, w // n_seg) * n_seg) / w)
 
     def totals(self, group=None) -> Dict[str, float]:
         """Error figures over all matrices of all ranks (see combine_distortion)."""

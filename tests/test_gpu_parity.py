@@ -658,3 +658,37 @@ def test_batch_with_the_polar_quantiser(orc):
     for x, y in zip(a, b):
         assert torch.equal(x["packed"], y["packed"]) and torch.equal(x["norm"], y["norm"])
         assert torch.equal(x["what"].view(torch.int16), y["what"].view(torch.int16))
+
+
+@pytest.mark.parametrize("K", [2, 8, 64, 128, 256, 1024, 2048, 4096])
+@pytest.mark.parametrize("d_out,d_in,block,dtype", [
+    (3, 8, 2, torch.float32), (65, 1000, 8, torch.bfloat16), (33, 1048, 4, torch.float32), (40, 2744, 8, torch.bfloat16),
+    (21, 4112, 16, torch.bfloat16), (150, 1024, 1024, torch.bfloat16), (9, 13312, 1024, torch.float32),
+    (30, 8192, 512, torch.bfloat16), (17, 3584, 256, torch.bfloat16), (12, 5632, 128, torch.float32)])
+def test_row_kernels_agree_with_the_general_ones_on_every_layout(orc, K, d_out, d_in, block, dtype):
+    """Calibration, encoder and decoder for every block class, odd widths and all index widths: the same streams, norms
+    and (to rounding) scales and weights as the kernels for arbitrary layouts."""
+    W, act = _make(d_out, d_in, dtype, K + d_in)
+    W[d_out // 2] *= 1e-3
+    W[1, ::7] *= 50.0
+    cb = q.Codebook(orc.train_codebook(K, 1 << 13, 5, 2, 1e-6)[0])
+    Wd = W.to(DEV)
+    s = torch.from_numpy(q.channel_scales(act, 0.3)).to(DEV)
+    signs = torch.from_numpy(q.make_signs(q.DEFAULT_SIGN_SEED, d_in)).to(DEV)
+    got = []
+    for flags in (0, q.FLAG_GENERAL_KERNELS):
+        p = q.make_params(Wd, d_out, d_in, block, K, flags)
+        sigma = torch.empty(d_in // 2, dtype=torch.float32, device=DEV)
+        ws = torch.empty(max(8, q.calibrate_workspace_bytes(p)), dtype=torch.uint8, device=DEV)
+        q.calibrate(Wd, p, s, signs, sigma, ws)
+        shared = got[0][0] if got else sigma  # both encode with the same pair scales
+        packed = torch.full((d_out, p.packed_row_stride), 0xAA, dtype=torch.uint8, device=DEV)
+        norm = torch.empty(d_out, dtype=torch.float32, device=DEV)
+        q.encode(Wd, p, s, signs, shared, cb, packed, norm)
+        w_hat = torch.empty((d_out, d_in), dtype=torch.bfloat16, device=DEV)
+        q.decode(packed, norm, s, signs, shared, cb, p, w_hat)
+        got.append((sigma, packed, norm, w_hat))
+    (sig, packed, norm, w_hat), (sig_g, packed_g, norm_g, w_hat_g) = got
+    torch.testing.assert_close(sig, sig_g, rtol=1e-6, atol=0)
+    assert torch.equal(packed, packed_g) and torch.equal(norm, norm_g)
+    assert torch.equal(w_hat.view(torch.int16), w_hat_g.view(torch.int16))
