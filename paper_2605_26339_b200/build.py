@@ -11,7 +11,7 @@ _INC = os.path.join(os.path.dirname(_PKG), "include")
 LIB_PATH = os.path.join(_PKG, "libqamw.so")
 EXT_PATH = os.path.join(_PKG, "_qamw.so")
 EXT_SOURCE = "qamw_py.cpp"
-SOURCES = ["qamw_kernels.cu", "qamw_rows.cu", "qamw_lloyd.cu", "qamw_variants.cu", "qamw_gemv.cu", "qamw_host.cpp", "qamw_table.cpp"]
+SOURCES = ["qamw_kernels.cu", "qamw_rows.cu", "qamw_prepare.cu", "qamw_lloyd.cu", "qamw_variants.cu", "qamw_gemv.cu", "qamw_host.cpp", "qamw_table.cpp"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC,-Wall,-Wextra", "-shared", "-t", "0"]
 

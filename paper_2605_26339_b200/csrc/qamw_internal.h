@@ -108,6 +108,9 @@ int rows_decode(const MatDesc* descs_dev, const MatDesc* descs_host, int n, cons
 int rows_encode(const MatDesc* descs_dev, const MatDesc* descs_host, int n, const void* spans_dev, int span_blocks,
                 int block, int K, int w_bf16, const ::qamw_codebook* cb, uint32_t flags, int32_t* status, void* stream,
                 void* calib_base = nullptr);  // calib_base: run the calibration pass instead (cb may be NULL)
+// Sign mask and, if act_host is not NULL, channel scales of the columns, on the stream (qamw_prepare.cu); act_host
+// may be overwritten as soon as the call returns.
+int prepare_columns(const float* act_host, int d_in, float alpha, uint64_t seed, float* chan_scale, int8_t* signs, void* stream);
 // The calibration pass and its finish for one matrix; QAMW_ERR_SHAPE as above.
 int rows_calibrate(MatDesc d, int block, int w_bf16, uint32_t flags, void* workspace, size_t workspace_bytes, int32_t* status,
                    void* stream);

@@ -1733,22 +1733,8 @@ extern "C" int qamw_quantize(const void* W, const qamw_params* p, const float* a
     const bool scaled = act_rms_host && alpha != 0.f;
     if (scaled && !chan_scale_out) return QAMW_ERR_ARG;
     if (workspace_bytes < qamw_calibrate_workspace_bytes(p)) return QAMW_ERR_NOMEM;
-    cudaStream_t st = static_cast<cudaStream_t>(stream);
-    // E0 and the sign mask are d_in numbers each: computed on the host, copied once
-    std::vector<int8_t> signs(size_t(p->d_in));
-    rc = qamw_make_signs(sign_seed, p->d_in, signs.data());
+    rc = prepare_columns(scaled ? act_rms_host : nullptr, p->d_in, alpha, sign_seed, chan_scale_out, signs_out, stream);
     if (rc) return rc;
-    cudaError_t e = cudaMemcpyAsync(signs_out, signs.data(), signs.size(), cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess && scaled) {
-        std::vector<float> s(size_t(p->d_in));
-        rc = qamw_channel_scales(act_rms_host, p->d_in, alpha, s.data());
-        if (rc) return rc;
-        e = cudaMemcpyAsync(chan_scale_out, s.data(), s.size() * sizeof(float), cudaMemcpyHostToDevice, st);
-    }
-    if (e != cudaSuccess) {
-        set_cuda_error("qamw_quantize: cudaMemcpyAsync", int(e));
-        return QAMW_ERR_CUDA;
-    }
     const float* cs = scaled ? chan_scale_out : nullptr;
     rc = qamw_calibrate(W, p, cs, signs_out, sigma_out, workspace, workspace_bytes, status_out, stream);
     if (rc) return rc;

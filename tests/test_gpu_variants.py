@@ -214,3 +214,23 @@ def test_fused_gemv_rows_off_16_byte_boundaries(orc, K, d_out, d_in, n_vec):
     ref = w64 @ x.numpy().astype(np.float64).T
     bound = 1e-5 * np.sqrt((w64 ** 2).sum(1))[:, None] * np.sqrt((x.numpy().astype(np.float64) ** 2).sum(1))[None, :]
     assert np.all(np.abs(y.cpu().numpy() - ref) <= bound + 1e-30)
+
+
+@pytest.mark.parametrize("d_in", [2, 1024, 1026, 2050, 4098, 8064, 8066, 16384])
+@pytest.mark.parametrize("alpha", [0.0, 0.3])
+def test_quantize_prepares_the_columns_as_the_host_functions_do(d_in, alpha):
+    """Channel scales and signs that qamw_quantize computes on the device, around every size of its parameter blocks."""
+    W, act = _problem(d_in, 3, d_in)
+    act[0], act[-1] = 0.0, 1e30
+    cb = q.Codebook(load_golden_codebook(64))
+    Wd = W.to(DEV)
+    p = q.make_params(Wd, 3, d_in, 2, 64)
+    new = lambda n, dt: torch.empty(n, dtype=dt, device=DEV)
+    s, signs, sigma, norm = new(d_in, torch.float32), new(d_in, torch.int8), new(d_in // 2, torch.float32), new(3, torch.float32)
+    packed, ws = new((3, p.packed_row_stride), torch.uint8), new(max(8, q.calibrate_workspace_bytes(p)), torch.uint8)
+    host = act.copy()
+    q.quantize(Wd, p, host, alpha, 123456789, cb, s, signs, sigma, packed, norm, ws)
+    host[:] = -1.0  # the statistics belong to the caller again
+    assert np.array_equal(signs.cpu().numpy(), q.make_signs(123456789, d_in))
+    if alpha:
+        np.testing.assert_allclose(s.cpu().numpy(), q.channel_scales(act, alpha), rtol=1.2e-7)
