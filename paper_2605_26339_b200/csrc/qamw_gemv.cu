@@ -201,14 +201,6 @@ __device__ __forceinline__ float warp_sums(float (&v)[N], int lane) {
     return v[0];
 }
 
-template <int N>
-__device__ __forceinline__ void cp_async_wait_pending() {
-    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
-}
-// 16 bytes of shared memory, of which the first n come from global memory (nothing else is read) and the rest is zero
-__device__ __forceinline__ void cp_async_upto16(unsigned char* dst, const unsigned char* src, int n) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_addr(dst)), "l"(src), "r"(n) : "memory");
-}
 
 // Rotated activations of one slice, by one warp: lane l gets chunk 32 slice + l of each vector,
 // xr[v][i] = sigma_k (F S D_s^-1 x_v) at pair k = 16 chunk + i; zero beyond the row.  The columns are read

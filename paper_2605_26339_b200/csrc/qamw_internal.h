@@ -122,11 +122,10 @@ int sm_count();
 int pick_copies(int K, long long gathers, size_t budget);
 int check_matrix_params(const qamw_params* p);
 long long distortion_items(int d_out, int d_in);  // work items of the distortion kernel for one matrix
-// zeroes every matrix's four sums, then one launch over all matrices (spans of the concatenated item list)
 // Where the blocks of the batched distortion kernel leave their partial sums: records of four doubles,
 // matrix by matrix; matrix m appears in the spans of blocks owner[m].first .. owner[m].last and block b's
-// record for it is number owner[m].offset + b - owner[m].first.  counter is the ticket of the blocks;
-// the one that finishes last adds the records up in a fixed order and resets it.
+// record for it is number owner[m].offset + b - owner[m].first.  counter[m] counts the blocks that have left theirs;
+// the last one adds the records up in a fixed order and resets it.
 struct DistOwner {
     int first, last;  // blocks
     int offset;       // first record of the matrix
@@ -134,9 +133,9 @@ struct DistOwner {
 struct DistReduce {
     double* partial;
     const DistOwner* owner;
-    unsigned int* counter;  // zero between launches
+    unsigned int* counter;  // one per matrix, zero between launches
 };
-int distortion_batch_launch(const MatDesc* descs_dev, int n, const void* spans_dev, int blocks, int w_bf16,
+int distortion_batch_launch(const MatDesc* descs_dev, const void* spans_dev, int blocks, int w_bf16,
                             const DistReduce& red, void* stream);  // QAMW_OK or the error code every entry point reports
 
 }  // namespace qamw

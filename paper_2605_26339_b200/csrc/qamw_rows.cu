@@ -1,5 +1,5 @@
-// Row kernels of libqamw for the common layouts (32-byte aligned rows, d_in a multiple of 16,
-// Hadamard blocks of 32 elements or more): one persistent launch walks any number of matrices.
+// Row kernels of libqamw for the common layouts (16-byte aligned rows of W, d_in a multiple of 8): one persistent launch
+// walks any number of matrices.
 //
 // Geometry.
 //   * A warp owns a "segment" of 256 * NS consecutive elements of a row: NS = 4 octets (32 elements)
@@ -216,10 +216,6 @@ __device__ __forceinline__ int4 block_span(const int4* spans, int d_out_single) 
 // decoder
 // ---------------------------------------------------------------------------------------------
 constexpr int kDecodeDepth = 4;
-template <int N>
-__device__ __forceinline__ void cp_async_wait_pending() {
-    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
-}
 
 struct Decode2Args {
     const MatDesc* descs;    // device array, or NULL: `one` is the only matrix
@@ -228,18 +224,20 @@ struct Decode2Args {
     const float2* codebook;  // device, K entries
     int K, log2K, log2c;
     int seg_bytes;           // packed bytes of one warp segment: 16 * NS * B
-    int stage_bytes;         // one staging buffer of a warp (128-byte aligned, at least seg_bytes + 16)
+    int stage_bytes;         // one staging buffer of a warp (128-byte aligned, at least seg_bytes + 28)
+    int log2b;               // log2 of the Hadamard block
     float inv_sqrt_b;
 };
 
 // A warp streams its segment of the packed row through its own shared-memory ring of kDecodeDepth rows
 // (16-byte asynchronous copies, kDecodeDepth - 1 rows ahead: with one row in flight per warp the reads
 // are bound by memory latency); nothing is shared between warps after the prologue, so there is no
-// barrier.
+// barrier.  A row that starts off a 16-byte boundary is copied from the boundary below it and read at an offset.
 // Per row a thread reads its 4 NS B index bits as two runs of 32-bit words, gathers the codewords
 // (stored as (x + y, x - y): butterfly stage h = 1) from its own bank-separated copy, scales them by
 // the pair scales, runs the remaining butterflies and writes bf16.
-template <int NS, int LOG2B>
+// ALIGNED: packed rows start on 16 bytes, rows of the output on 32, d_in is a multiple of 16.
+template <int NS, int LOG2B, bool ALIGNED>
 __global__ void __launch_bounds__(NS == 4 ? 512 : 896, 1) decode2_kernel(const Decode2Args a) {
     typedef Lay2<NS, LOG2B> Lay;
     constexpr int TOP = Lay::TOP;
@@ -255,8 +253,6 @@ __global__ void __launch_bounds__(NS == 4 ? 512 : 896, 1) decode2_kernel(const D
 
     chain_release();
     fill_codebook_copies(reinterpret_cast<float2*>(smem), a.codebook, a.K, a.log2c, true);
-    // the 16 bytes after a staged segment are read (and masked away) by the last threads: keep them defined
-    if (lane < 4 * kDecodeDepth) reinterpret_cast<uint32_t*>(stage + (lane >> 2) * a.stage_bytes + a.seg_bytes)[lane & 3] = 0u;
     __syncthreads();
     chain_wait();
 
@@ -284,19 +280,29 @@ __global__ void __launch_bounds__(NS == 4 ? 512 : 896, 1) decode2_kernel(const D
         const int row_step = groups;
         const int n_rows = (row_end - row0 + row_step - 1) / row_step;
         const long long pstride = d.packed_row_stride;
-        const int row_bytes = int((((long long)n_pairs * B + 7) / 8 + 15) & ~15LL);  // <= stride (a multiple of 16)
+        constexpr int kGran = ALIGNED ? 16 : 4;  // of row starts: the stride is a multiple of it, and a row may be read up to one
+        const int row_bytes = int((((long long)n_pairs * B + 7) / 8 + kGran - 1) & ~(long long)(kGran - 1));
         const long long seg_off = (long long)seg * a.seg_bytes;
-        const int n_chunks = max(0, min(a.seg_bytes, row_bytes - int(seg_off))) >> 4;
-        // at most 48 chunks of 16 bytes per segment: two predicated copies per lane, no loop
-        const bool copy0 = lane < n_chunks, copy1 = lane + 32 < n_chunks;
+        const int seg_len = max(0, min(a.seg_bytes, row_bytes - int(seg_off)));
         const unsigned char* src = d.packed + (long long)row0 * pstride + seg_off;  // next row to fetch
         const long long src_step = (long long)row_step * pstride;
+        uint32_t off = ALIGNED ? 0u : uint32_t(reinterpret_cast<uintptr_t>(src) & 15);  // of the row decoded next from the boundary below it
+        const uint32_t off_step = ALIGNED ? 0u : uint32_t(src_step & 15);
+        const bool copy0 = (lane << 4) < seg_len, copy1 = (lane << 4) + 512 < seg_len;  // two pieces of 16 bytes per lane, no loop
         int issued = 0;
         auto issue_row = [&]() {  // one commit group per row, empty past the end
             if (issued < n_rows) {
-                unsigned char* dst = stage + (issued % kDecodeDepth) * a.stage_bytes;
-                if (copy0) cp_async(dst + (lane << 4), src + (lane << 4), 4);
-                if (copy1) cp_async(dst + ((lane + 32) << 4), src + ((lane + 32) << 4), 4);
+                unsigned char* dst = stage + (issued % kDecodeDepth) * a.stage_bytes + (lane << 4);
+                if constexpr (ALIGNED) {
+                    if (copy0) cp_async(dst, src + (lane << 4), 4);
+                    if (copy1) cp_async(dst + 512, src + (lane << 4) + 512, 4);
+                } else {
+                    const int mis = int(reinterpret_cast<uintptr_t>(src) & 15);
+                    const unsigned char* from = src - mis + (lane << 4);
+                    const int left = mis + seg_len - (lane << 4);
+                    if (left > 0) cp_async_upto16(dst, from, min(16, left));
+                    if (left > 512) cp_async_upto16(dst + 512, from + 512, min(16, left - 512));
+                }
                 src += src_step;
             }
             ++issued;
@@ -309,7 +315,6 @@ __global__ void __launch_bounds__(NS == 4 ? 512 : 896, 1) decode2_kernel(const D
         const int oct0 = seg * (WE / 8);  // first octet of the segment
         float sg[NS][4];
         f32x2 mcol[NS][4];
-        bool store_ok[NS];
         int e_out[NS];
 #pragma unroll
         for (int p = 0; p < NS; ++p) {
@@ -317,7 +322,6 @@ __global__ void __launch_bounds__(NS == 4 ? 512 : 896, 1) decode2_kernel(const D
             load4f(d.sigma, k0, n_pairs, 1, 0.f, sg[p]);
             const int e0 = 8 * (oct0 + Lay::octet_after(lane, p));
             e_out[p] = e0;
-            store_ok[p] = e0 < d_in;
             float cs[8], sgn[8];
             if (d.chan_scale) {
                 load8f(d.chan_scale, e0, d_in, 1, 1.0f, cs);
@@ -341,7 +345,8 @@ __global__ void __launch_bounds__(NS == 4 ? 512 : 896, 1) decode2_kernel(const D
             cp_async_wait_pending<kDecodeDepth - 2>();
             __syncwarp();  // every lane's part of this row has landed; the buffer refilled next is no longer read
             issue_row();
-            const uint32_t in = stage_addr + uint32_t((it % kDecodeDepth) * a.stage_bytes);
+            const uint32_t in = stage_addr + uint32_t((it % kDecodeDepth) * a.stage_bytes) + off;
+            if (!ALIGNED) off = (off + off_step) & 15u;
             f32x2 P[NS][4];
 #pragma unroll
             for (int x = 0; x < 2; ++x) {
@@ -382,7 +387,7 @@ __global__ void __launch_bounds__(NS == 4 ? 512 : 896, 1) decode2_kernel(const D
                     }
                 }
             }
-            fwht2<NS, LOG2B, true>(P, lane, LOG2B);
+            fwht2<NS, LOG2B, true>(P, lane, a.log2b);
             const f32x2 rn2 = pack2(rn, rn);
 #pragma unroll
             for (int p = 0; p < NS; p += (NS == 4 ? 2 : 1)) {
@@ -397,12 +402,13 @@ __global__ void __launch_bounds__(NS == 4 ? 512 : 896, 1) decode2_kernel(const D
                         __nv_bfloat162 h2 = __floats2bfloat162_rn(y0, y1);
                         w[4 * t + i] = *reinterpret_cast<uint32_t*>(&h2);
                     }
-                if (store_ok[p]) {
-                    if constexpr (NS == 4) {
-                        st_global_256(orow + e_out[p], w);
-                    } else {
-                        *reinterpret_cast<uint4*>(orow + e_out[p]) = make_uint4(w[0], w[1], w[2], w[3]);
-                    }
+                if constexpr (NS == 4 && ALIGNED) {
+                    if (e_out[p] < d_in) st_global_256(orow + e_out[p], w);
+                } else {
+#pragma unroll
+                    for (int t = 0; t < NP; ++t)
+                        if (e_out[p + t] < d_in)
+                            *reinterpret_cast<uint4*>(orow + e_out[p + t]) = make_uint4(w[4 * t], w[4 * t + 1], w[4 * t + 2], w[4 * t + 3]);
                 }
             }
         }
@@ -944,10 +950,11 @@ int raise_smem_limit(const void* kernel) {
 }
 
 template <int NS, int LOG2B>
-int launch_decode2(const Decode2Args& a, int blocks, int threads, size_t smem, cudaStream_t st) {
-    int rc = raise_smem_limit(reinterpret_cast<const void*>(&decode2_kernel<NS, LOG2B>));
+int launch_decode2(const Decode2Args& a, bool fits, int blocks, int threads, size_t smem, cudaStream_t st) {
+    auto kernel = fits ? decode2_kernel<NS, LOG2B, true> : decode2_kernel<NS, LOG2B, false>;
+    int rc = raise_smem_limit(reinterpret_cast<const void*>(kernel));
     if (rc) return rc;
-    return launch_check("decode2_kernel", launch_chained(decode2_kernel<NS, LOG2B>, blocks, threads, smem, st, a));
+    return launch_check("decode2_kernel", launch_chained(kernel, blocks, threads, smem, st, a));
 }
 
 template <bool BF16, int LOG2B, int NS, int MAXT>
@@ -1009,17 +1016,29 @@ int rows_decode(const MatDesc* descs_dev, const MatDesc* descs_host, int n, cons
                 int block, int K, const float* codebook_dev, uint32_t flags, void* stream) {
     constexpr int NS = 4, WE = 256 * NS, kWarps = 16;
     const int log2b = ilog2(block);
-    if (log2b < 5 || n <= 0) return QAMW_ERR_SHAPE;
-    long long max_rows = 0;
+    if (n <= 0) return QAMW_ERR_SHAPE;
+    long long pairs = 0;
+    bool fits = true;
     for (int i = 0; i < n; ++i) {
         const MatDesc& d = descs_host[i];
-        if (d.d_in % 16 || d.d_in > WE * kWarps) return QAMW_ERR_SHAPE;
-        if (!aligned(d.w_hat, 32) || !aligned(d.packed, 16) || d.packed_row_stride % 16) return QAMW_ERR_SHAPE;
+        if (d.d_in % 8 || d.d_in > WE * kWarps) return QAMW_ERR_SHAPE;
+        if (!aligned(d.w_hat, 16) || !aligned(d.packed, 16) || d.packed_row_stride % 4) return QAMW_ERR_SHAPE;
         if (!aligned(d.chan_scale, 16) || !aligned(d.signs, 8) || !aligned(d.sigma, 16)) return QAMW_ERR_SHAPE;
-        const int n_seg = (d.d_in + WE - 1) / WE;
-        max_rows = std::max(max_rows, (long long)(d.d_out + kWarps / n_seg - 1) / (kWarps / n_seg));
+        fits = fits && aligned(d.w_hat, 32) && d.d_in % 16 == 0 && d.packed_row_stride % 16 == 0;
+        pairs += (long long)d.d_out * (d.d_in / 2);
     }
-    if (max_rows == 0) return QAMW_OK;
+    if (pairs == 0) return QAMW_OK;
+    int grid = sm_count();
+    if (flags & QAMW_FLAG_HALF_DEVICE) grid = std::max(1, grid / 2);
+    // A single matrix is spread over all SMs before a block gets a second row, so a small one runs with few warps
+    // per block and few codebook copies.
+    int warps = kWarps, blocks = span_blocks;
+    if (!spans_dev) {
+        const int n_seg = (descs_host[0].d_in + WE - 1) / WE;
+        const int groups = std::max(1, std::min(kWarps / n_seg, (descs_host[0].d_out + grid - 1) / grid));
+        warps = groups * n_seg;
+        blocks = std::max(1, std::min(grid, (descs_host[0].d_out + groups - 1) / groups));
+    }
     Decode2Args a;
     a.descs = descs_dev;
     a.one = descs_host[0];
@@ -1028,23 +1047,22 @@ int rows_decode(const MatDesc* descs_dev, const MatDesc* descs_host, int n, cons
     a.K = K;
     a.log2K = ilog2(K);
     a.seg_bytes = 16 * NS * a.log2K;
-    a.stage_bytes = (a.seg_bytes + 16 + 127) & ~127;  // 128-byte aligned ring buffers
+    a.stage_bytes = (a.seg_bytes + 28 + 127) & ~127;  // 12 bytes before a row off its boundary, 16 read past its end
+    a.log2b = log2b;
     a.inv_sqrt_b = float(1.0 / std::sqrt(double(block)));
-    const size_t stage_total = size_t(kWarps) * kDecodeDepth * a.stage_bytes;
-    a.log2c = pick_copies(K, 1 << 20, std::min(size_t(128) * 1024, kSmemLimit - stage_total));
+    const size_t stage_total = size_t(warps) * kDecodeDepth * a.stage_bytes;
+    a.log2c = pick_copies(K, pairs / 32 / blocks, std::min(size_t(128) * 1024, kSmemLimit - stage_total));
     const size_t smem = (size_t(K) * 8 << a.log2c) + stage_total;
-    int grid = sm_count();
-    if (flags & QAMW_FLAG_HALF_DEVICE) grid = std::max(1, grid / 2);
-    const int blocks = spans_dev ? span_blocks : int(std::max<long long>(1, std::min<long long>(grid, max_rows)));
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     int rc = QAMW_ERR_SHAPE;
-    switch (log2b) {
-        case 5: rc = launch_decode2<NS, 5>(a, blocks, kWarps * 32, smem, st); break;
-        case 6: rc = launch_decode2<NS, 6>(a, blocks, kWarps * 32, smem, st); break;
-        case 7: rc = launch_decode2<NS, 7>(a, blocks, kWarps * 32, smem, st); break;
-        case 8: rc = launch_decode2<NS, 8>(a, blocks, kWarps * 32, smem, st); break;
-        case 9: rc = launch_decode2<NS, 9>(a, blocks, kWarps * 32, smem, st); break;
-        case 10: rc = launch_decode2<NS, 10>(a, blocks, kWarps * 32, smem, st); break;
+    switch (log2b >= 5 ? log2b : 0) {
+        case 0: rc = launch_decode2<NS, 0>(a, fits, blocks, warps * 32, smem, st); break;
+        case 5: rc = launch_decode2<NS, 5>(a, fits, blocks, warps * 32, smem, st); break;
+        case 6: rc = launch_decode2<NS, 6>(a, fits, blocks, warps * 32, smem, st); break;
+        case 7: rc = launch_decode2<NS, 7>(a, fits, blocks, warps * 32, smem, st); break;
+        case 8: rc = launch_decode2<NS, 8>(a, fits, blocks, warps * 32, smem, st); break;
+        case 9: rc = launch_decode2<NS, 9>(a, fits, blocks, warps * 32, smem, st); break;
+        case 10: rc = launch_decode2<NS, 10>(a, fits, blocks, warps * 32, smem, st); break;
         default: break;
     }
     return rc;
@@ -1232,7 +1250,7 @@ struct qamw_batch {
     int n_blocks_dist = 0;
     double* d_dist_partial = nullptr;   // one record of four sums per (block, matrix of its span)
     DistOwner* d_dist_owner = nullptr;  // per matrix: first and last block whose span holds it, first record
-    unsigned int* d_dist_counter = nullptr;  // ticket of the blocks; zero between launches
+    unsigned int* d_dist_counter = nullptr;  // tickets of the blocks, per matrix; zero between launches
     MatDesc* d_cal_all = nullptr;       // calibration descriptors of all block-size classes, for the one finish launch
     int cal_all_n = 0, cal_all_max_pairs = 0;
     RowSet cal[kEncodeClasses];     // calibration: the encoder's sets again, spans over the calibration rows
@@ -1394,8 +1412,8 @@ extern "C" int qamw_batch_create(const qamw_matrix* items, int n, const qamw_cod
         if (e == cudaSuccess) e = cudaMalloc(&b->d_dist_partial, sizeof(double) * 4 * size_t(std::max(1, n_rec)));
         if (e == cudaSuccess) e = cudaMalloc(&b->d_dist_owner, sizeof(DistOwner) * size_t(n));
         if (e == cudaSuccess) e = cudaMemcpy(b->d_dist_owner, owner.data(), sizeof(DistOwner) * size_t(n), cudaMemcpyHostToDevice);
-        if (e == cudaSuccess) e = cudaMalloc(&b->d_dist_counter, sizeof(unsigned int));
-        if (e == cudaSuccess) e = cudaMemset(b->d_dist_counter, 0, sizeof(unsigned int));
+        if (e == cudaSuccess) e = cudaMalloc(&b->d_dist_counter, sizeof(unsigned int) * size_t(n));
+        if (e == cudaSuccess) e = cudaMemset(b->d_dist_counter, 0, sizeof(unsigned int) * size_t(n));
     }
     if (e != cudaSuccess) {
         set_cuda_error("qamw_batch_create", int(e));
@@ -1535,6 +1553,6 @@ extern "C" int qamw_distortion_batch(const qamw_batch* b, void* stream) {
     red.partial = b->d_dist_partial;
     red.owner = b->d_dist_owner;
     red.counter = b->d_dist_counter;
-    return distortion_batch_launch(b->dec.d_descs, b->n, b->d_spans_dist, b->n_blocks_dist, b->w_dtype == QAMW_DTYPE_BF16,
+    return distortion_batch_launch(b->dec.d_descs, b->d_spans_dist, b->n_blocks_dist, b->w_dtype == QAMW_DTYPE_BF16,
                                    red, stream);
 }
