@@ -27,9 +27,12 @@
 #include <chrono>
 #include <cmath>
 #include <cstdint>
+#include <mutex>
 #include <vector>
 
+#include "qamw_device.cuh"
 #include "qamw_internal.h"
+#include "qamw_launch.h"
 
 using namespace qamw;
 
@@ -55,6 +58,8 @@ __device__ __forceinline__ unsigned long long mix64(unsigned long long x) {  // 
 // Unit circular Gaussian samples by Box-Muller from the counter stream of the header: sample i uses
 // the uniforms of counters 2i and 2i+1.
 __global__ void sample_kernel(unsigned long long key, unsigned long long n, double2* out) {
+    chain_release();
+    chain_wait();
     const unsigned long long golden = 0x9E3779B97F4A7C15ULL;
     for (unsigned long long i = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; i < n;
          i += (unsigned long long)gridDim.x * blockDim.x) {
@@ -83,6 +88,8 @@ struct TrainState {
 
 // Root mean square coordinate of the first samples.  It only decides how well the tiles are packed.
 __global__ void __launch_bounds__(1024) scale_kernel(const double2* samples, unsigned long long n, float* scale) {
+    chain_release();
+    chain_wait();
     __shared__ float part[32];
     float s = 0.f;
     const int m = int(min(n, 4096ull));
@@ -107,6 +114,8 @@ __global__ void __launch_bounds__(1024) scale_kernel(const double2* samples, uns
 // others together (1128 candidates for the worst of 4096 tiles of 256 samples, K = 2048); with cells of equal mass the
 // central tiles get too wide (18 candidates on average); this is between the two (10 on average, at most 335).
 __global__ void hilbert_kernel(const double2* samples, unsigned long long n, const float* scale, int* key) {
+    chain_release();
+    chain_wait();
     const float e = *scale, inv = e > 0.f ? 1.f / (1.4f * e) : 0.f;
     for (unsigned long long i = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; i < n;
          i += (unsigned long long)gridDim.x * blockDim.x) {
@@ -149,6 +158,8 @@ __device__ __forceinline__ TileBox make_box(double x0, double x1, double y0, dou
     return b;
 }
 __global__ void __launch_bounds__(kTile) box_kernel(const double2* sorted, unsigned long long n, TileBox* boxes) {
+    chain_release();
+    chain_wait();
     __shared__ double lo[2][kTileWarps], hi[2][kTileWarps];
     __shared__ int any_bad;
     if (threadIdx.x == 0) any_bad = 0;
@@ -209,6 +220,8 @@ __global__ void __launch_bounds__(kTile, 3) assign_kernel(const double2* sorted,
                                                        const TileBox* boxes, const double2* codebook,
                                                        const float2* codebook32, int K, int* assign, double* tile_err,
                                                        const TrainState* state) {
+    chain_release();
+    chain_wait();
     __shared__ unsigned short list[QAMW_MAX_K];
     __shared__ double2 cand[kTile];
     __shared__ float2 cand32[kTile];
@@ -322,6 +335,8 @@ struct KeyOf {
 __global__ void __launch_bounds__(512) hist_kernel(KeyOf key, unsigned long long n, int chunk, int bins, int* hist,
                                                    const double* tile_err, int n_tiles, double rel_tol, int max_iters,
                                                    TrainState* state) {
+    chain_release();
+    chain_wait();
     extern __shared__ int h[];
     __shared__ double err_part[16];
     if (tile_err && state->done) return;
@@ -381,6 +396,8 @@ __device__ __forceinline__ int block_scan(int v, int* warp_part, int& total) {
 // histogram) by 32 runs of chunks (warps) per block.  The block that finishes last turns the bins'
 // totals into start positions.
 __global__ void __launch_bounds__(1024) prefix_kernel(int* hist, int n_chunks, int bins, int* start, TrainState* state) {
+    chain_release();
+    chain_wait();
     __shared__ int run_sum[32][33];
     __shared__ int warp_part[32];
     __shared__ bool last;
@@ -437,6 +454,8 @@ __global__ void __launch_bounds__(1024) prefix_kernel(int* hist, int n_chunks, i
 __global__ void __launch_bounds__(32 * kSortWarps) scatter_kernel(KeyOf key, unsigned long long n, int chunk, int bins,
                                                                   const int* hist, const int* start, const double2* samples,
                                                                   int* ids_out, double2* z_out, const TrainState* state) {
+    chain_release();
+    chain_wait();
     extern __shared__ int cursor[];  // [bins], then 16-bit counters [warp][bins + 1 rounded up to an even number]
     if (state && state->done) return;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -531,6 +550,8 @@ constexpr int kCellWarps = 4;
 __global__ void __launch_bounds__(32 * kCellWarps) centroid_kernel(const double2* by_cell, const int* start, int K,
                                                                    double2* codebook, float2* codebook32,
                                                                    const TrainState* state) {
+    chain_release();
+    chain_wait();
     __shared__ __align__(16) double stage[kCellWarps][2][64];
     if (state->done) return;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, c = blockIdx.x * kCellWarps + warp;
@@ -583,6 +604,8 @@ __global__ void __launch_bounds__(32 * kCellWarps) centroid_kernel(const double2
 
 // Initial codewords sqrt(2) * sample_i, and the f32 copy of the codebook that the filter reads.
 __global__ void init_kernel(const double2* samples, int K, double2* codebook, float2* codebook32, TrainState* state) {
+    chain_release();
+    chain_wait();
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c == 0) *state = TrainState{};
     if (c >= K) return;
@@ -590,6 +613,33 @@ __global__ void init_kernel(const double2* samples, int K, double2* codebook, fl
     const double2 z = samples[c];
     codebook[c] = make_double2(root2 * z.x, root2 * z.y);
     codebook32[c] = make_float2(float(root2 * z.x), float(root2 * z.y));
+}
+
+// Where the scratch memory of a call comes from: a pool per device that keeps up to 256 MB between calls (the
+// default size takes 60 MB; with cudaMalloc and cudaFree a call cost 3 ms more) and gives it back to the driver
+// when another allocation of the process needs it.  NULL if the device has no pools of its own.
+constexpr int kMaxDevices = 64;
+cudaMemPool_t scratch_pool() {
+    static std::mutex mu;
+    static cudaMemPool_t pools[kMaxDevices] = {};
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev >= kMaxDevices) return nullptr;
+    std::lock_guard<std::mutex> lock(mu);
+    if (!pools[dev]) {
+        cudaMemPoolProps props{};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = dev;
+        cudaMemPool_t p = nullptr;
+        if (cudaMemPoolCreate(&p, &props) != cudaSuccess) {
+            cudaGetLastError();
+            return nullptr;
+        }
+        uint64_t keep = 256ull << 20;
+        cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep);
+        pools[dev] = p;
+    }
+    return pools[dev];
 }
 
 }  // namespace
@@ -618,14 +668,19 @@ extern "C" int qamw_train_codebook_gpu(int K, uint64_t n_samples, uint64_t seed,
                  o_cb = piece(sizeof(double2) * K), o_cb32 = piece(sizeof(float2) * K), o_err = piece(sizeof(double) * n_tiles),
                  o_box = piece(sizeof(TileBox) * n_tiles * kBoxes), o_state = piece(sizeof(TrainState)), o_scale = piece(sizeof(float));
     unsigned char* base = nullptr;
-    cudaError_t e = cudaMalloc(&base, bytes);
+    cudaError_t e = cudaSuccess;
+    if (cudaMemPool_t pool = scratch_pool()) {
+        e = cudaMallocFromPoolAsync(reinterpret_cast<void**>(&base), bytes, pool, nullptr);
+    } else {
+        e = cudaMallocAsync(reinterpret_cast<void**>(&base), bytes, nullptr);
+    }
     if (e != cudaSuccess) {
-        set_cuda_error("qamw_train_codebook_gpu: cudaMalloc", int(e));
+        set_cuda_error("qamw_train_codebook_gpu: cudaMallocAsync", int(e));
         return QAMW_ERR_CUDA;
     }
     struct Free {
         void* p;
-        ~Free() { cudaFree(p); }
+        ~Free() { cudaFreeAsync(p, nullptr); }
     } owner{base};
     auto ok = [&](cudaError_t r) {
         if (e == cudaSuccess) e = r;
@@ -650,29 +705,29 @@ extern "C" int qamw_train_codebook_gpu(int K, uint64_t n_samples, uint64_t seed,
         key ^= key >> 27;
         key *= 0x94D049BB133111EBULL;
         key ^= key >> 31;
-        sample_kernel<<<8 * sm_count(), 256>>>(key, n, generated);
+        ok(launch_chained(sample_kernel, 8 * sm_count(), 256, 0, nullptr, key, n, generated));
     }
     auto sort_smem = [](int b) { return sizeof(int) * size_t(b) + size_t(kSortWarps) * size_t((b + 1) & ~1) * 2; };
     if (sort_smem(bins) > 48 * 1024)  // beyond the default dynamic limit
         ok(cudaFuncSetAttribute(scatter_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sort_smem(bins))));
-    init_kernel<<<(K + 255) / 256, 256>>>(samples, K, d_cb, d_cb32, state);
+    ok(launch_chained(init_kernel, (K + 255) / 256, 256, 0, nullptr, samples, K, d_cb, d_cb32, state));
 
     // spatial order: two stable passes over the Hilbert position's bytes (the cells' buffers are free so far)
     int *pos = assign, *half = reinterpret_cast<int*>(by_cell);
-    scale_kernel<<<1, 1024>>>(samples, n, scale);
-    hilbert_kernel<<<8 * sm_count(), 256>>>(samples, n, scale, pos);
+    ok(launch_chained(scale_kernel, 1, 1024, 0, nullptr, samples, n, scale));
+    ok(launch_chained(hilbert_kernel, 8 * sm_count(), 256, 0, nullptr, samples, n, scale, pos));
     for (int pass = 0; pass < 2; ++pass) {
         const KeyOf key{pos, pass ? half : nullptr, 8 * pass, 255};
-        hist_kernel<<<n_chunks, 512, sizeof(int) * 256>>>(key, n, chunk, 256, hist, nullptr, 0, 0.0, 0, state);
-        prefix_kernel<<<8, 1024>>>(hist, n_chunks, 256, start, state);
-        scatter_kernel<<<n_chunks, 32 * kSortWarps, sort_smem(256)>>>(key, n, chunk, 256, hist, start, samples, pass ? ids : half,
-                                                            pass ? sorted : nullptr, nullptr);
+        ok(launch_chained(hist_kernel, n_chunks, 512, sizeof(int) * 256, nullptr, key, n, chunk, 256, hist, nullptr, 0, 0.0, 0, state));
+        ok(launch_chained(prefix_kernel, 8, 1024, 0, nullptr, hist, n_chunks, 256, start, state));
+        ok(launch_chained(scatter_kernel, n_chunks, 32 * kSortWarps, sort_smem(256), nullptr, key, n, chunk, 256, hist, start, samples, pass ? ids : half,
+                                                            pass ? sorted : nullptr, nullptr));
     }
-    box_kernel<<<n_tiles, kTile>>>(sorted, n, boxes);
+    ok(launch_chained(box_kernel, n_tiles, kTile, 0, nullptr, sorted, n, boxes));
 
     auto assign_pass = [&](int* to, const TrainState* st) {
         auto go = [&](auto kernel) {
-            kernel<<<n_tiles, kTile>>>(sorted, ids, n, boxes, d_cb, d_cb32, K, to, tile_err, st);
+            ok(launch_chained(kernel, n_tiles, kTile, 0, nullptr, sorted, ids, n, boxes, d_cb, d_cb32, K, to, tile_err, st));
         };
         switch (K / kTile) {
             case 8: go(assign_kernel<8>); break;
@@ -687,11 +742,11 @@ extern "C" int qamw_train_codebook_gpu(int K, uint64_t n_samples, uint64_t seed,
     while (ok(cudaGetLastError())) {
         for (int k = 0; k < kBatch && recorded + k <= max_iters; ++k) {
             assign_pass(assign, state);
-            hist_kernel<<<n_chunks + 1, 512, sizeof(int) * K>>>(cell, n, chunk, K, hist, tile_err, n_tiles, rel_tol, max_iters,
-                                                                 state);
-            prefix_kernel<<<(K + 31) / 32, 1024>>>(hist, n_chunks, K, start, state);
-            scatter_kernel<<<n_chunks, 32 * kSortWarps, sort_smem(K)>>>(cell, n, chunk, K, hist, start, samples, nullptr, by_cell, state);
-            centroid_kernel<<<(K + kCellWarps - 1) / kCellWarps, 32 * kCellWarps>>>(by_cell, start, K, d_cb, d_cb32, state);
+            ok(launch_chained(hist_kernel, n_chunks + 1, 512, sizeof(int) * K, nullptr, cell, n, chunk, K, hist, tile_err, n_tiles, rel_tol, max_iters,
+                                                                 state));
+            ok(launch_chained(prefix_kernel, (K + 31) / 32, 1024, 0, nullptr, hist, n_chunks, K, start, state));
+            ok(launch_chained(scatter_kernel, n_chunks, 32 * kSortWarps, sort_smem(K), nullptr, cell, n, chunk, K, hist, start, samples, nullptr, by_cell, state));
+            ok(launch_chained(centroid_kernel, (K + kCellWarps - 1) / kCellWarps, 32 * kCellWarps, 0, nullptr, by_cell, start, K, d_cb, d_cb32, state));
         }
         if (!ok(cudaMemcpy(&seen, state, sizeof(seen), cudaMemcpyDeviceToHost))) break;
         for (; recorded < seen.passes; ++recorded)
