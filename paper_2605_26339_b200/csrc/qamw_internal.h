@@ -75,8 +75,8 @@ bool pack_search_table(const CellLists& cl, SearchTable* out);
 // K), shrunk until the table fits in budget_bytes.
 bool choose_search_table(const float* codebook, int K, int grid, size_t budget_bytes, SearchTable* out, int first = 0);
 // The records as the kernels read them (SearchSmem in qamw_device.cuh), for codebook entries of 2^log2_entry bytes:
-// grid * grid * 2 words, then the overflow lists.  False if the lists do not fit their fields.
-bool pack_device_table(const SearchTable& t, int K, int log2_entry, std::vector<uint32_t>* words, std::vector<uint16_t>* lists);
+// grid * grid * 2 words, and the list words.  False if the lists do not fit their fields.
+bool pack_device_table(const SearchTable& t, int K, int log2_entry, std::vector<uint32_t>* words, std::vector<uint32_t>* lists);
 
 void set_cuda_error(const char* what, int code);
 void set_error_text(const char* text);

@@ -587,7 +587,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1) encode_kernel(const EncodeArgs
                     if (cell_overflows(word1[0] | word1[1] | word1[2] | word1[3])) {
 #pragma unroll
                         for (int p = 0; p < 4; ++p)
-                            if (cell_overflows(word1[p])) v[p] = search_overflow(s, word1[p], v[p], z[p].x, z[p].y);
+                            if (cell_overflows(word1[p])) v[p] = search_overflow<true>(s, word1[p], first_list_word(s, word1[p]), v[p], z[p].x, z[p].y);
                     }
 #pragma unroll
                     for (int p = 0; p < 4; ++p) v[p] >>= s.log2_entry;
@@ -1395,8 +1395,7 @@ extern "C" int qamw_codebook_create(const float* codebook_host, int K, int grid,
     const size_t budget = kSmemLimit - kEncodeStaticSmem - (size_t(K) * 8 << log2c);
     const int first = 2 * std::max(15, std::min(int(1.55 * std::sqrt(double(K))), 127)) + 1;
     if (!choose_search_table(codebook_host, K, grid, budget, &t, first)) return QAMW_ERR_NOMEM;
-    std::vector<uint32_t> words;
-    std::vector<uint16_t> lists;
+    std::vector<uint32_t> words, lists;
     if (!pack_device_table(t, K, 3 + log2c, &words, &lists)) return QAMW_ERR_NOMEM;
     qamw_codebook* cb = new (std::nothrow) qamw_codebook();
     if (!cb) return QAMW_ERR_NOMEM;
@@ -1408,12 +1407,12 @@ extern "C" int qamw_codebook_create(const float* codebook_host, int K, int grid,
     cb->h_codebook.assign(codebook_host, codebook_host + 2 * K);
     cb->off_cells = size_t(K) * 8;
     cb->off_overflow = cb->off_cells + words.size() * 4;
-    cb->blob_bytes = cb->off_overflow + lists.size() * 2;
+    cb->blob_bytes = cb->off_overflow + lists.size() * 4;
     cb->log2c = log2c;
     std::vector<unsigned char> blob(cb->blob_bytes, 0);
     std::memcpy(blob.data(), codebook_host, size_t(K) * 8);
     std::memcpy(blob.data() + cb->off_cells, words.data(), words.size() * 4);
-    std::memcpy(blob.data() + cb->off_overflow, lists.data(), lists.size() * 2);
+    std::memcpy(blob.data() + cb->off_overflow, lists.data(), lists.size() * 4);
     cudaError_t e = cudaGetDevice(&cb->device);
     if (e == cudaSuccess) e = cudaMalloc(&cb->d_blob, cb->blob_bytes);
     if (e == cudaSuccess) e = cudaMemcpy(cb->d_blob, blob.data(), cb->blob_bytes, cudaMemcpyHostToDevice);

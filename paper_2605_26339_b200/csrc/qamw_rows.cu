@@ -818,7 +818,7 @@ __global__ void __launch_bounds__(MAXT, 1) encode2_kernel(const Encode2Args a) {
                                 if (careful && !(fmaxf(fabsf(z[i].x), fabsf(z[i].y)) < a.reach))
                                     v[i] = search_exhaustive(s, z[i].x, z[i].y);
                                 else if (cell_overflows(word1[i]))
-                                    v[i] = search_overflow(s, word1[i], v[i], z[i].x, z[i].y);
+                                    v[i] = search_overflow<false>(s, word1[i], first_list_word(s, word1[i]), v[i], z[i].x, z[i].y);
                             }
                         }
 #pragma unroll

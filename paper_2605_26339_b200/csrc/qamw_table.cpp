@@ -272,14 +272,12 @@ bool pack_search_table(const CellLists& cl, SearchTable* out) {
     return true;
 }
 
-bool pack_device_table(const SearchTable& t, int K, int log2_entry, std::vector<uint32_t>* words, std::vector<uint16_t>* lists) {
+bool pack_device_table(const SearchTable& t, int K, int log2_entry, std::vector<uint32_t>* words, std::vector<uint32_t>* lists) {
     const int B = ilog2(K), list_shift = log2_entry + B;
     const size_t n_cells = t.cells.size() / 4;
     words->assign(2 * n_cells, 0);
     lists->clear();
-    std::vector<uint16_t> entries;
     auto word = [&](uint32_t lo, uint32_t hi) { return (lo << log2_entry) | (hi << (32 - B)); };
-    const size_t base = size_t(t.n_overflow_cells) + 1;  // the lists come after their starts
     for (size_t c = 0; c < n_cells; ++c) {
         const uint16_t* rec = &t.cells[4 * c];
         uint32_t* w = &(*words)[2 * c];
@@ -289,16 +287,13 @@ bool pack_device_table(const SearchTable& t, int K, int log2_entry, std::vector<
             continue;
         }
         const uint16_t* list = &t.overflow[rec[1]];
-        if ((lists->size() >> (32 - list_shift)) != 0 || base + entries.size() > 0xFFFF) return false;
+        const int n = rec[2];
+        if ((lists->size() >> (32 - list_shift)) != 0) return false;
         w[0] = word(list[0], list[1]);
         w[1] = (uint32_t(list[2]) << log2_entry) | (uint32_t(lists->size()) << list_shift) | 1u;
-        lists->push_back(uint16_t(base + entries.size()));
-        entries.insert(entries.end(), list + 3, list + rec[2]);
+        for (int i = 3; i < n; i += 2) lists->push_back(word(list[i], list[std::min(i + 1, n - 1)]) | (i + 2 < n ? 1u : 0u));
     }
-    if (base + entries.size() > 0xFFFF) return false;
-    lists->push_back(uint16_t(base + entries.size()));
-    lists->insert(lists->end(), entries.begin(), entries.end());
-    while ((words->size() * 4 + lists->size() * 2) % 16) lists->push_back(0);  // copied in 16-byte pieces
+    while ((words->size() + lists->size()) % 4) lists->push_back(0);  // copied in 16-byte pieces
     return true;
 }
 
