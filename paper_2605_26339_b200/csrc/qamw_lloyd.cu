@@ -4,7 +4,7 @@
 // ties) and a centroid pass in which every cell's samples are added in sample order, so the sums are bit
 // for bit those of a sequential loop over the samples and training gives the same codebook run after run.
 //
-// Assignment.  Once per call the samples are put in the order of a Hilbert curve, so that 512
+// Assignment.  Once per call the samples are put in the order of a Hilbert curve, so that 256
 // consecutive ones (a tile, one block) lie in a small box.  Per iteration a block finds the codewords that
 // can be nearest to some point of its box -- those whose smallest distance to the box does not exceed the
 // smallest of all largest distances -- and each of its warps narrows the list again with the box of its own 32
@@ -39,7 +39,7 @@ using namespace qamw;
 namespace {
 
 constexpr unsigned kFullMask = 0xffffffffu;
-constexpr int kTile = 512;           // samples per tile, threads of its block
+constexpr int kTile = 256;           // samples per tile, threads of its block
 constexpr int kSortWarps = 16;       // warps that sort a chunk
 constexpr int kMinChunk = 4096;      // samples per sorting chunk; more when there would be more than this
 constexpr int kManyChunks = 1024;    // many chunks,
@@ -213,10 +213,12 @@ constexpr float kTiny = 1e-36f;  // squares down there are no longer relatively 
 // Exact nearest codeword of the samples of a tile: d = dx*dx + dy*dy with one rounding per
 // operation (no fused multiply-add: the result must not depend on how a compiler contracts the
 // expression), the lowest index among equal distances.  Also adds up the distances of the tile in a fixed
-// order (a shuffle tree, then by warp).  Bound by the f32 filter over all codewords (K / 512 per thread) and
+// order (a shuffle tree, then by warp).  Bound by the f32 filter over all codewords (K / 256 per thread) and
+// the waits between its four steps, which is why the SM is filled with small blocks (eight of 256 threads; three of
+// 512: 9.06 against 8.93 ms a call at K = 2048, 12.3 against 9.8 at K = 512), then by
 // the double comparisons with those that remain; both arrays come from L1/L2.
 template <int PER>  // codewords per thread: K / kTile, or 1 for a smaller codebook
-__global__ void __launch_bounds__(kTile, 3) assign_kernel(const double2* sorted, const int* ids, unsigned long long n,
+__global__ void __launch_bounds__(kTile, 8) assign_kernel(const double2* sorted, const int* ids, unsigned long long n,
                                                        const TileBox* boxes, const double2* codebook,
                                                        const float2* codebook32, int K, int* assign, double* tile_err,
                                                        const TrainState* state) {
@@ -730,6 +732,7 @@ extern "C" int qamw_train_codebook_gpu(int K, uint64_t n_samples, uint64_t seed,
             ok(launch_chained(kernel, n_tiles, kTile, 0, nullptr, sorted, ids, n, boxes, d_cb, d_cb32, K, to, tile_err, st));
         };
         switch (K / kTile) {
+            case 16: go(assign_kernel<16>); break;
             case 8: go(assign_kernel<8>); break;
             case 4: go(assign_kernel<4>); break;
             case 2: go(assign_kernel<2>); break;
