@@ -869,7 +869,9 @@ __global__ void __launch_bounds__(MAXT, 1) encode2_kernel(const Encode2Args a) {
 
 // sigma_k of every matrix from the slots of partial sums, one per block that the matrix was spread over.  A block
 // owns 32 pair positions of one matrix; its eight warps each add a contiguous slice of the slots in ascending
-// order, and the eight slice sums are then added in ascending order: the result does not depend on timing.
+// order, and the slice sums are then added in ascending order: the result does not depend on timing.  Bound by the
+// latency of its loads: with a slot per SM, the 19 of a slice come in two
+// steps.  (Sixteen slices: 1 us less for one matrix, 2 to 10 us more for the batches, whose slots are few.)
 constexpr int kFinishSlices = 8;
 __global__ void __launch_bounds__(32 * kFinishSlices) calibrate_finish2_kernel(const MatDesc* descs, const MatDesc one,
                                                                              const unsigned char* calib_base) {
@@ -887,15 +889,14 @@ __global__ void __launch_bounds__(32 * kFinishSlices) calibrate_finish2_kernel(c
     double sum = 0.0, used = 0.0;
     for (int slot = s0 + lane; slot < s1; slot += 32) used += ws[size_t(d.calib_slots) * pair_stride + slot];  // whole numbers: any order
     if (k < n_pairs) {
-        int slot = s0;
-        for (; slot + 8 <= s1; slot += 8) {
-            double v[8];
+        constexpr int U = 10;
+        for (int slot = s0; slot < s1; slot += U) {
+            double v[U];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) v[u] = ws[size_t(slot + u) * pair_stride + k];
+            for (int u = 0; u < U; ++u) v[u] = slot + u < s1 ? ws[size_t(slot + u) * pair_stride + k] : 0.0;
 #pragma unroll
-            for (int u = 0; u < 8; ++u) sum += v[u];
+            for (int u = 0; u < U; ++u) sum += v[u];
         }
-        for (; slot < s1; ++slot) sum += ws[size_t(slot) * pair_stride + k];
     }
     used = warp_total(used);
     part_sum[slice][lane] = sum;
