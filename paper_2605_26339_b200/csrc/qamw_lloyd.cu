@@ -20,7 +20,7 @@
 // after the last wanted update return at once, and the host reads the errors once per batch.
 //
 // K = 2048 on 2^20 samples, 100 updates on a B200: 235 ms with the exhaustive scan, a serial scan of the histograms
-// and one host round trip per update; 10.1 ms now.
+// and one host round trip per update; 8.9 ms now.
 #include <cuda_runtime.h>
 
 #include <algorithm>

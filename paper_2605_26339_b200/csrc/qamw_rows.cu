@@ -557,8 +557,10 @@ __device__ __forceinline__ void store_indices(const uint2 (&u)[NS], const uint32
 // row's warps -- a named barrier for the norm -- searches its pairs and writes its 16 NS B bytes of the packed
 // row.  W is read once.
 //
-// Bound by the shared-memory pipe: of 26 wavefronts per 32 points a cell record (8 random bytes) takes 5.6, the candidate
-// codewords 14 (4 per read from eight copies; the fourth candidate only where there is one), rotation shuffles 3.
+// Bound by the shared-memory pipe and by issue slots, both at 60 %, with too few warps to hide what depends on what: 27.5
+// wavefronts per 32 points (a cell record, 8 random bytes, takes 5.6, the candidate codewords 14: 4 per read from
+// eight copies, the fourth only where there is one; rotation shuffles 3) and 117 instructions.  Four layers of 13B,
+// K = 2048: 4.01 ms with 33.7 wavefronts per 32 points, 3.14 ms now.
 // QUANT: 0 = nearest codeword through the cell table, 1 = polar quantiser, 2 = no quantiser at all:
 // the kernel then is the calibration pass of Section 3.4, which visits n = min(d_out, 1024) rows
 // floor(t d_out / n) and adds up the pair moduli |(y_2k, y_2k+1)| per pair position.  The row groups of a
@@ -1387,8 +1389,8 @@ extern "C" int qamw_batch_create(const qamw_matrix* items, int n, const qamw_cod
     }
     // Distortion: equal numbers of work items per block.  Five blocks fit an SM; with up to 32 items for each of them one
     // wave is best (a 1.1B layer 45.8 -> 40.2 us, in f32 75 -> 60: a block of one item only fills and drains its ring),
-    // beyond that two waves even out what the blocks lose to each other (four layers of 13B: 890 us with 5, 861 with 10,
-    // 874 with 16 per SM).
+    // beyond that sixteen per SM even out what the blocks lose to each other (four layers of 13B: 890 us with 5, 861 with
+    // 10, 874 with 16; forty layers: 8.20 ms with 10, 7.98 with 16).
     if (e == cudaSuccess) {
         std::vector<MatDesc> items_as_rows(b->dec.descs);
         std::vector<int> unit(size_t(n), 1);
@@ -1398,7 +1400,7 @@ extern "C" int qamw_batch_create(const qamw_matrix* items, int n, const qamw_cod
             total += items_as_rows[size_t(i)].d_out;
         }
         const long long wave = 5LL * b->n_blocks;
-        b->n_blocks_dist = int(std::max<long long>(1, std::min<long long>(total < 32 * wave ? wave : 2 * wave, total)));
+        b->n_blocks_dist = int(std::max<long long>(1, std::min<long long>(total < 32 * wave ? wave : 16LL * b->n_blocks, total)));
         std::vector<int4> spans;
         make_spans(items_as_rows.data(), n, b->n_blocks_dist, unit.data(), &spans);
         e = cudaMalloc(&b->d_spans_dist, sizeof(int4) * spans.size());
