@@ -97,7 +97,7 @@ __global__ void __launch_bounds__(512, 1) gemv_kernel(const GemvArgs a) {
             const uint32_t sh = bit0 & 31u;
             uint32_t word[8];
 #pragma unroll
-            for (int i = 0; i < 8; ++i) word[i] = (i <= words_per_chunk + 1 && w0 + i < row_words) ? __ldg(w + w0 + i) : 0u;
+            for (int i = 0; i < 8; ++i) word[i] = (i <= words_per_chunk + 1 && w0 + i < row_words) ? w[w0 + i] : 0u;
             // shift the window down to bit 0, then cut two indices per step of 2 B bits
             uint32_t win[7];
 #pragma unroll
@@ -121,7 +121,7 @@ __global__ void __launch_bounds__(512, 1) gemv_kernel(const GemvArgs a) {
                 }
             }
         }
-        const float rn = __ldg(a.row_norm + row);
+        const float rn = a.row_norm[row];
 #pragma unroll
         for (int v = 0; v < NVEC; ++v) {
             float s = acc[v];
@@ -209,44 +209,51 @@ __device__ __forceinline__ float warp_sums(float (&v)[N], int lane) {
 template <int NVEC>
 __device__ __forceinline__ void rotate_slice(const Gemv2Args& a, int slice, int v0, unsigned char* stage, int lane, f32x2 (&xr)[NVEC][16]) {
     const int col0 = 1024 * slice, chunk = 32 * slice + lane;
+    // the loads of a vector before the first store to `stage`, which the compiler must take for a store to `x`
+    float4 q[8];
+    auto fetch = [&](int v) {
+        const float* x = a.x + size_t(v0 + v) * a.d_in;
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            const int col = col0 + 128 * e + 4 * lane;
+            q[e] = col < a.d_in ? *reinterpret_cast<const float4*>(x + col) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+    };
+    fetch(0);
+    float4 sg4[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+        sg4[e] = chunk < a.n_chunks ? reinterpret_cast<const float4*>(a.sigma + 16 * chunk)[e] : make_float4(0.f, 0.f, 0.f, 0.f);
     float tj[32];  // sign_j / s_j of columns col0 + 128 e + 4 lane + i
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
         const int col = col0 + 128 * e + 4 * lane;
         const bool in = col < a.d_in;
-        const uint32_t sw = in ? __ldg(reinterpret_cast<const uint32_t*>(a.signs + col)) : 0u;
-        float4 q = make_float4(1.f, 1.f, 1.f, 1.f);
-        if (in && a.chan_scale) q = __ldg(reinterpret_cast<const float4*>(a.chan_scale + col));
-        tj[4 * e] = __fdividef(float(int(int8_t(sw & 0xffu))), q.x);
-        tj[4 * e + 1] = __fdividef(float(int(int8_t((sw >> 8) & 0xffu))), q.y);
-        tj[4 * e + 2] = __fdividef(float(int(int8_t((sw >> 16) & 0xffu))), q.z);
-        tj[4 * e + 3] = __fdividef(float(int(int8_t(sw >> 24))), q.w);
+        const uint32_t sw = in ? *reinterpret_cast<const uint32_t*>(a.signs + col) : 0u;
+        float4 s = make_float4(1.f, 1.f, 1.f, 1.f);
+        if (in && a.chan_scale) s = *reinterpret_cast<const float4*>(a.chan_scale + col);
+        tj[4 * e] = __fdividef(float(int(int8_t(sw & 0xffu))), s.x);
+        tj[4 * e + 1] = __fdividef(float(int(int8_t((sw >> 8) & 0xffu))), s.y);
+        tj[4 * e + 2] = __fdividef(float(int(int8_t((sw >> 16) & 0xffu))), s.z);
+        tj[4 * e + 3] = __fdividef(float(int(int8_t(sw >> 24))), s.w);
     }
-    float4 sg4[4];
-#pragma unroll
-    for (int e = 0; e < 4; ++e)
-        sg4[e] = chunk < a.n_chunks ? __ldg(reinterpret_cast<const float4*>(a.sigma + 16 * chunk) + e) : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
     for (int v = 0; v < NVEC; ++v) {
-        const float* x = a.x + size_t(v0 + v) * a.d_in;
         __syncwarp();  // the staging memory is free
 #pragma unroll
-        for (int e = 0; e < 8; ++e) {
-            const int col = col0 + 128 * e + 4 * lane;
-            float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (col < a.d_in) q = __ldg(reinterpret_cast<const float4*>(x + col));
+        for (int e = 0; e < 8; ++e)
             *reinterpret_cast<float4*>(stage + (4 * e + (lane >> 3)) * 144 + (lane & 7) * 16) =
-                make_float4(q.x * tj[4 * e], q.y * tj[4 * e + 1], q.z * tj[4 * e + 2], q.w * tj[4 * e + 3]);
-        }
+                make_float4(q[e].x * tj[4 * e], q[e].y * tj[4 * e + 1], q[e].z * tj[4 * e + 2], q[e].w * tj[4 * e + 3]);
+        if (v + 1 < NVEC) fetch(v + 1);
         __syncwarp();
         float t[32];
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
-            const float4 q = *reinterpret_cast<const float4*>(stage + lane * 144 + 16 * e);
-            t[4 * e] = q.x;
-            t[4 * e + 1] = q.y;
-            t[4 * e + 2] = q.z;
-            t[4 * e + 3] = q.w;
+            const float4 u = *reinterpret_cast<const float4*>(stage + lane * 144 + 16 * e);
+            t[4 * e] = u.x;
+            t[4 * e + 1] = u.y;
+            t[4 * e + 2] = u.z;
+            t[4 * e + 3] = u.w;
         }
 #pragma unroll
         for (int st = 0; st < 5; ++st) {  // butterflies inside the lane's 32 columns
@@ -452,15 +459,19 @@ __global__ void __launch_bounds__(GemvGeom<NVEC>::kThreads, 1) gemv2_kernel(cons
                     if (it + r < n_rows) ps[(s0 * TI + (jj + r) * G + g) * NVEC + v] = total;
                 }
             }
+            // the norm of this thread's first row travels while the block's warps meet
+            const int i0 = tile * TI + int(threadIdx.x) / NVEC;
+            float rn = i0 < n_b ? a.row_norm[(long long)blockIdx.x + (long long)gridDim.x * i0] : 0.f;
             __syncthreads();  // the tile's partial sums are complete
             for (int idx = threadIdx.x; idx < TI * NVEC; idx += blockDim.x) {
                 const int il = idx / NVEC, v = idx - il * NVEC;
                 const int i = tile * TI + il;
                 if (i >= n_b) continue;
                 const long long row = (long long)blockIdx.x + (long long)gridDim.x * i;
+                if (idx >= int(blockDim.x)) rn = a.row_norm[row];
                 float sum = 0.f;
                 for (int sl = 0; sl < n_live; ++sl) sum += ps[(sl * TI + il) * NVEC + v];
-                sum *= __ldg(a.row_norm + row);
+                sum *= rn;
                 if (pass == 0) a.y[row * NVEC + v] = sum;
                 else a.y[row * NVEC + v] += sum;
             }

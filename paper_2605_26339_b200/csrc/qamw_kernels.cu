@@ -252,10 +252,10 @@ __device__ __forceinline__ void load_row(RawRow<BF16>& raw, const void* W, long 
             if (e0 < g.d_in) {
                 const uint4* p = reinterpret_cast<const uint4*>(base + size_t(e0) * (BF16 ? 2 : 4));
                 if (BF16) {
-                    raw.v[r] = __ldg(p);
+                    raw.v[r] = *p;
                 } else {
-                    raw.v[2 * r] = __ldg(p);
-                    raw.v[2 * r + 1] = __ldg(p + 1);
+                    raw.v[2 * r] = p[0];
+                    raw.v[2 * r + 1] = p[1];
                 }
             } else {
                 if (BF16) {
@@ -457,7 +457,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1) encode_kernel(const EncodeArgs
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
                 const int i = base + u * blockDim.x + threadIdx.x;
-                if (i < n16) v[u] = __ldg(a.table + i);
+                if (i < n16) v[u] = load_blob(a.table + i);
             }
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
@@ -986,7 +986,7 @@ __device__ __forceinline__ void dist_load(const void* W, long long w_row_stride,
     const char* wrow = static_cast<const char*>(W) + (long long)row * w_row_stride * (BF16 ? 2 : 4);
     const __nv_bfloat16* hrow = What + (long long)row * d_in;
     if (vec) {
-        const uint4 hv = __ldg(reinterpret_cast<const uint4*>(hrow + j0));
+        const uint4 hv = *reinterpret_cast<const uint4*>(hrow + j0);
         const uint32_t hw[4] = {hv.x, hv.y, hv.z, hv.w};
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
@@ -994,7 +994,7 @@ __device__ __forceinline__ void dist_load(const void* W, long long w_row_stride,
             h[2 * i + 1] = __uint_as_float(hw[i] & 0xffff0000u);
         }
         if (BF16) {
-            const uint4 wv = __ldg(reinterpret_cast<const uint4*>(reinterpret_cast<const __nv_bfloat16*>(wrow) + j0));
+            const uint4 wv = *reinterpret_cast<const uint4*>(reinterpret_cast<const __nv_bfloat16*>(wrow) + j0);
             const uint32_t ww[4] = {wv.x, wv.y, wv.z, wv.w};
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
@@ -1003,7 +1003,7 @@ __device__ __forceinline__ void dist_load(const void* W, long long w_row_stride,
             }
         } else {
             const float4* p = reinterpret_cast<const float4*>(reinterpret_cast<const float*>(wrow) + j0);
-            const float4 a = __ldg(p), c = __ldg(p + 1);
+            const float4 a = p[0], c = p[1];
             w[0] = a.x; w[1] = a.y; w[2] = a.z; w[3] = a.w;
             w[4] = c.x; w[5] = c.y; w[6] = c.z; w[7] = c.w;
         }
@@ -1076,7 +1076,7 @@ __device__ __forceinline__ void dist_items_stream(const __nv_bfloat16* W, long l
     for (int taken = 0; cons.item < last; ++taken) {
         if (fresh) {  // the activation weights of this item's columns, needed when the item ends
 #pragma unroll
-            for (int e = 0; e < 8; ++e) rj[e] = act_rms && cons.valid ? __ldg(act_rms + cons.j0 + e) : 1.0f;
+            for (int e = 0; e < 8; ++e) rj[e] = act_rms && cons.valid ? act_rms[cons.j0 + e] : 1.0f;
             fresh = false;
         }
         asm volatile("cp.async.wait_group %0;" ::"n"(kDistDepth - 2) : "memory");

@@ -194,7 +194,7 @@ __device__ __forceinline__ void st_global_256(void* p, const uint32_t (&w)[8]) {
                  : "memory");
 }
 __device__ __forceinline__ void ld_global_256(const void* p, uint32_t (&w)[8]) {
-    asm volatile("ld.global.nc.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+    asm volatile("ld.global.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
                  : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]), "=r"(w[4]), "=r"(w[5]), "=r"(w[6]), "=r"(w[7])
                  : "l"(p));
 }
@@ -341,7 +341,7 @@ __global__ void __launch_bounds__(NS == 4 ? 512 : 896, 1) decode2_kernel(const D
         const float* rnp = d.row_norm + row0;
 
         for (int it = 0; it < n_rows; ++it, orow += out_step, rnp += row_step) {
-            const float rn = __ldg(rnp);
+            const float rn = *rnp;
             cp_async_wait_pending<kDecodeDepth - 2>();
             __syncwarp();  // every lane's part of this row has landed; the buffer refilled next is no longer read
             issue_row();
@@ -591,7 +591,7 @@ __global__ void __launch_bounds__(MAXT, 1) encode2_kernel(const Encode2Args a) {
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
                 const int i = base + u * blockDim.x + threadIdx.x;
-                if (i < n16) v[u] = __ldg(a.table + i);
+                if (i < n16) v[u] = load_blob(a.table + i);
             }
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
@@ -726,7 +726,7 @@ __global__ void __launch_bounds__(MAXT, 1) encode2_kernel(const Encode2Args a) {
 #pragma unroll
                 for (int h = 0; h < kRaw / 4; ++h)  // 16 bytes: an octet of bf16, half of one of f32
                     if (col0 + 16 * h / kEsz < d_in) {
-                        const uint4 w = __ldg(reinterpret_cast<const uint4*>(wp + 16 * h));
+                        const uint4 w = *reinterpret_cast<const uint4*>(wp + 16 * h);
                         raw[4 * h] = w.x;
                         raw[4 * h + 1] = w.y;
                         raw[4 * h + 2] = w.z;

@@ -5,6 +5,7 @@
 
 #include <algorithm>
 
+#include "qamw_device.cuh"
 #include "qamw_internal.h"
 
 using namespace qamw;
@@ -32,7 +33,7 @@ __global__ void renorm_kernel(const uint8_t* packed, long long stride, const flo
         const int wi = int(bit >> 5);
         const uint32_t lo = w[wi], hi = wi + 1 < n_words ? w[wi + 1] : 0u;
         const uint32_t idx = __funnelshift_r(lo, hi, bit & 31u) & mask;
-        const float2 c = __ldg(codebook + idx);
+        const float2 c = load_blob(codebook + idx);
         const double sg = double(sigma[k]);
         const double cx = double(c.x) * sg, cy = double(c.y) * sg;
         ss += cx * cx + cy * cy;

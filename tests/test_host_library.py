@@ -227,3 +227,26 @@ def test_polar_levels_and_table_agree_with_oracle(orc, Ba):
     assert lib.qamw_codebook_create_polar(None, 2, 2, C.byref(h)) == q.ERR_ARG
     bad = np.array([1.0, 0.5], np.float32)  # not ascending
     assert lib.qamw_codebook_create_polar(bad.ctypes.data, 1, 2, C.byref(h)) == q.ERR_ARG
+
+
+def _kernel_sources():
+    src = os.path.join(ROOT, "paper_2605_26339_b200", "csrc")
+    for name in sorted(os.listdir(src)):
+        if name.endswith((".cu", ".cuh")):
+            text = open(os.path.join(src, name)).read()
+            yield name, re.sub(r"//[^\n]*", "", re.sub(r"/\*.*?\*/", "", text, flags=re.S))
+
+
+def test_only_the_codebook_is_read_through_the_read_only_path():
+    """A kernel may start while its predecessor on the stream still writes, and a read-only load is valid only for
+    memory that nothing writes while the kernel runs.  That holds for the codebook's blob alone: one function reads
+    through that path, and it is given nothing but codewords and cell records."""
+    direct, through = [], []
+    for name, text in _kernel_sources():
+        direct += [(name, m) for m in re.findall(r"__ldg\s*\(|ld\.global[a-z0-9.:_]*\.nc|__restrict__", text)]
+        through += [(name, m) for m in re.findall(r"(?<!T )\bload_blob\(([^)]*)\)", text)]
+    assert direct == [("qamw_device.cuh", "__ldg(")]
+    assert through and {arg for _, arg in through} <= {"src + i", "a.table + i", "codebook + idx"}
+    # `src` is the source of the codebook copies: every caller hands over the blob's codewords
+    fills = [arg for _, text in _kernel_sources() for arg in re.findall(r"fill_codebook_copies\(reinterpret_cast<float2\*>\(smem\), ([a-z.]+),", text)]
+    assert fills and set(fills) == {"a.codebook"}
