@@ -48,7 +48,10 @@ namespace qamw {
 
 static thread_local char g_last_error[256] = "";
 
+// Records the error of a call for qamw_last_cuda_error().  The runtime keeps it too, for the next cudaGetLastError() of
+// the thread; it has been reported here and must not turn up again as the error of a later, sound call.
 void set_cuda_error(const char* what, int code) {
+    cudaGetLastError();
     std::snprintf(g_last_error, sizeof(g_last_error), "%s: %s", what, cudaGetErrorString(cudaError_t(code)));
 }
 void set_error_text(const char* text) { std::snprintf(g_last_error, sizeof(g_last_error), "%s", text); }

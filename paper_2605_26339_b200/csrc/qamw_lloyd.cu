@@ -742,7 +742,7 @@ extern "C" int qamw_train_codebook_gpu(int K, uint64_t n_samples, uint64_t seed,
     const KeyOf cell{assign, nullptr, 0, 0x7fffffff};
     TrainState seen{};
     int recorded = 0;
-    while (ok(cudaGetLastError())) {
+    while (e == cudaSuccess) {
         for (int k = 0; k < kBatch && recorded + k <= max_iters; ++k) {
             assign_pass(assign, state);
             ok(launch_chained(hist_kernel, n_chunks + 1, 512, sizeof(int) * K, nullptr, cell, n, chunk, K, hist, tile_err, n_tiles, rel_tol, max_iters,

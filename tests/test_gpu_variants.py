@@ -1,5 +1,6 @@
 """GPU side of the variants around the path: 16-bit metadata (Section 3.2), the decoder's optional
 renormalisation (Section A.3), the alpha grid (Section B.2) and the on-disk blob."""
+import ctypes as C
 import os
 
 import numpy as np
@@ -234,3 +235,33 @@ def test_quantize_prepares_the_columns_as_the_host_functions_do(d_in, alpha):
     assert np.array_equal(signs.cpu().numpy(), q.make_signs(123456789, d_in))
     if alpha:
         np.testing.assert_allclose(s.cpu().numpy(), q.channel_scales(act, alpha), rtol=1.2e-7)
+
+
+def test_a_refused_launch_is_reported_once():
+    """A launch that the runtime refuses on the host is the error of the call that made it, and of no later one.  The
+    refusal: work for the default stream while another stream that synchronises with it is being captured."""
+    rt = C.CDLL("libcudart.so.12")  # torch's copy, loaded already
+    W, act = _problem(51, 8, 256)
+    W = W.to(DEV)
+    p = q.make_params(W, 8, 256, 64, 256)
+    signs = torch.from_numpy(q.make_signs(1, 256)).to(DEV)
+    y, norm = torch.empty((8, 256), device=DEV), torch.empty(8, device=DEV)
+    half = torch.ones(4, device=DEV)
+    q.rotate(W, p, None, signs, y, norm)
+    torch.cuda.synchronize()
+    stream, graph = C.c_void_p(), C.c_void_p()
+    assert rt.cudaStreamCreate(C.byref(stream)) == 0
+    try:
+        assert rt.cudaStreamBeginCapture(stream, 0) == 0
+        try:
+            with pytest.raises(q.QamwError) as e:
+                q.rotate(W, p, None, signs, y, norm)
+            assert e.value.code == q.ERR_CUDA
+        finally:
+            rt.cudaStreamEndCapture(stream, C.byref(graph))  # the refusal has ended the capture
+            rt.cudaGetLastError()
+        q.round_f16(half)
+        out = q.train_codebook_gpu(2, 4096, 0, 2)
+        assert out["iters"] == 2 and np.isfinite(out["codebook"]).all()
+    finally:
+        assert rt.cudaStreamDestroy(stream) == 0
