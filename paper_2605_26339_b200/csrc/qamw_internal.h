@@ -78,6 +78,26 @@ bool choose_search_table(const float* codebook, int K, int grid, size_t budget_b
 // grid * grid * 2 words, and the list words.  False if the lists do not fit their fields.
 bool pack_device_table(const SearchTable& t, int K, int log2_entry, std::vector<uint32_t>* words, std::vector<uint32_t>* lists);
 
+#ifdef __CUDACC__
+#define QAMW_HOST_DEVICE __host__ __device__
+#else
+#define QAMW_HOST_DEVICE
+#endif
+
+// The samples [lo, hi) of a cell as a warp walks them, kStep at a time.  Positions are 64-bit: a call may have up to
+// 2^31 - 1 samples, so a position of the next step need not fit an int.
+struct CellWalk {
+    static constexpr int kStep = 64;
+    long long base, hi;
+    QAMW_HOST_DEVICE CellWalk(int lo, int end) : base(lo), hi(end) {}
+    QAMW_HOST_DEVICE bool more() const { return base < hi; }
+    QAMW_HOST_DEVICE bool full() const { return hi - base >= kStep; }
+    QAMW_HOST_DEVICE int left() const { return int(hi - base); }
+    QAMW_HOST_DEVICE bool has(int k) const { return base + k < hi; }  // k < 2 kStep: this step's samples and the next one's
+    QAMW_HOST_DEVICE long long at(int k) const { return base + k; }
+    QAMW_HOST_DEVICE void step() { base += kStep; }
+};
+
 void set_cuda_error(const char* what, int code);
 void set_error_text(const char* text);
 

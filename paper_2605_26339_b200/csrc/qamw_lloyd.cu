@@ -554,27 +554,27 @@ __global__ void __launch_bounds__(32 * kCellWarps) centroid_kernel(const double2
                                                                    const TrainState* state) {
     chain_release();
     chain_wait();
-    __shared__ __align__(16) double stage[kCellWarps][2][64];
+    __shared__ __align__(16) double stage[kCellWarps][2][CellWalk::kStep];
     if (state->done) return;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, c = blockIdx.x * kCellWarps + warp;
     if (c >= K) return;
     const int lo = start[c], hi = start[c + 1];
     if (hi <= lo) return;
     double (*st)[64] = stage[warp];
-    const double2 zero = make_double2(0.0, 0.0);
-    double2 a = lo + lane < hi ? by_cell[lo + lane] : zero, b = lo + 32 + lane < hi ? by_cell[lo + 32 + lane] : zero;
+    CellWalk walk(lo, hi);
+    auto sample = [&](int k) { return walk.has(k) ? by_cell[walk.at(k)] : make_double2(0.0, 0.0); };
+    double2 a = sample(lane), b = sample(32 + lane);
     double sum = 0.0;
-    for (int base = lo; base < hi; base += 64) {
+    for (; walk.more(); walk.step()) {
         st[0][lane] = a.x;
         st[1][lane] = a.y;
         st[0][32 + lane] = b.x;
         st[1][32 + lane] = b.y;
-        const int next = base + 64 + lane;
-        a = next < hi ? by_cell[next] : zero;
-        b = next + 32 < hi ? by_cell[next + 32] : zero;
+        a = sample(64 + lane);
+        b = sample(96 + lane);
         __syncwarp();
         if (lane < 2) {
-            if (hi - base >= 64) {
+            if (walk.full()) {
                 const double2* v = reinterpret_cast<const double2*>(st[lane]);
                 double2 q[2][8];
 #pragma unroll
@@ -592,7 +592,7 @@ __global__ void __launch_bounds__(32 * kCellWarps) centroid_kernel(const double2
                     }
                 }
             } else {
-                for (int k = 0; k < hi - base; ++k) sum += st[lane][k];
+                for (int k = 0; k < walk.left(); ++k) sum += st[lane][k];
             }
         }
         __syncwarp();

@@ -5,6 +5,7 @@ launched.  No compute call needs a GPU here."""
 import ctypes as C
 import os
 import re
+import subprocess
 
 import numpy as np
 import pytest
@@ -250,3 +251,35 @@ def test_only_the_codebook_is_read_through_the_read_only_path():
     # `src` is the source of the codebook copies: every caller hands over the blob's codewords
     fills = [arg for _, text in _kernel_sources() for arg in re.findall(r"fill_codebook_copies\(reinterpret_cast<float2\*>\(smem\), ([a-z.]+),", text)]
     assert fills and set(fills) == {"a.codebook"}
+
+
+@pytest.mark.parametrize("lo,hi", [(0, 1), (5, 69), (7, 200), (2**31 - 1 - 300, 2**31 - 1), (2**31 - 1 - 64, 2**31 - 1),
+                                   (2**31 - 40, 2**31 - 1), (2**31 - 2, 2**31 - 1)])
+def test_a_cell_is_walked_inside_its_bounds(tmp_path_factory, lo, hi):
+    """The positions at which the centroid kernel reads a cell's samples, for cells up to the largest sample number
+    that the trainer accepts: each sample once, in order, none outside."""
+    out = tmp_path_factory.getbasetemp() / "walk"
+    if not out.exists():
+        src = out.with_suffix(".cpp")
+        src.write_text(r'''
+#include <cstdio>
+#include <cstdlib>
+#include "qamw_internal.h"
+int main(int, char** v) {
+    const int lo = std::atoi(v[1]), hi = std::atoi(v[2]);
+    qamw::CellWalk w(lo, hi);
+    long long next = lo, steps = 0, outside = 0;
+    auto read = [&](int k) { if (w.has(k)) outside += w.at(k) < lo || w.at(k) >= hi; };
+    for (int k = 0; k < qamw::CellWalk::kStep; ++k) read(k);
+    for (; w.more() && ++steps < 100; w.step()) {
+        for (int k = 0; k < qamw::CellWalk::kStep; ++k) read(qamw::CellWalk::kStep + k);
+        const int n = w.full() ? int(qamw::CellWalk::kStep) : w.left();
+        for (int k = 0; k < n; ++k) outside += w.at(k) != next++;
+    }
+    std::printf("%lld %lld %lld", next, steps, outside);
+}
+''')
+        subprocess.run(["g++", "-O1", "-std=c++17", "-fsanitize=undefined", "-fno-sanitize-recover", "-I", os.path.join(ROOT, "include"), "-I",
+                        os.path.join(ROOT, "paper_2605_26339_b200", "csrc"), str(src), "-o", str(out)], check=True)
+    got = subprocess.run([str(out), str(lo), str(hi)], check=True, capture_output=True, text=True).stdout
+    assert [int(x) for x in got.split()] == [hi, -(-(hi - lo) // 64), 0]
