@@ -104,8 +104,9 @@ int qamw_train_codebook(int K, uint64_t n_samples, uint64_t seed, int max_iters,
  * ties), every cell's samples added in sample order, same stopping rule, same final order and f32
  * rounding; the result does not vary from run to run.
  * samples_dev: device, n_samples (x, y) pairs of doubles to train on -- e.g. normalised pairs of a
- * checkpoint -- or NULL: the unit circular Gaussian samples of counter stream `seed` are generated on
- * the device (the device's log / sin / cos may differ from the host's in the last bit).
+ * checkpoint (work that still writes them may be queued on any stream: the call waits for the device
+ * first) -- or NULL: the unit circular Gaussian samples of counter stream `seed` are generated on the
+ * device (the device's log / sin / cos may differ from the host's in the last bit).
  * codebook_out: host, K*2 floats.  Optional host outputs (NULL to skip): train_mse_out as in
  * qamw_train_codebook; iters_out: centroid updates done; mse_trace_out: max_iters + 1 doubles, the
  * mean squared distance before every update; seconds_out: wall time of the call.

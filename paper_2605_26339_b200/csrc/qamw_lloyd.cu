@@ -699,6 +699,9 @@ extern "C" int qamw_train_codebook_gpu(int K, uint64_t n_samples, uint64_t seed,
     TrainState* state = reinterpret_cast<TrainState*>(base + o_state);
     float* scale = reinterpret_cast<float*>(base + o_scale);
     const double2* samples = samples_dev ? reinterpret_cast<const double2*>(samples_dev) : generated;
+    // The kernels run on the default stream; the caller's samples may still be on their way on one that does not wait
+    // for it and that it does not wait for.
+    if (samples_dev) ok(cudaDeviceSynchronize());
     if (!samples_dev) {
         // stream key as in the header of qamw_train_codebook: mix64(seed ^ 0xD1B54A32D192ED03)
         unsigned long long key = seed ^ 0xD1B54A32D192ED03ULL;

@@ -99,3 +99,18 @@ def test_tiles_and_chunks_that_do_not_fill(orc, K, n):
     out = q.train_codebook_gpu(K, max_iters=9, rel_tol=1e-9, samples=torch.from_numpy(z).to(DEV))
     assert out["iters"] == ref_iters and np.array_equal(out["codebook"], ref_cb)
     assert abs(out["mse"] - ref_mse) <= 1e-12 * ref_mse
+
+
+def test_samples_still_on_their_way_on_another_stream():
+    """Samples that a stream of the caller's is still writing when the call is made: the call waits for them."""
+    g = torch.Generator(device=DEV)
+    g.manual_seed(5)
+    z = torch.randn((20000, 2), generator=g, device=DEV, dtype=torch.float64)
+    want = q.train_codebook_gpu(64, max_iters=5, rel_tol=0.0, samples=z)
+    late = torch.zeros_like(z)
+    torch.cuda.synchronize()
+    with torch.cuda.stream(torch.cuda.Stream()):
+        torch.cuda._sleep(50_000_000)  # clocks: some 25 ms
+        late.copy_(z)
+        got = q.train_codebook_gpu(64, max_iters=5, rel_tol=0.0, samples=late)
+    assert np.array_equal(got["codebook"], want["codebook"]) and np.array_equal(got["trace"], want["trace"])
