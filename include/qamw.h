@@ -14,7 +14,8 @@
  *     prints or traps.  Argument errors are detected on the host before anything is launched.
  *   - "device" pointers are CUDA global-memory addresses on the current device, "host" pointers
  *     are ordinary process memory.  The caller owns every buffer; the library allocates device
- *     memory only inside a qamw_codebook (released by qamw_codebook_destroy).
+ *     memory only inside a qamw_codebook and a qamw_batch (released by their destroy functions) and
+ *     for codebook training (kept in part between calls, see qamw_release_scratch).
  *   - Device-side functions are asynchronous: they enqueue kernels on `stream` (a cudaStream_t
  *     passed as void*, NULL = the default stream) and return without synchronising.
  *   - Matrices are row-major.  W is f32 or bf16 (QAMW_DTYPE_*), with `w_row_stride` elements
@@ -110,12 +111,18 @@ int qamw_train_codebook(int K, uint64_t n_samples, uint64_t seed, int max_iters,
  * codebook_out: host, K*2 floats.  Optional host outputs (NULL to skip): train_mse_out as in
  * qamw_train_codebook; iters_out: centroid updates done; mse_trace_out: max_iters + 1 doubles, the
  * mean squared distance before every update; seconds_out: wall time of the call.
- * Synchronous; allocates and frees its device scratch (about 40 bytes per sample,
- * 16 more for generated samples) itself.
+ * Synchronous; allocates its device scratch (about 45 bytes per sample, 16 more for generated samples)
+ * itself, from a pool that keeps up to 256 MB of it on the device for the next call:
+ * qamw_release_scratch gives that back.
  * n_samples < 2^31. */
 int qamw_train_codebook_gpu(int K, uint64_t n_samples, uint64_t seed, const double* samples_dev, int max_iters,
                             double rel_tol, float* codebook_out, double* train_mse_out, int* iters_out,
                             double* mse_trace_out, double* seconds_out);
+
+/* Gives the device memory that qamw_train_codebook_gpu has kept on the current device back to the driver.
+ * Waits for the default stream; any thread may call it, also while another one trains (scratch in use
+ * stays).  Nothing to do, and QAMW_OK, where nothing is kept. */
+int qamw_release_scratch(void);
 
 /* Section B.2: s_j = clamp(r_j^alpha / geomean(r^alpha), 1/16, 16); r_j floored at FLT_MIN;
  * alpha == 0 gives all ones.  act_rms, s_out: host, d_in floats. */

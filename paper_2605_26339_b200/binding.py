@@ -36,7 +36,7 @@ EXPORTED = [
     "qamw_distortion", "qamw_last_cuda_error",
     "qamw_batch_create", "qamw_batch_destroy", "qamw_batch_workspace_bytes", "qamw_calibrate_batch",
     "qamw_encode_batch", "qamw_decode_batch", "qamw_distortion_batch",
-    "qamw_quantize", "qamw_gemv_workspace_bytes", "qamw_decode_gemv", "qamw_measure_fp32_peak", "qamw_train_codebook_gpu", "qamw_round_f16", "qamw_renorm_row_norms", "qamw_polar_train", "qamw_polar_codebook", "qamw_codebook_create_polar",
+    "qamw_quantize", "qamw_gemv_workspace_bytes", "qamw_decode_gemv", "qamw_measure_fp32_peak", "qamw_train_codebook_gpu", "qamw_release_scratch", "qamw_round_f16", "qamw_renorm_row_norms", "qamw_polar_train", "qamw_polar_codebook", "qamw_codebook_create_polar",
 ]
 
 
@@ -176,6 +176,11 @@ def train_codebook_gpu(K: int, n_samples: int = 1 << 20, seed: int = 0, max_iter
         K, n_samples, seed, _dp(samples), max_iters, rel_tol, cb.ctypes.data, C.addressof(mse), C.addressof(iters),
         trace.ctypes.data, C.addressof(secs)))
     return dict(codebook=cb, mse=mse.value, iters=iters.value, trace=trace[~np.isnan(trace)], seconds=secs.value)
+
+
+def release_scratch():
+    """Gives the device memory that training keeps for its next call (up to 256 MB per device) back to the driver."""
+    _check("qamw_release_scratch", lib().qamw_release_scratch())
 
 
 def channel_scales(act_rms, alpha: float) -> np.ndarray:

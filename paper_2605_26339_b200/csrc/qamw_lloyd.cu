@@ -618,16 +618,17 @@ __global__ void init_kernel(const double2* samples, int K, double2* codebook, fl
 }
 
 // Where the scratch memory of a call comes from: a pool per device that keeps up to 256 MB between calls (the
-// default size takes 60 MB; with cudaMalloc and cudaFree a call cost 3 ms more) and gives it back to the driver
-// when another allocation of the process needs it.  NULL if the device has no pools of its own.
+// default size takes 60 MB; with cudaMalloc and cudaFree a call cost 3 ms more) until qamw_release_scratch gives it
+// back.  NULL if the device has no pools of its own, or, without `create`, if there is none yet.
 constexpr int kMaxDevices = 64;
-cudaMemPool_t scratch_pool() {
+constexpr size_t kKeepBytes = size_t(256) << 20;
+cudaMemPool_t scratch_pool(bool create) {
     static std::mutex mu;
     static cudaMemPool_t pools[kMaxDevices] = {};
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev >= kMaxDevices) return nullptr;
     std::lock_guard<std::mutex> lock(mu);
-    if (!pools[dev]) {
+    if (!pools[dev] && create) {
         cudaMemPoolProps props{};
         props.allocType = cudaMemAllocationTypePinned;
         props.location.type = cudaMemLocationTypeDevice;
@@ -637,7 +638,7 @@ cudaMemPool_t scratch_pool() {
             cudaGetLastError();
             return nullptr;
         }
-        uint64_t keep = 256ull << 20;
+        uint64_t keep = kKeepBytes;
         cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep);
         pools[dev] = p;
     }
@@ -645,6 +646,18 @@ cudaMemPool_t scratch_pool() {
 }
 
 }  // namespace
+
+extern "C" int qamw_release_scratch(void) {
+    cudaMemPool_t pool = scratch_pool(false);
+    if (!pool) return QAMW_OK;
+    cudaError_t e = cudaStreamSynchronize(nullptr);  // the last call's scratch is freed in the order of this stream
+    if (e == cudaSuccess) e = cudaMemPoolTrimTo(pool, 0);
+    if (e != cudaSuccess) {
+        set_cuda_error("qamw_release_scratch", int(e));
+        return QAMW_ERR_CUDA;
+    }
+    return QAMW_OK;
+}
 
 extern "C" int qamw_train_codebook_gpu(int K, uint64_t n_samples, uint64_t seed, const double* samples_dev,
                                        int max_iters, double rel_tol, float* codebook_out, double* train_mse_out,
@@ -671,7 +684,7 @@ extern "C" int qamw_train_codebook_gpu(int K, uint64_t n_samples, uint64_t seed,
                  o_box = piece(sizeof(TileBox) * n_tiles * kBoxes), o_state = piece(sizeof(TrainState)), o_scale = piece(sizeof(float));
     unsigned char* base = nullptr;
     cudaError_t e = cudaSuccess;
-    if (cudaMemPool_t pool = scratch_pool()) {
+    if (cudaMemPool_t pool = scratch_pool(true)) {
         e = cudaMallocFromPoolAsync(reinterpret_cast<void**>(&base), bytes, pool, nullptr);
     } else {
         e = cudaMallocAsync(reinterpret_cast<void**>(&base), bytes, nullptr);
@@ -682,8 +695,12 @@ extern "C" int qamw_train_codebook_gpu(int K, uint64_t n_samples, uint64_t seed,
     }
     struct Free {
         void* p;
-        ~Free() { cudaFreeAsync(p, nullptr); }
-    } owner{base};
+        size_t bytes;
+        ~Free() {
+            cudaFreeAsync(p, nullptr);
+            if (bytes > kKeepBytes) cudaStreamSynchronize(nullptr);  // a pool lets go of what it may not keep when it is waited for
+        }
+    } owner{base, bytes};
     auto ok = [&](cudaError_t r) {
         if (e == cudaSuccess) e = r;
         return e == cudaSuccess;

@@ -114,3 +114,23 @@ def test_samples_still_on_their_way_on_another_stream():
         late.copy_(z)
         got = q.train_codebook_gpu(64, max_iters=5, rel_tol=0.0, samples=late)
     assert np.array_equal(got["codebook"], want["codebook"]) and np.array_equal(got["trace"], want["trace"])
+
+
+def test_scratch_kept_between_calls_is_bounded_and_given_back():
+    """Device memory that training holds on to: at most 256 MB whatever a call needed, none after release_scratch, and
+    the next call works as before."""
+    q.train_codebook_gpu(16, 1 << 12, 0, 1)  # contexts, modules
+    q.release_scratch()
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    slack = 4 << 20
+    first = q.train_codebook_gpu(256, 1 << 20, 0, 2)  # 60 MB of scratch
+    kept = free - torch.cuda.mem_get_info()[0]
+    assert (40 << 20) <= kept <= (256 << 20)
+    q.train_codebook_gpu(256, 1 << 23, 0, 1)  # 480 MB
+    assert free - torch.cuda.mem_get_info()[0] <= (256 << 20) + slack
+    q.release_scratch()
+    assert free - torch.cuda.mem_get_info()[0] <= slack
+    q.release_scratch()
+    assert np.array_equal(q.train_codebook_gpu(256, 1 << 20, 0, 2)["codebook"], first["codebook"])
+    q.release_scratch()

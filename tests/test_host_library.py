@@ -283,3 +283,7 @@ int main(int, char** v) {
                         os.path.join(ROOT, "paper_2605_26339_b200", "csrc"), str(src), "-o", str(out)], check=True)
     got = subprocess.run([str(out), str(lo), str(hi)], check=True, capture_output=True, text=True).stdout
     assert [int(x) for x in got.split()] == [hi, -(-(hi - lo) // 64), 0]
+
+
+def test_release_scratch_without_anything_kept():
+    assert q.lib().qamw_release_scratch() == q.QAMW_OK
