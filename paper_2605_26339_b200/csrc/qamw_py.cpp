@@ -14,15 +14,15 @@ namespace {
 
 struct Failed {};  // a Python error has been set
 
-void* tensor_ptr(PyObject* o) {
-    if (o == Py_None) return nullptr;
+const at::Tensor& tensor(PyObject* o) {
     if (!THPVariable_Check(o)) {
         PyErr_Format(PyExc_TypeError, "expected a torch tensor, got %s", Py_TYPE(o)->tp_name);
         throw Failed{};
     }
-    return const_cast<void*>(THPVariable_Unpack(o).const_data_ptr());
+    return THPVariable_Unpack(o);
 }
-size_t tensor_bytes(PyObject* o) { return THPVariable_Unpack(o).numel() * THPVariable_Unpack(o).element_size(); }
+void* tensor_ptr(PyObject* o) { return o == Py_None ? nullptr : const_cast<void*>(tensor(o).const_data_ptr()); }
+size_t tensor_bytes(PyObject* o) { return tensor(o).numel() * tensor(o).element_size(); }
 
 // The memory of an object with the buffer interface (a ctypes structure or pointer, a numpy array).
 struct Bytes {
@@ -113,9 +113,9 @@ PyObject* py_decode_gemv(PyObject*, PyObject* const* a, Py_ssize_t n) {
         const auto* cb = handle<qamw_codebook>(a[5]);
         const Params p(a[6]);
         auto* y = ptr<float>(a[8]);
-        const int n_vec = int(THPVariable_Unpack(a[7]).size(0));
+        const int n_vec = int(tensor(a[7]).size(0));
+        const size_t ws_bytes = tensor(a[9]).numel();
         void *ws = tensor_ptr(a[9]), *st = stream_ptr(a[10]);
-        const size_t ws_bytes = THPVariable_Unpack(a[9]).numel();
         return call([&] { return qamw_decode_gemv(packed, norm, scale, signs, sigma, cb, p.get(), x, n_vec, y, ws, ws_bytes, st); });
     });
 }

@@ -9,6 +9,7 @@ import subprocess
 
 import numpy as np
 import pytest
+import torch
 
 from conftest import ROOT, load_golden_codebook
 from paper_2605_26339_b200 import binding as q
@@ -287,3 +288,15 @@ int main(int, char** v) {
 
 def test_release_scratch_without_anything_kept():
     assert q.lib().qamw_release_scratch() == q.QAMW_OK
+
+
+def test_the_python_entry_refuses_what_is_no_tensor():
+    """An argument that has to be a tensor and is not: a Python error, whatever stands in its place."""
+    p = q.Params(4, 256, 64, 256, q.DTYPE_BF16, 0, 256, 128)
+    t, x, none = torch.zeros(1024, dtype=torch.uint8), torch.zeros((1, 256)), C.c_void_p()
+    for bad in (None, 7, np.zeros((1, 256), np.float32)):
+        with pytest.raises(TypeError):
+            q.ext().decode_gemv(t, t, None, t, t, none, p, bad, t, t, None)
+    for bad in (None, "t"):
+        with pytest.raises(TypeError):
+            q.ext().decode_gemv(t, t, None, t, t, none, p, x, t, bad, None)
