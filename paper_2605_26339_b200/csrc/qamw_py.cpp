@@ -21,7 +21,10 @@ const at::Tensor& tensor(PyObject* o) {
     }
     return THPVariable_Unpack(o);
 }
-void* tensor_ptr(PyObject* o) { return o == Py_None ? nullptr : const_cast<void*>(tensor(o).const_data_ptr()); }
+// Memory that the call reads; memory that it writes.  Asking for the second makes a tensor that shares its memory until it
+// is written (a lazy clone) take its own.
+const void* tensor_ptr(PyObject* o) { return o == Py_None ? nullptr : tensor(o).const_data_ptr(); }
+void* written_ptr(PyObject* o) { return o == Py_None ? nullptr : tensor(o).mutable_data_ptr(); }
 size_t tensor_bytes(PyObject* o) { return tensor(o).numel() * tensor(o).element_size(); }
 
 // The memory of an object with the buffer interface (a ctypes structure or pointer, a numpy array).
@@ -91,31 +94,33 @@ int call(F f) {
     return rc;
 }
 template <class T>
-T* ptr(PyObject* o) { return static_cast<T*>(tensor_ptr(o)); }
+const T* in(PyObject* o) { return static_cast<const T*>(tensor_ptr(o)); }
+template <class T>
+T* out(PyObject* o) { return static_cast<T*>(written_ptr(o)); }
 
 PyObject* py_decode(PyObject*, PyObject* const* a, Py_ssize_t n) {
     return guarded(n, 9, [&] {
-        const auto* packed = ptr<uint8_t>(a[0]);
-        const auto *norm = ptr<float>(a[1]), *scale = ptr<float>(a[2]), *sigma = ptr<float>(a[4]);
-        const auto* signs = ptr<int8_t>(a[3]);
+        const auto* packed = in<uint8_t>(a[0]);
+        const auto *norm = in<float>(a[1]), *scale = in<float>(a[2]), *sigma = in<float>(a[4]);
+        const auto* signs = in<int8_t>(a[3]);
         const auto* cb = handle<qamw_codebook>(a[5]);
         const Params p(a[6]);
-        void *out = tensor_ptr(a[7]), *st = stream_ptr(a[8]);
-        return call([&] { return qamw_decode(packed, norm, scale, signs, sigma, cb, p.get(), out, st); });
+        void *w_hat = written_ptr(a[7]), *st = stream_ptr(a[8]);
+        return call([&] { return qamw_decode(packed, norm, scale, signs, sigma, cb, p.get(), w_hat, st); });
     });
 }
 
 PyObject* py_decode_gemv(PyObject*, PyObject* const* a, Py_ssize_t n) {
     return guarded(n, 11, [&] {
-        const auto* packed = ptr<uint8_t>(a[0]);
-        const auto *norm = ptr<float>(a[1]), *scale = ptr<float>(a[2]), *sigma = ptr<float>(a[4]), *x = ptr<float>(a[7]);
-        const auto* signs = ptr<int8_t>(a[3]);
+        const auto* packed = in<uint8_t>(a[0]);
+        const auto *norm = in<float>(a[1]), *scale = in<float>(a[2]), *sigma = in<float>(a[4]), *x = in<float>(a[7]);
+        const auto* signs = in<int8_t>(a[3]);
         const auto* cb = handle<qamw_codebook>(a[5]);
         const Params p(a[6]);
-        auto* y = ptr<float>(a[8]);
+        auto* y = out<float>(a[8]);
         const int n_vec = int(tensor(a[7]).size(0));
         const size_t ws_bytes = tensor(a[9]).numel();
-        void *ws = tensor_ptr(a[9]), *st = stream_ptr(a[10]);
+        void *ws = written_ptr(a[9]), *st = stream_ptr(a[10]);
         return call([&] { return qamw_decode_gemv(packed, norm, scale, signs, sigma, cb, p.get(), x, n_vec, y, ws, ws_bytes, st); });
     });
 }
@@ -124,12 +129,12 @@ PyObject* py_encode(PyObject*, PyObject* const* a, Py_ssize_t n) {
     return guarded(n, 10, [&] {
         const void* W = tensor_ptr(a[0]);
         const Params p(a[1]);
-        const auto *scale = ptr<float>(a[2]), *sigma = ptr<float>(a[4]);
-        const auto* signs = ptr<int8_t>(a[3]);
+        const auto *scale = in<float>(a[2]), *sigma = in<float>(a[4]);
+        const auto* signs = in<int8_t>(a[3]);
         const auto* cb = handle<qamw_codebook>(a[5]);
-        auto* packed = ptr<uint8_t>(a[6]);
-        auto* norm = ptr<float>(a[7]);
-        auto* status = ptr<int32_t>(a[8]);
+        auto* packed = out<uint8_t>(a[6]);
+        auto* norm = out<float>(a[7]);
+        auto* status = out<int32_t>(a[8]);
         void* st = stream_ptr(a[9]);
         return call([&] { return qamw_encode(W, p.get(), scale, signs, sigma, cb, packed, norm, status, st); });
     });
@@ -139,12 +144,12 @@ PyObject* py_calibrate(PyObject*, PyObject* const* a, Py_ssize_t n) {
     return guarded(n, 8, [&] {
         const void* W = tensor_ptr(a[0]);
         const Params p(a[1]);
-        const auto* scale = ptr<float>(a[2]);
-        const auto* signs = ptr<int8_t>(a[3]);
-        auto* sigma = ptr<float>(a[4]);
-        void* ws = tensor_ptr(a[5]);
+        const auto* scale = in<float>(a[2]);
+        const auto* signs = in<int8_t>(a[3]);
+        auto* sigma = out<float>(a[4]);
+        void* ws = written_ptr(a[5]);
         const size_t ws_bytes = ws ? tensor_bytes(a[5]) : 0;
-        auto* status = ptr<int32_t>(a[6]);
+        auto* status = out<int32_t>(a[6]);
         void* st = stream_ptr(a[7]);
         return call([&] { return qamw_calibrate(W, p.get(), scale, signs, sigma, ws, ws_bytes, status, st); });
     });
@@ -160,13 +165,13 @@ PyObject* py_quantize(PyObject*, PyObject* const* a, Py_ssize_t n) {
         const uint64_t seed = PyLong_AsUnsignedLongLongMask(a[4]);
         if (PyErr_Occurred()) throw Failed{};
         const auto* cb = handle<qamw_codebook>(a[5]);
-        auto* scale = ptr<float>(a[6]);
-        auto* signs = ptr<int8_t>(a[7]);
-        auto *sigma = ptr<float>(a[8]), *norm = ptr<float>(a[10]);
-        auto* packed = ptr<uint8_t>(a[9]);
-        void* ws = tensor_ptr(a[11]);
+        auto* scale = out<float>(a[6]);
+        auto* signs = out<int8_t>(a[7]);
+        auto *sigma = out<float>(a[8]), *norm = out<float>(a[10]);
+        auto* packed = out<uint8_t>(a[9]);
+        void* ws = written_ptr(a[11]);
         const size_t ws_bytes = ws ? tensor_bytes(a[11]) : 0;
-        auto* status = ptr<int32_t>(a[12]);
+        auto* status = out<int32_t>(a[12]);
         void* st = stream_ptr(a[13]);
         return call([&] {
             return qamw_quantize(W, p.get(), act_rms, alpha, seed, cb, scale, signs, sigma, packed, norm, ws, ws_bytes, status, st);
@@ -177,9 +182,9 @@ PyObject* py_quantize(PyObject*, PyObject* const* a, Py_ssize_t n) {
 PyObject* py_calibrate_batch(PyObject*, PyObject* const* a, Py_ssize_t n) {
     return guarded(n, 4, [&] {
         const auto* b = handle<qamw_batch>(a[0]);
-        void* ws = tensor_ptr(a[1]);
+        void* ws = written_ptr(a[1]);
         const size_t ws_bytes = ws ? tensor_bytes(a[1]) : 0;
-        auto* status = ptr<int32_t>(a[2]);
+        auto* status = out<int32_t>(a[2]);
         void* st = stream_ptr(a[3]);
         return call([&] { return qamw_calibrate_batch(b, ws, ws_bytes, status, st); });
     });
@@ -187,7 +192,7 @@ PyObject* py_calibrate_batch(PyObject*, PyObject* const* a, Py_ssize_t n) {
 PyObject* py_encode_batch(PyObject*, PyObject* const* a, Py_ssize_t n) {
     return guarded(n, 3, [&] {
         const auto* b = handle<qamw_batch>(a[0]);
-        auto* status = ptr<int32_t>(a[1]);
+        auto* status = out<int32_t>(a[1]);
         void* st = stream_ptr(a[2]);
         return call([&] { return qamw_encode_batch(b, status, st); });
     });

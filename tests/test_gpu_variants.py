@@ -265,3 +265,18 @@ def test_a_refused_launch_is_reported_once():
         assert out["iters"] == 2 and np.isfinite(out["codebook"]).all()
     finally:
         assert rt.cudaStreamDestroy(stream) == 0
+
+
+def test_outputs_that_share_memory_until_they_are_written(orc):
+    """An output tensor that still shares its memory with another (a lazy clone) takes its own before the call writes."""
+    W, act = _problem(52, 16, 256)
+    e = _encode(W, act, 0.3, 64, 256)
+    plain = torch.empty((16, 256), dtype=torch.bfloat16, device=DEV)
+    q.decode(e["packed"], e["norm"], e["s"], e["signs"], e["sigma"], e["cb"], e["p"], plain)
+    base = torch.zeros_like(plain)
+    out = torch._lazy_clone(base)
+    q.decode(e["packed"], e["norm"], e["s"], e["signs"], e["sigma"], e["cb"], e["p"], out)
+    assert torch.equal(out, plain) and not base.any()
+    packed, norm = torch.zeros_like(e["packed"]), torch.zeros_like(e["norm"])
+    q.encode(e["W"], e["p"], e["s"], e["signs"], e["sigma"], e["cb"], torch._lazy_clone(packed), torch._lazy_clone(norm))
+    assert not packed.any() and not norm.any()
