@@ -88,10 +88,11 @@ PyObject* guarded(Py_ssize_t got, Py_ssize_t want, F body) {
 }
 template <class F>
 int call(F f) {
-    PyThreadState* save = PyEval_SaveThread();
-    const int rc = f();
-    PyEval_RestoreThread(save);
-    return rc;
+    struct Unlocked {  // also when the call throws (out of host memory): guarded() needs the lock to report it
+        PyThreadState* save = PyEval_SaveThread();
+        ~Unlocked() { PyEval_RestoreThread(save); }
+    } unlocked;
+    return f();
 }
 template <class T>
 const T* in(PyObject* o) { return static_cast<const T*>(tensor_ptr(o)); }
