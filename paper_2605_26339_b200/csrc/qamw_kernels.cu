@@ -1419,6 +1419,7 @@ extern "C" int qamw_codebook_create(const float* codebook_host, int K, int grid,
     cudaError_t e = cudaGetDevice(&cb->device);
     if (e == cudaSuccess) e = cudaMalloc(&cb->d_blob, cb->blob_bytes);
     if (e == cudaSuccess) e = cudaMemcpy(cb->d_blob, blob.data(), cb->blob_bytes, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);  // a copy from pageable memory may return before it has arrived
     if (e != cudaSuccess) {
         set_cuda_error("qamw_codebook_create", int(e));
         if (cb->d_blob) cudaFree(cb->d_blob);
@@ -1469,6 +1470,7 @@ extern "C" int qamw_codebook_create_polar(const float* levels_host, int Ba, int 
     cudaError_t e = cudaGetDevice(&cb->device);
     if (e == cudaSuccess) e = cudaMalloc(&cb->d_blob, cb->blob_bytes);
     if (e == cudaSuccess) e = cudaMemcpy(cb->d_blob, blob.data(), cb->blob_bytes, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);  // a copy from pageable memory may return before it has arrived
     if (e != cudaSuccess) {
         set_cuda_error("qamw_codebook_create_polar", int(e));
         if (cb->d_blob) cudaFree(cb->d_blob);

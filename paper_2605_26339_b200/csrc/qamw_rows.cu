@@ -1423,6 +1423,8 @@ extern "C" int qamw_batch_create(const qamw_matrix* items, int n, const qamw_cod
         if (e == cudaSuccess) e = cudaMalloc(&b->d_dist_counter, sizeof(unsigned int) * size_t(n));
         if (e == cudaSuccess) e = cudaMemset(b->d_dist_counter, 0, sizeof(unsigned int) * size_t(n));
     }
+    // the handle may be used on a stream that does not wait for the default one
+    if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
     if (e != cudaSuccess) {
         set_cuda_error("qamw_batch_create", int(e));
         qamw_batch_destroy(b);
