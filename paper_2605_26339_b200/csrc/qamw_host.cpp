@@ -13,18 +13,6 @@ using namespace qamw;
 
 namespace {
 
-// SplitMix64 finaliser (Steele, Lea, Flood 2014).
-inline uint64_t mix64(uint64_t x) {
-    x ^= x >> 30;
-    x *= 0xBF58476D1CE4E5B9ULL;
-    x ^= x >> 27;
-    x *= 0x94D049BB133111EBULL;
-    x ^= x >> 31;
-    return x;
-}
-
-constexpr uint64_t kGolden = 0x9E3779B97F4A7C15ULL;
-
 inline double uniform01(uint64_t stream_key, uint64_t n) {
     uint64_t h = mix64(stream_key + kGolden * (n + 1));
     return (double(h >> 11) + 0.5) * (1.0 / 9007199254740992.0);
@@ -32,7 +20,7 @@ inline double uniform01(uint64_t stream_key, uint64_t n) {
 
 // Unit circular Gaussian samples by Box-Muller, sample i from counters 2i and 2i+1.
 void gaussian_pairs(uint64_t seed, uint64_t begin, uint64_t end, double* out) {
-    const uint64_t key = mix64(seed ^ 0xD1B54A32D192ED03ULL);
+    const uint64_t key = sample_key(seed);
     const double two_pi = 6.283185307179586476925286766559;
     for (uint64_t i = begin; i < end; ++i) {
         double u1 = uniform01(key, 2 * i), u2 = uniform01(key, 2 * i + 1);
@@ -193,7 +181,7 @@ extern "C" int qamw_channel_scales(const float* act_rms, int d_in, float alpha, 
 
 extern "C" int qamw_make_signs(uint64_t seed, int d_in, int8_t* signs_out) {
     if (!signs_out || d_in <= 0) return QAMW_ERR_ARG;
-    for (int j = 0; j < d_in; ++j) signs_out[j] = (mix64(seed + kGolden * uint64_t(j + 1)) >> 63) ? int8_t(-1) : int8_t(1);
+    for (int j = 0; j < d_in; ++j) signs_out[j] = column_sign(seed, j);
     return QAMW_OK;
 }
 

@@ -84,6 +84,21 @@ bool pack_device_table(const SearchTable& t, int K, int log2_entry, std::vector<
 #define QAMW_HOST_DEVICE
 #endif
 
+// SplitMix64 finaliser (Steele, Lea, Flood 2014) and the increment of its counter: signs and Gaussian samples.
+constexpr uint64_t kGolden = 0x9E3779B97F4A7C15ULL;
+QAMW_HOST_DEVICE inline uint64_t mix64(uint64_t x) {
+    x ^= x >> 30;
+    x *= 0xBF58476D1CE4E5B9ULL;
+    x ^= x >> 27;
+    x *= 0x94D049BB133111EBULL;
+    x ^= x >> 31;
+    return x;
+}
+// Key of the sample stream `seed`: sample i takes counters 2i and 2i + 1.
+QAMW_HOST_DEVICE inline uint64_t sample_key(uint64_t seed) { return mix64(seed ^ 0xD1B54A32D192ED03ULL); }
+// Sign of column j: -1 or 1.
+QAMW_HOST_DEVICE inline int8_t column_sign(uint64_t seed, int j) { return (mix64(seed + kGolden * uint64_t(j + 1)) >> 63) ? int8_t(-1) : int8_t(1); }
+
 // The samples [lo, hi) of a cell as a warp walks them, kStep at a time.  Positions are 64-bit: a call may have up to
 // 2^31 - 1 samples, so a position of the next step need not fit an int.
 struct CellWalk {

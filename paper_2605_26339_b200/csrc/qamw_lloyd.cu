@@ -46,25 +46,15 @@ constexpr int kManyChunks = 1024;    // many chunks,
 constexpr int kMaxChunk = 65504;     // but not more than 16-bit counters hold
 constexpr int kBatch = 8;            // iterations enqueued between two looks at the stopping rule
 
-__device__ __forceinline__ unsigned long long mix64(unsigned long long x) {  // SplitMix64 finaliser
-    x ^= x >> 30;
-    x *= 0xBF58476D1CE4E5B9ULL;
-    x ^= x >> 27;
-    x *= 0x94D049BB133111EBULL;
-    x ^= x >> 31;
-    return x;
-}
-
 // Unit circular Gaussian samples by Box-Muller from the counter stream of the header: sample i uses
 // the uniforms of counters 2i and 2i+1.
 __global__ void sample_kernel(unsigned long long key, unsigned long long n, double2* out) {
     chain_release();
     chain_wait();
-    const unsigned long long golden = 0x9E3779B97F4A7C15ULL;
     for (unsigned long long i = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; i < n;
          i += (unsigned long long)gridDim.x * blockDim.x) {
-        const double u1 = (double(mix64(key + golden * (2 * i + 1)) >> 11) + 0.5) * (1.0 / 9007199254740992.0);
-        const double u2 = (double(mix64(key + golden * (2 * i + 2)) >> 11) + 0.5) * (1.0 / 9007199254740992.0);
+        const double u1 = (double(mix64(key + kGolden * (2 * i + 1)) >> 11) + 0.5) * (1.0 / 9007199254740992.0);
+        const double u2 = (double(mix64(key + kGolden * (2 * i + 2)) >> 11) + 0.5) * (1.0 / 9007199254740992.0);
         const double rad = sqrt(-2.0 * log(u1));
         double s, c;
         sincos(6.283185307179586476925286766559 * u2, &s, &c);
@@ -720,14 +710,7 @@ extern "C" int qamw_train_codebook_gpu(int K, uint64_t n_samples, uint64_t seed,
     // for it and that it does not wait for.
     if (samples_dev) ok(cudaDeviceSynchronize());
     if (!samples_dev) {
-        // stream key as in the header of qamw_train_codebook: mix64(seed ^ 0xD1B54A32D192ED03)
-        unsigned long long key = seed ^ 0xD1B54A32D192ED03ULL;
-        key ^= key >> 30;
-        key *= 0xBF58476D1CE4E5B9ULL;
-        key ^= key >> 27;
-        key *= 0x94D049BB133111EBULL;
-        key ^= key >> 31;
-        ok(launch_chained(sample_kernel, 8 * sm_count(), 256, 0, nullptr, key, n, generated));
+        ok(launch_chained(sample_kernel, 8 * sm_count(), 256, 0, nullptr, sample_key(seed), n, generated));
     }
     auto sort_smem = [](int b) { return sizeof(int) * size_t(b) + size_t(kSortWarps) * size_t((b + 1) & ~1) * 2; };
     if (sort_smem(bins) > 48 * 1024)  // beyond the default dynamic limit

@@ -20,17 +20,11 @@ namespace {
 constexpr int kPrepBlocks = 8, kPrepThreads = 256;  // one cluster; 512 threads take 0.5 us longer at 1024 channels
 constexpr int kPrepMaxPerThread = 16384 / (kPrepBlocks * kPrepThreads);
 
-__device__ __forceinline__ unsigned long long mix64(unsigned long long x) {  // SplitMix64 finaliser
-    x = (x ^ (x >> 30)) * 0xBF58476D1CE4E5B9ULL;
-    x = (x ^ (x >> 27)) * 0x94D049BB133111EBULL;
-    return x ^ (x >> 31);
-}
-
 struct PrepArgs {
     const float* act;   // NULL: in the parameters
     float* chan_scale;  // NULL: signs only
     int8_t* signs;
-    unsigned long long seed;
+    uint64_t seed;
     float alpha;
     int d_in;
 };
@@ -56,7 +50,7 @@ __global__ void __cluster_dims__(kPrepBlocks) __launch_bounds__(kPrepThreads) pr
         const int j = j0 + i * kStep;
         t[i] = 0.0;
         if (j >= a.d_in) break;
-        a.signs[j] = (mix64(a.seed + 0x9E3779B97F4A7C15ULL * (unsigned long long)(j + 1)) >> 63) ? int8_t(-1) : int8_t(1);
+        a.signs[j] = column_sign(a.seed, j);
         if (!a.chan_scale) continue;
         double r = double(a.act ? a.act[j] : p.act[j < N ? j : 0]);
         if (!(r > double(FLT_MIN))) r = double(FLT_MIN);
