@@ -237,8 +237,10 @@ struct Decode2Args {
 // (stored as (x + y, x - y): butterfly stage h = 1) from its own bank-separated copy, scales them by
 // the pair scales, runs the remaining butterflies and writes bf16.
 // ALIGNED: packed rows start on 16 bytes, rows of the output on 32, d_in is a multiple of 16.
-template <int NS, int LOG2B, bool ALIGNED>
-__global__ void __launch_bounds__(NS == 4 ? 512 : 896, 1) decode2_kernel(const Decode2Args a) {
+constexpr int kDecodeSlots = 4, kDecodeWarps = 16;  // octets per thread; warps of a block at most
+template <int LOG2B, bool ALIGNED>
+__global__ void __launch_bounds__(32 * kDecodeWarps, 1) decode2_kernel(const Decode2Args a) {
+    constexpr int NS = kDecodeSlots;
     typedef Lay2<NS, LOG2B> Lay;
     constexpr int TOP = Lay::TOP;
     constexpr int WE = 256 * NS;  // elements of a warp segment
@@ -353,28 +355,18 @@ __global__ void __launch_bounds__(NS == 4 ? 512 : 896, 1) decode2_kernel(const D
                 const uint32_t w = in + run_word[x];
                 const uint32_t sh = run_shift[x];
                 uint32_t id[4 * TOP];
-                if (NS == 4) {
-                    // 8 indices = 8 B bits <= 96: four words, shifted down to three, then cut in steps of 2 B bits
-                    const uint32_t w0 = lds_u32(w), w1 = lds_u32(w + 4), w2 = lds_u32(w + 8), w3 = lds_u32(w + 12);
-                    uint32_t v0 = __funnelshift_r(w0, w1, sh), v1 = __funnelshift_r(w1, w2, sh), v2 = __funnelshift_r(w2, w3, sh);
+                // 8 indices = 8 B bits <= 96: four words, shifted down to three, then cut in steps of 2 B bits
+                const uint32_t w0 = lds_u32(w), w1 = lds_u32(w + 4), w2 = lds_u32(w + 8), w3 = lds_u32(w + 12);
+                uint32_t v0 = __funnelshift_r(w0, w1, sh), v1 = __funnelshift_r(w1, w2, sh), v2 = __funnelshift_r(w2, w3, sh);
 #pragma unroll
-                    for (int t = 0; t < 4; ++t) {
-                        id[2 * t] = v0 & mask;
-                        id[2 * t + 1] = (v0 >> B) & mask;
-                        if (t < 3) {
-                            v0 = __funnelshift_r(v0, v1, 2 * B);
-                            v1 = __funnelshift_r(v1, v2, 2 * B);
-                            v2 >>= 2 * B;
-                        }
+                for (int t = 0; t < 4; ++t) {
+                    id[2 * t] = v0 & mask;
+                    id[2 * t + 1] = (v0 >> B) & mask;
+                    if (t < 3) {
+                        v0 = __funnelshift_r(v0, v1, 2 * B);
+                        v1 = __funnelshift_r(v1, v2, 2 * B);
+                        v2 >>= 2 * B;
                     }
-                } else {
-                    const uint32_t w0 = lds_u32(w), w1 = lds_u32(w + 4), w2 = lds_u32(w + 8);
-                    const uint32_t a0 = __funnelshift_r(w0, w1, sh), a1 = __funnelshift_r(w1, w2, sh);
-                    const uint32_t b0 = __funnelshift_r(a0, a1, 2 * B);
-                    id[0] = a0 & mask;
-                    id[1] = (a0 >> B) & mask;
-                    id[2] = b0 & mask;
-                    id[3] = (b0 >> B) & mask;
                 }
 #pragma unroll
                 for (int t = 0; t < TOP; ++t) {
@@ -390,8 +382,8 @@ __global__ void __launch_bounds__(NS == 4 ? 512 : 896, 1) decode2_kernel(const D
             fwht2<NS, LOG2B, true>(P, lane, a.log2b);
             const f32x2 rn2 = pack2(rn, rn);
 #pragma unroll
-            for (int p = 0; p < NS; p += (NS == 4 ? 2 : 1)) {
-                constexpr int NP = NS == 4 ? 2 : 1;  // adjacent octets written by one store
+            for (int p = 0; p < NS; p += 2) {
+                constexpr int NP = 2;  // adjacent octets written by one store
                 uint32_t w[4 * NP];
 #pragma unroll
                 for (int t = 0; t < NP; ++t)
@@ -402,7 +394,7 @@ __global__ void __launch_bounds__(NS == 4 ? 512 : 896, 1) decode2_kernel(const D
                         __nv_bfloat162 h2 = __floats2bfloat162_rn(y0, y1);
                         w[4 * t + i] = *reinterpret_cast<uint32_t*>(&h2);
                     }
-                if constexpr (NS == 4 && ALIGNED) {
+                if constexpr (ALIGNED) {
                     if (e_out[p] < d_in) st_global_256(orow + e_out[p], w);
                 } else {
 #pragma unroll
@@ -952,9 +944,9 @@ int raise_smem_limit(const void* kernel) {
     return QAMW_OK;
 }
 
-template <int NS, int LOG2B>
+template <int LOG2B>
 int launch_decode2(const Decode2Args& a, bool fits, int blocks, int threads, size_t smem, cudaStream_t st) {
-    auto kernel = fits ? decode2_kernel<NS, LOG2B, true> : decode2_kernel<NS, LOG2B, false>;
+    auto kernel = fits ? decode2_kernel<LOG2B, true> : decode2_kernel<LOG2B, false>;
     int rc = raise_smem_limit(reinterpret_cast<const void*>(kernel));
     if (rc) return rc;
     return launch_check("decode2_kernel", launch_chained(kernel, blocks, threads, smem, st, a));
@@ -1017,7 +1009,7 @@ void make_spans(const MatDesc* descs, int n, int n_blocks, const int* row_cost, 
 
 int rows_decode(const MatDesc* descs_dev, const MatDesc* descs_host, int n, const void* spans_dev, int span_blocks,
                 int block, int K, const float* codebook_dev, uint32_t flags, void* stream) {
-    constexpr int NS = 4, WE = 256 * NS, kWarps = 16;
+    constexpr int NS = kDecodeSlots, WE = 256 * NS, kWarps = kDecodeWarps;
     const int log2b = ilog2(block);
     if (n <= 0) return QAMW_ERR_SHAPE;
     long long pairs = 0;
@@ -1059,13 +1051,13 @@ int rows_decode(const MatDesc* descs_dev, const MatDesc* descs_host, int n, cons
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     int rc = QAMW_ERR_SHAPE;
     switch (log2b >= 5 ? log2b : 0) {
-        case 0: rc = launch_decode2<NS, 0>(a, fits, blocks, warps * 32, smem, st); break;
-        case 5: rc = launch_decode2<NS, 5>(a, fits, blocks, warps * 32, smem, st); break;
-        case 6: rc = launch_decode2<NS, 6>(a, fits, blocks, warps * 32, smem, st); break;
-        case 7: rc = launch_decode2<NS, 7>(a, fits, blocks, warps * 32, smem, st); break;
-        case 8: rc = launch_decode2<NS, 8>(a, fits, blocks, warps * 32, smem, st); break;
-        case 9: rc = launch_decode2<NS, 9>(a, fits, blocks, warps * 32, smem, st); break;
-        case 10: rc = launch_decode2<NS, 10>(a, fits, blocks, warps * 32, smem, st); break;
+        case 0: rc = launch_decode2<0>(a, fits, blocks, warps * 32, smem, st); break;
+        case 5: rc = launch_decode2<5>(a, fits, blocks, warps * 32, smem, st); break;
+        case 6: rc = launch_decode2<6>(a, fits, blocks, warps * 32, smem, st); break;
+        case 7: rc = launch_decode2<7>(a, fits, blocks, warps * 32, smem, st); break;
+        case 8: rc = launch_decode2<8>(a, fits, blocks, warps * 32, smem, st); break;
+        case 9: rc = launch_decode2<9>(a, fits, blocks, warps * 32, smem, st); break;
+        case 10: rc = launch_decode2<10>(a, fits, blocks, warps * 32, smem, st); break;
         default: break;
     }
     return rc;
@@ -1099,7 +1091,7 @@ int encode_warps(int n_seg, int block) {
 int encode_class(int warps) {  // rows too long for any size end up in the last class and fall back later
     return warps ? (warps - 16) / 4 : kEncodeClasses - 1;
 }
-int decode_groups(int n_seg) { return 16 / n_seg; }
+int decode_groups(int n_seg) { return kDecodeWarps / n_seg; }
 constexpr int kCostUnit = 360360;  // divisible by every group count 1..15
 
 int rows_encode(const MatDesc* descs_dev, const MatDesc* descs_host, int n, const void* spans_dev, int span_blocks,
