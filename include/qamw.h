@@ -356,12 +356,16 @@ void qamw_batch_destroy(qamw_batch* b);
 /* Device scratch qamw_calibrate_batch needs (the per-matrix needs, each rounded up to 256 bytes). */
 size_t qamw_batch_workspace_bytes(const qamw_batch* b);
 
+/* Kernels that the four phases launch on this batch, one after the other (QAMW_ERR_ARG for NULL). */
+int qamw_batch_launches(const qamw_batch* b);
+
 /* The four phases over all matrices of the batch, each equivalent to calling the single-matrix
  * entry point on every item in order (same results bit for bit, same error codes), asynchronous on
- * `stream`.  Matrices in the common layout (rows and metadata 16-byte aligned, d_in a multiple of
- * 16, block >= 32) are handled by one launch per phase -- up to three in calibrate and encode, whose
- * kernels run with one of three block sizes chosen by row length; if any item falls outside, the
- * phase falls back to one launch per matrix.  Two exceptions to "bit for
+ * `stream`.  Matrices in the common layout (rows of W and W_hat and metadata 16-byte aligned, packed rows on 4
+ * bytes, d_in a multiple of 8) are handled by one launch per phase -- up to four in calibrate and encode, whose
+ * kernels run with one of four block sizes chosen by row length, and one that finishes the calibration; if an item
+ * falls outside, the phase (calibrate, encode: the items with its block size) falls back to launches per
+ * matrix.  Two exceptions to "bit for
  * bit": the batched calibration groups the rows differently (pair scales agree to the last bits,
  * about 1e-7 relative), and the batched distortion adds its partial sums in a fixed order, so its four
  * sums are the same bits on every run (the single-matrix call uses atomic adds; both agree to about

@@ -34,7 +34,7 @@ EXPORTED = [
     "qamw_codebook_destroy", "qamw_codebook_table_info", "qamw_search_table_build",
     "qamw_calibrate_workspace_bytes", "qamw_calibrate", "qamw_calibrate_static", "qamw_encode", "qamw_rotate", "qamw_decode",
     "qamw_distortion", "qamw_last_cuda_error",
-    "qamw_batch_create", "qamw_batch_destroy", "qamw_batch_workspace_bytes", "qamw_calibrate_batch",
+    "qamw_batch_create", "qamw_batch_destroy", "qamw_batch_workspace_bytes", "qamw_batch_launches", "qamw_calibrate_batch",
     "qamw_encode_batch", "qamw_decode_batch", "qamw_distortion_batch",
     "qamw_quantize", "qamw_gemv_workspace_bytes", "qamw_decode_gemv", "qamw_measure_fp32_peak", "qamw_train_codebook_gpu", "qamw_release_scratch", "qamw_round_f16", "qamw_renorm_row_norms", "qamw_polar_train", "qamw_polar_codebook", "qamw_codebook_create_polar",
 ]
@@ -111,6 +111,7 @@ def lib() -> C.CDLL:
         L.qamw_batch_destroy.restype = None
         L.qamw_batch_workspace_bytes.argtypes = [vp]
         L.qamw_batch_workspace_bytes.restype = sz
+        L.qamw_batch_launches.argtypes = [vp]
         L.qamw_calibrate_batch.argtypes = [vp, vp, sz, vp, vp]
         L.qamw_encode_batch.argtypes = [vp, vp, vp]
         L.qamw_decode_batch.argtypes = [vp, vp]
@@ -436,6 +437,10 @@ class Batch:
 
     def workspace_bytes(self) -> int:
         return int(lib().qamw_batch_workspace_bytes(self._h))
+
+    def launches(self) -> int:
+        """Kernels that calibrate, encode, decode and distortion launch, one after the other."""
+        return int(lib().qamw_batch_launches(self._h))
 
     def calibrate(self, workspace: torch.Tensor, status: Optional[torch.Tensor] = None, stream=None):
         _check("qamw_calibrate_batch", ext().calibrate_batch(self._h, workspace, status, stream))

@@ -137,12 +137,14 @@ struct MatDesc {
 
 // Fast multi-matrix paths (qamw_rows.cu).  `descs` is a device array of n descriptors, or NULL with
 // n == 1 and the single descriptor passed by value.  They return QAMW_ERR_SHAPE without launching
-// when a matrix does not meet the fast kernels' layout rules; the caller then uses the general kernels.
+// when a matrix does not meet the fast kernels' layout rules; the caller then uses the general kernels.  With `count`
+// they only add the number of their launches to it.
 int rows_decode(const MatDesc* descs_dev, const MatDesc* descs_host, int n, const void* spans_dev, int span_blocks,
-                int block, int K, const float* codebook_dev, uint32_t flags, void* stream);
+                int block, int K, const float* codebook_dev, uint32_t flags, void* stream, int* count = nullptr);
 int rows_encode(const MatDesc* descs_dev, const MatDesc* descs_host, int n, const void* spans_dev, int span_blocks,
                 int block, int K, int w_bf16, const ::qamw_codebook* cb, uint32_t flags, int32_t* status, void* stream,
-                void* calib_base = nullptr);  // calib_base: run the calibration pass instead (cb may be NULL)
+                void* calib_base = nullptr,  // run the calibration pass instead (cb may be NULL)
+                int* count = nullptr);
 // Sign mask and, if act_host is not NULL, channel scales of the columns, on the stream (qamw_prepare.cu); act_host
 // may be overwritten as soon as the call returns.
 int prepare_columns(const float* act_host, int d_in, float alpha, uint64_t seed, float* chan_scale, int8_t* signs, void* stream);

@@ -1008,7 +1008,7 @@ void make_spans(const MatDesc* descs, int n, int n_blocks, const int* row_cost, 
 }
 
 int rows_decode(const MatDesc* descs_dev, const MatDesc* descs_host, int n, const void* spans_dev, int span_blocks,
-                int block, int K, const float* codebook_dev, uint32_t flags, void* stream) {
+                int block, int K, const float* codebook_dev, uint32_t flags, void* stream, int* count) {
     constexpr int NS = kDecodeSlots, WE = 256 * NS, kWarps = kDecodeWarps;
     const int log2b = ilog2(block);
     if (n <= 0) return QAMW_ERR_SHAPE;
@@ -1048,6 +1048,10 @@ int rows_decode(const MatDesc* descs_dev, const MatDesc* descs_host, int n, cons
     const size_t stage_total = size_t(warps) * kDecodeDepth * a.stage_bytes;
     a.log2c = pick_copies(K, pairs / 32 / blocks, std::min(size_t(128) * 1024, kSmemLimit - stage_total));
     const size_t smem = (size_t(K) * 8 << a.log2c) + stage_total;
+    if (count) {
+        ++*count;
+        return QAMW_OK;
+    }
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     int rc = QAMW_ERR_SHAPE;
     switch (log2b >= 5 ? log2b : 0) {
@@ -1096,7 +1100,7 @@ constexpr int kCostUnit = 360360;  // divisible by every group count 1..15
 
 int rows_encode(const MatDesc* descs_dev, const MatDesc* descs_host, int n, const void* spans_dev, int span_blocks,
                 int block, int K, int w_bf16, const ::qamw_codebook* cb, uint32_t flags, int32_t* status, void* stream,
-                void* calib_base) {
+                void* calib_base, int* count) {
     const int log2b = ilog2(block), WE = encode_segment(block), NS = WE / 256;
     if (n <= 0) return QAMW_ERR_SHAPE;
     const size_t esz = w_bf16 ? 2 : 4;
@@ -1161,6 +1165,10 @@ int rows_encode(const MatDesc* descs_dev, const MatDesc* descs_host, int n, cons
     if (flags & QAMW_FLAG_HALF_DEVICE) grid = std::max(1, grid / 2);
     int blocks = spans_dev ? span_blocks : int(std::max<long long>(1, std::min<long long>(grid, rows)));
     if (!spans_dev && calib) blocks = descs_host[0].calib_slots;
+    if (count) {
+        ++*count;
+        return QAMW_OK;
+    }
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     int rc = QAMW_ERR_SHAPE;
 #define QAMW_ENC2(LB)                                                                          \
@@ -1557,4 +1565,30 @@ extern "C" int qamw_distortion_batch(const qamw_batch* b, void* stream) {
     red.counter = b->d_dist_counter;
     return distortion_batch_launch(b->dec.d_descs, b->d_spans_dist, b->n_blocks_dist, b->w_dtype == QAMW_DTYPE_BF16,
                                    red, stream);
+}
+
+// Kernels that the four phases launch, by the rules that they launch them by.
+extern "C" int qamw_batch_launches(const qamw_batch* b) {
+    if (!b) return QAMW_ERR_ARG;
+    const uint32_t flags = b->items[0].p.flags;
+    const bool general = flags & QAMW_FLAG_GENERAL_KERNELS, bf16 = b->w_dtype == QAMW_DTYPE_BF16;
+    int launches = 1;  // distortion
+    int passes = 0, single = 0;
+    char any = 0;  // stands for the workspace, which a counted call does not touch
+    for (int c = 0; c < kEncodeClasses; ++c) {
+        const RowSet &cal = b->cal[c], &enc = b->enc[c];
+        const int n = int(enc.descs.size());
+        if (n == 0) continue;
+        if (general || rows_encode(cal.d_descs, cal.descs.data(), n, cal.d_spans, b->n_blocks, b->block, b->K, bf16, nullptr, flags,
+                                   nullptr, nullptr, &any, &passes))
+            single += n;
+        if (general || rows_encode(enc.d_descs, enc.descs.data(), n, enc.d_spans, b->n_blocks, b->block, b->K, bf16, b->cb, flags,
+                                   nullptr, nullptr, nullptr, &launches))
+            for (const MatDesc& d : enc.descs) launches += d.d_out > 0;
+    }
+    launches += passes + 2 * single + (single ? passes : passes > 0);  // one finish for all classes, or one each
+    if (general || rows_decode(b->dec.d_descs, b->dec.descs.data(), b->n, b->dec.d_spans, b->n_blocks, b->block, b->K, nullptr, flags,
+                               nullptr, &launches))
+        for (const MatDesc& d : b->dec.descs) launches += d.d_out > 0;
+    return launches;
 }

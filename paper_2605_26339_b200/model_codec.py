@@ -237,8 +237,7 @@ class ModelCodec:
         self.distortion_all()
 
     def capture_step(self) -> "torch.cuda.CUDAGraph":
-        """The whole step as one CUDA graph (seven kernel nodes and a memset for a batched model): replaying
-        it costs one launch, which is what small models need -- their kernels take a few microseconds
+        """The whole step as one CUDA graph (a node for each of kernel_launches_per_step()): replaying it costs one launch, which is what small models need -- their kernels take a few microseconds
         each and the per-call overhead of the host dominates otherwise.  The batched phases launch on the
         current stream and allocate nothing, so they can be captured as they are."""
         if not (self.use_batch and self.batch is not None):
@@ -266,25 +265,10 @@ class ModelCodec:
         return enc, dec
 
     def kernel_launches_per_step(self) -> int:
-        # per matrix: calibrate = 2 kernels, distortion 1 (its memset is not a kernel of ours); encode and
-        # decode are per matrix too unless batched: then one decode launch and one encode launch per
-        # class of row lengths (rows of up to 11264 elements, longer rows)
-        n = len(self.slots)
         if self.use_batch and self.batch is not None:
-            # one encoder block size per class of row lengths: a calibration pass and an encode launch per
-            # class; one finish launch, one decode launch, one distortion launch
-            classes = len({self._encoder_class(s.d_in, self.spec.block) for s in self.slots})
-            return 2 * classes + 3
-        return 5 * n
-
-    @staticmethod
-    def _encoder_class(d_in: int, block: int) -> int:
-        """Warps of the encoder's block for this row length (the rule of the library)."""
-        if block == 1024:
-            return 16
-        n_seg = (d_in + 511) // 512
-        full = {16: 1.0, 20: 45.9 / 47.6, 24: 45.9 / 51.2, 28: 45.9 / 49.4}
-        return max(full, key=lambda w: full[w] * (min(15, w // n_seg) * n_seg) / w)
+            return self.batch.launches()
+        # per matrix: calibrate 2, encode 1, decode 1, distortion 1 (its memset is not a kernel of ours)
+        return 5 * len(self.slots)
 
     def totals(self, group=None) -> Dict[str, float]:
         """Error figures over all matrices of all ranks (see combine_distortion)."""

@@ -14,6 +14,8 @@ Exactness rules of this codec:
     must stay below kFarFraction;
   * calibration within 1e-5 relative; distortion sums within 1e-9 relative.
 """
+import ctypes as C
+
 import numpy as np
 import pytest
 import torch
@@ -692,3 +694,42 @@ def test_row_kernels_agree_with_the_general_ones_on_every_layout(orc, K, d_out, 
     torch.testing.assert_close(sig, sig_g, rtol=1e-6, atol=0)
     assert torch.equal(packed, packed_g) and torch.equal(norm, norm_g)
     assert torch.equal(w_hat.view(torch.int16), w_hat_g.view(torch.int16))
+
+
+@pytest.mark.parametrize("shapes,block", [
+    ([(64, 1024), (32, 5632), (16, 13824)], 128),      # rows of three block sizes
+    ([(64, 2048), (8, 4096)], 1024),
+    ([(64, 1024), (48, 1032), (16, 13824), (9, 6)], 2),  # one row too short for the row kernels
+    ([(64, 1024), (0, 1024)], 64)])
+def test_launches_of_a_batch(orc, shapes, block):
+    """The library's count of a step's kernels is the number of nodes of the captured step, also where some matrices
+    take the kernels for arbitrary layouts."""
+    cb = q.Codebook(load_golden_codebook(64))
+    keep, mats = [], []
+    for i, (d_out, d_in) in enumerate(shapes):
+        W = _make(max(1, d_out), d_in, torch.bfloat16, 900 + i)[0][:d_out].to(DEV)
+        p = q.make_params(W, d_out, d_in, block, 64)
+        t = dict(W=W, signs=torch.from_numpy(q.make_signs(3, d_in)).to(DEV), sigma=torch.ones(d_in // 2, device=DEV),
+                 packed=torch.zeros((d_out, p.packed_row_stride), dtype=torch.uint8, device=DEV), row_norm=torch.ones(d_out, device=DEV),
+                 w_hat=torch.zeros((d_out, d_in), dtype=torch.bfloat16, device=DEV), dist4=torch.zeros(4, dtype=torch.float64, device=DEV))
+        if d_out == 0:  # an empty tensor has no address
+            t.update({k: torch.zeros(8, dtype=t[k].dtype, device=DEV) for k in ("W", "packed", "row_norm", "w_hat")})
+        keep.append(t)
+        mats.append(q.make_matrix(p, **t))
+    b = q.Batch(mats, cb)
+    ws = torch.empty(max(8, b.workspace_bytes()), dtype=torch.uint8, device=DEV)
+
+    def step():
+        b.calibrate(ws)
+        b.encode()
+        b.decode()
+        b.distortion()
+
+    step()
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(g):
+        step()
+    n = C.c_size_t()
+    assert C.CDLL("libcudart.so.12").cudaGraphGetNodes(C.c_void_p(g.raw_cuda_graph()), None, C.byref(n)) == 0
+    assert b.launches() == n.value
