@@ -88,9 +88,10 @@ def test_codebook_fitted_to_a_matrix_beats_the_gaussian_one_on_it(orc):
     assert fit["mse"] < mse_gauss
 
 
-@pytest.mark.parametrize("K,n", [(2, 1027), (32, 511), (512, 513), (1024, 4097), (2048, 9000)])
+@pytest.mark.parametrize("K,n", [(2, 1027), (32, 255), (64, 256), (128, 257), (32, 511), (512, 513), (16, 4095), (256, 4096),
+                                 (1024, 4097), (2048, 9000)])
 def test_tiles_and_chunks_that_do_not_fill(orc, K, n):
-    """Sample counts around the edges of the spatial tiles (512) and sorting chunks (4096), every number of
+    """Sample counts around the edges of the spatial tiles (256) and sorting chunks (4096), every number of
     codewords per thread, samples with far outliers, exact duplicates and ties: same codebook as the oracle."""
     rng = np.random.default_rng(K + n)
     z = np.round(rng.standard_normal((n, 2)) * 8) / 8 + (rng.standard_normal((n, 2)) * 1e-3) * (rng.random((n, 1)) < 0.7)

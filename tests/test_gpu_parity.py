@@ -227,12 +227,10 @@ def test_cfg0_full(orc):
 @pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
 @pytest.mark.parametrize("block", [2, 4, 8, 16, 32, 64, 128, 256, 512, 1024])
 def test_block_sizes(orc, block, dtype, kernels):
-    """Every block size through the kernels for the common layouts (block >= 32) and, with
-    QAMW_FLAG_GENERAL_KERNELS, through the general row kernels."""
+    """Every block size through the kernels for the common layouts and, with QAMW_FLAG_GENERAL_KERNELS, through the
+    general row kernels."""
     W, act = _make(37, 2048, dtype, 100 + block)
     flags = q.FLAG_GENERAL_KERNELS if kernels == "general" else 0
-    if kernels == "general" and block < 32:
-        pytest.skip("blocks below 32 always run the general kernels")
     Case(orc, W, act, 0.3, block, 256, flags=flags).check_all()
 
 
