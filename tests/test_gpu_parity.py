@@ -442,8 +442,9 @@ def _batch_problem(shapes, K, block, dtype, flags=0):
 
 
 @pytest.mark.parametrize("shapes,block", [
-    ([(300, 2048), (64, 11776), (129, 512), (40, 5120)], 128),   # both encoder classes (rows beyond 11264 elements)
-    ([(77, 1024), (5, 24), (33, 2048)], 8),                      # a matrix outside the common layout: falls back
+    ([(300, 2048), (64, 11776), (129, 512), (40, 5120)], 128),   # rows of several encoder block sizes
+    ([(77, 1024), (5, 24), (33, 2048)], 8),                      # rows of a few octets
+    ([(77, 1024), (5, 20), (33, 2048)], 4),                      # a matrix outside the common layout: falls back
 ])
 def test_batch_equals_single_matrix_calls(orc, shapes, block):
     """qamw_*_batch over several matrices gives, bit for bit, what the single-matrix entry points give."""
@@ -560,7 +561,7 @@ def test_polar_encoder_refuses_layouts_outside_its_kernels(orc):
     lv, _ = q.polar_train(2)
     cb = q.Codebook.polar(lv, 2, 2)
     W = torch.zeros((4, 64), dtype=torch.float32, device=DEV)
-    p = q.make_params(W, 4, 64, 16, 16)  # block 16: only the general kernels take it
+    p = q.make_params(W, 4, 64, 16, 16)  # the polar quantiser takes blocks of 32 to 512
     dummy = torch.zeros(64, dtype=torch.uint8, device=DEV)
     signs = torch.ones(64, dtype=torch.int8, device=DEV)
     sigma = torch.ones(32, dtype=torch.float32, device=DEV)
