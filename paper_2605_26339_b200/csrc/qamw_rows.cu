@@ -1387,10 +1387,13 @@ extern "C" int qamw_batch_create(const qamw_matrix* items, int n, const qamw_cod
             if (e == cudaSuccess) e = cudaMemcpy(b->d_cal_all, all.data(), sizeof(MatDesc) * all.size(), cudaMemcpyHostToDevice);
         }
     }
-    // Distortion: equal numbers of work items per block.  Five blocks fit an SM; with up to 32 items for each of them one
-    // wave is best (a 1.1B layer 45.8 -> 40.2 us, in f32 75 -> 60: a block of one item only fills and drains its ring),
-    // beyond that sixteen per SM even out what the blocks lose to each other (four layers of 13B: 890 us with 5, 861 with
-    // 10, 874 with 16; forty layers: 8.20 ms with 10, 7.98 with 16).
+    // Distortion: equal numbers of work items per block.  Five blocks fit an SM, one wave.  bf16 rows run through a ring that
+    // a block fills and drains once: with few items one wave is best, with many more and shorter blocks even out what the
+    // SMs lose to each other.  us with 5, 16 and 24 blocks per SM, by items per block of one wave: 3.7 (a layer of 1.1B)
+    // 40.0, 45.9, 43.6; 14.9 (four of them) 137.9, 140.0, 137.4; 16.8 (a layer of 7B) 157.3, 157.6, 154.9; 26.4 (13B) 241,
+    // 238, 237; 33.6 306, 301, 285; 105 (four layers of 13B) 974, 909, 886; 1055 (forty) 10114, 9322, 9197.  f32 rows and
+    // rows off 16 bytes have no ring and lose what a last partial wave leaves idle: 58.8, 74.9, 66.3 at 3.7; 349, 408, 379
+    // at 26.4; 1365, 1579, 1409 at 105.
     if (e == cudaSuccess) {
         std::vector<MatDesc> items_as_rows(b->dec.descs);
         std::vector<int> unit(size_t(n), 1);
@@ -1400,7 +1403,8 @@ extern "C" int qamw_batch_create(const qamw_matrix* items, int n, const qamw_cod
             total += items_as_rows[size_t(i)].d_out;
         }
         const long long wave = 5LL * b->n_blocks;
-        b->n_blocks_dist = int(std::max<long long>(1, std::min<long long>(total < 32 * wave ? wave : 16LL * b->n_blocks, total)));
+        const bool many = b->w_dtype == QAMW_DTYPE_BF16 && total >= 20 * wave;
+        b->n_blocks_dist = int(std::max<long long>(1, std::min<long long>(many ? 24LL * b->n_blocks : wave, total)));
         std::vector<int4> spans;
         make_spans(items_as_rows.data(), n, b->n_blocks_dist, unit.data(), &spans);
         e = cudaMalloc(&b->d_spans_dist, sizeof(int4) * spans.size());
