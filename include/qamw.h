@@ -19,7 +19,7 @@
  *   - Device-side functions are asynchronous: they enqueue kernels on `stream` (a cudaStream_t
  *     passed as void*, NULL = the default stream) and return without synchronising.
  *   - Matrices are row-major.  W is f32 or bf16 (QAMW_DTYPE_*), with `w_row_stride` elements
- *     between rows; every row must start on a 16-byte boundary.
+ *     between rows.  Rows that start on a 16-byte boundary take the faster kernels.
  *   - Packed rows start `packed_row_stride` bytes apart (>= qamw_packed_row_bytes, a multiple
  *     of 4); index k of a row occupies stream bits [k*B, (k+1)*B), stream bit t being bit
  *     (t mod 8) of byte floor(t/8); padding bits up to the row stride are written as zero.
@@ -100,9 +100,9 @@ int qamw_train_codebook(int K, uint64_t n_samples, uint64_t seed, int max_iters,
 
 /* The same training on the current CUDA device (Section 3.6; the paper's Limitations section puts
  * its own trainer at about 5 s per bitrate level and names per-checkpoint codebooks as follow-up).
- * Same rules as qamw_train_codebook: same initial codewords, exact assignment in double (every
- * sample against every codeword, d = dx*dx + dy*dy with one rounding per operation, lowest index on
- * ties), every cell's samples added in sample order, same stopping rule, same final order and f32
+ * Same rules as qamw_train_codebook: same initial codewords, exact assignment in double (the result
+ * of comparing every sample with every codeword, d = dx*dx + dy*dy with one rounding per operation,
+ * lowest index on ties; codewords that a bound rules out are not compared), every cell's samples added in sample order, same stopping rule, same final order and f32
  * rounding; the result does not vary from run to run.
  * samples_dev: device, n_samples (x, y) pairs of doubles to train on -- e.g. normalised pairs of a
  * checkpoint (work that still writes them may be queued on any stream: the call waits for the device
@@ -156,8 +156,8 @@ int qamw_status_to_error(int32_t status_word);
  * codewords and widening outwards; every cell lists all codewords whose nearest-neighbour region
  * can meet the cell, so a scan of the list returns what a scan of the whole codebook returns.
  * The outermost cells reach to |z| < 16384; points beyond are scanned exhaustively.  grid = 0
- * picks a default (about 2.2 sqrt(K), at least 31, shrunk until the table fits next to the encoder's
- * other shared memory); an explicit grid must be odd and at most 255, else
+ * picks a default (3.1 sqrt(K), at least 31 and at most 255, shrunk until the table fits next to the
+ * encoder's other shared memory); an explicit grid must be odd and at most 255, else
  * QAMW_ERR_ARG.  Synchronous.
  * *out must be released with qamw_codebook_destroy on the same device. */
 int qamw_codebook_create(const float* codebook_host, int K, int grid, qamw_codebook** out);
@@ -253,13 +253,14 @@ int qamw_encode(const void* W, const qamw_params* p, const float* chan_scale, co
 
 /* The whole encoder side in one call, with the arguments of the paper's problem statement (Section
  * 3.1 with the scaling of Section B.2): W, activation statistics, scaling exponent, block size and
- * K (in p), codebook in; packed stream, row norms and the per-matrix metadata out.  Runs
- * qamw_channel_scales and qamw_make_signs on the host (act_rms_host: host, d_in floats, or NULL; no
- * scaling when it is NULL or alpha == 0, chan_scale_out may then be NULL), copies their d_in values
- * to chan_scale_out / signs_out, then qamw_calibrate and qamw_encode on `stream`.  All other
- * pointers device; workspace as for qamw_calibrate.  The two small host-to-device copies are issued
- * on `stream` from pageable memory (the call may wait for the stream's earlier work before them).
- * Results are those of the four calls made one after the other. */
+ * K (in p), codebook in; packed stream, row norms and the per-matrix metadata out.  Computes
+ * channel scales and signs on the device by the rules of qamw_channel_scales and qamw_make_signs
+ * (act_rms_host: host, d_in floats, read before the call returns, or NULL; no scaling when it is NULL
+ * or alpha == 0, chan_scale_out may then be NULL), then runs qamw_calibrate and qamw_encode, all on
+ * `stream`; nothing is copied or waited for.  All other pointers device; workspace as for
+ * qamw_calibrate.  Results are those of the four calls made one after the other, as far as the
+ * device's log and exp and the order of the mean's sum agree with the host's to f32: a scale may
+ * differ in its last bit (none of 12 million did). */
 int qamw_quantize(const void* W, const qamw_params* p, const float* act_rms_host, float alpha, uint64_t sign_seed,
                   const qamw_codebook* cb, float* chan_scale_out, int8_t* signs_out, float* sigma_out,
                   uint8_t* packed_out, float* row_norm_out, void* workspace, size_t workspace_bytes,
@@ -296,9 +297,9 @@ int qamw_renorm_row_norms(const uint8_t* packed, const float* row_norm, const fl
  * per call and no row is ever rotated back or written out.
  * x: device, n_vec vectors of d_in floats (n_vec in {1, 2, 4}); y_out: device, [d_out, n_vec] floats;
  * workspace: device, qamw_gemv_workspace_bytes(p, n_vec) bytes, 8-byte aligned.  d_in must be a
- * multiple of 32 (QAMW_ERR_SHAPE).  Packed rows and x that are 16-byte aligned (base and stride) take
- * the kernel that keeps the rotated activations in registers (one launch, any d_in up to the row-length
- * limit above); any other layout, or QAMW_FLAG_GENERAL_KERNELS, takes a layout-agnostic pair of kernels
+ * multiple of 32 (QAMW_ERR_SHAPE).  Arrays that start on 16 bytes (packed rows themselves on any 4) take
+ * the kernel that keeps the rotated activations in registers (one launch, two for four vectors; any d_in
+ * up to the row-length limit above); any other layout, or QAMW_FLAG_GENERAL_KERNELS, takes a layout-agnostic pair of kernels
  * whose rotated activations (n_vec * d_in floats) must fit in shared memory next to the codebook
  * (QAMW_ERR_NOMEM otherwise).  f32 accumulation in a fixed order: results are reproducible run to run;
  * asynchronous on `stream`. */

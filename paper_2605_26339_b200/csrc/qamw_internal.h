@@ -180,7 +180,7 @@ int distortion_batch_launch(const MatDesc* descs_dev, const void* spans_dev, int
 struct qamw_codebook {
     int K = 0;
     int device = -1;
-    // one device allocation: [codebook K*2 f32][cells grid^2 * 4 u16][overflow u16]
+    // one device allocation: [codebook K*2 f32][cell records grid^2 * 2 words][list words] (see pack_device_table)
     void* d_blob = nullptr;
     size_t blob_bytes = 0;
     size_t off_cells = 0, off_overflow = 0;

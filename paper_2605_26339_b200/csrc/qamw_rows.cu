@@ -4,7 +4,7 @@
 // Geometry.
 //   * A warp owns a "segment" of 256 * NS consecutive elements of a row: NS = 4 octets (32 elements)
 //     per thread in the decoder, NS = 2 (16 elements) in the encoder, whose register budget then
-//     allows 20 to 28 resident warps per SM instead of 15.  A row is owned by a group of
+//     allows up to 28 resident warps per SM (16 to 28 by row length, see encode_warps).  A row is owned by a group of
 //     ceil(d_in / (256 NS)) warps; a block holds as many groups as fit and the grid is persistent.
 //   * A launch takes an array of matrix descriptors.  The rows of all matrices form one list, cut
 //     into one contiguous span per block with (nearly) equal numbers of weights, so a block meets one
