@@ -162,6 +162,10 @@ PyObject* py_quantize(PyObject*, PyObject* const* a, Py_ssize_t n) {
         const Params p(a[1]);
         const Bytes act(a[2] == Py_None ? a[1] : a[2]);  // float32, checked by the caller
         const auto* act_rms = a[2] == Py_None ? nullptr : static_cast<const float*>(act.view.buf);
+        if (act_rms && act.view.len < Py_ssize_t(sizeof(float)) * p.get()->d_in) {
+            PyErr_Format(PyExc_ValueError, "%zd activation statistics for %d columns", act.view.len / Py_ssize_t(sizeof(float)), int(p.get()->d_in));
+            throw Failed{};
+        }
         const float alpha = float(PyFloat_AsDouble(a[3]));
         const uint64_t seed = PyLong_AsUnsignedLongLongMask(a[4]);
         if (PyErr_Occurred()) throw Failed{};

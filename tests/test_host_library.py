@@ -300,3 +300,10 @@ def test_the_python_entry_refuses_what_is_no_tensor():
     for bad in (None, "t"):
         with pytest.raises(TypeError):
             q.ext().decode_gemv(t, t, None, t, t, none, p, x, t, bad, None)
+
+
+def test_activation_statistics_cover_every_column():
+    p = q.Params(4, 256, 64, 256, q.DTYPE_BF16, 0, 256, 128)
+    t, none = torch.zeros(1024, dtype=torch.uint8), C.c_void_p()
+    with pytest.raises(ValueError, match="255 activation statistics for 256 columns"):
+        q.ext().quantize(t, p, np.ones(255, np.float32), 0.3, 1, none, t, t, t, t, t, t, t, None)
