@@ -293,8 +293,7 @@ def run_ours(args):
         return
 
     peak, peak_kind = measured_peaks()
-    enc_launches = len({mc._encoder_class(s.d_in, mc.spec.block) for s in mc.slots}) if mc.use_batch else len(mc.slots)
-    dec_launches = 1 if mc.use_batch else len(mc.slots)
+    _, enc_launches, dec_launches, _ = mc.batch.launches() if mc.use_batch else (0, len(mc.slots), len(mc.slots), 0)
     fp32_peak = q.measure_fp32_peak()
     pipe = load_pipe_note()
     enc_gbs = enc_bytes / (enc_ms * 1e-3) / 1e9

@@ -357,8 +357,9 @@ void qamw_batch_destroy(qamw_batch* b);
 /* Device scratch qamw_calibrate_batch needs (the per-matrix needs, each rounded up to 256 bytes). */
 size_t qamw_batch_workspace_bytes(const qamw_batch* b);
 
-/* Kernels that the four phases launch on this batch, one after the other (QAMW_ERR_ARG for NULL). */
-int qamw_batch_launches(const qamw_batch* b);
+/* Kernels that the four phases launch on this batch, one after the other (QAMW_ERR_ARG for NULL);
+ * per_phase_out (host, may be NULL): those of calibrate, encode, decode, distortion. */
+int qamw_batch_launches(const qamw_batch* b, int32_t* per_phase_out);
 
 /* The four phases over all matrices of the batch, each equivalent to calling the single-matrix
  * entry point on every item in order (same results bit for bit, same error codes), asynchronous on

@@ -111,7 +111,7 @@ def lib() -> C.CDLL:
         L.qamw_batch_destroy.restype = None
         L.qamw_batch_workspace_bytes.argtypes = [vp]
         L.qamw_batch_workspace_bytes.restype = sz
-        L.qamw_batch_launches.argtypes = [vp]
+        L.qamw_batch_launches.argtypes = [vp, vp]
         L.qamw_calibrate_batch.argtypes = [vp, vp, sz, vp, vp]
         L.qamw_encode_batch.argtypes = [vp, vp, vp]
         L.qamw_decode_batch.argtypes = [vp, vp]
@@ -438,9 +438,12 @@ class Batch:
     def workspace_bytes(self) -> int:
         return int(lib().qamw_batch_workspace_bytes(self._h))
 
-    def launches(self) -> int:
-        """Kernels that calibrate, encode, decode and distortion launch, one after the other."""
-        return int(lib().qamw_batch_launches(self._h))
+    def launches(self) -> Tuple[int, int, int, int]:
+        """Kernels that calibrate, encode, decode and distortion launch."""
+        n = (C.c_int32 * 4)()
+        if lib().qamw_batch_launches(self._h, n) < 0:
+            raise QamwError("qamw_batch_launches", ERR_ARG)
+        return tuple(n)
 
     def calibrate(self, workspace: torch.Tensor, status: Optional[torch.Tensor] = None, stream=None):
         _check("qamw_calibrate_batch", ext().calibrate_batch(self._h, workspace, status, stream))

@@ -1572,12 +1572,11 @@ extern "C" int qamw_distortion_batch(const qamw_batch* b, void* stream) {
 }
 
 // Kernels that the four phases launch, by the rules that they launch them by.
-extern "C" int qamw_batch_launches(const qamw_batch* b) {
+extern "C" int qamw_batch_launches(const qamw_batch* b, int32_t* per_phase_out) {
     if (!b) return QAMW_ERR_ARG;
     const uint32_t flags = b->items[0].p.flags;
     const bool general = flags & QAMW_FLAG_GENERAL_KERNELS, bf16 = b->w_dtype == QAMW_DTYPE_BF16;
-    int launches = 1;  // distortion
-    int passes = 0, single = 0;
+    int passes = 0, single = 0, encode = 0, decode = 0;
     char any = 0;  // stands for the workspace, which a counted call does not touch
     for (int c = 0; c < kEncodeClasses; ++c) {
         const RowSet &cal = b->cal[c], &enc = b->enc[c];
@@ -1587,12 +1586,14 @@ extern "C" int qamw_batch_launches(const qamw_batch* b) {
                                    nullptr, nullptr, &any, &passes))
             single += n;
         if (general || rows_encode(enc.d_descs, enc.descs.data(), n, enc.d_spans, b->n_blocks, b->block, b->K, bf16, b->cb, flags,
-                                   nullptr, nullptr, nullptr, &launches))
-            for (const MatDesc& d : enc.descs) launches += d.d_out > 0;
+                                   nullptr, nullptr, nullptr, &encode))
+            for (const MatDesc& d : enc.descs) encode += d.d_out > 0;
     }
-    launches += passes + 2 * single + (single ? passes : passes > 0);  // one finish for all classes, or one each
+    const int calibrate = passes + 2 * single + (single ? passes : passes > 0);  // one finish for all classes, or one each
     if (general || rows_decode(b->dec.d_descs, b->dec.descs.data(), b->n, b->dec.d_spans, b->n_blocks, b->block, b->K, nullptr, flags,
-                               nullptr, &launches))
-        for (const MatDesc& d : b->dec.descs) launches += d.d_out > 0;
-    return launches;
+                               nullptr, &decode))
+        for (const MatDesc& d : b->dec.descs) decode += d.d_out > 0;
+    const int phases[4] = {calibrate, encode, decode, 1};
+    if (per_phase_out) std::copy(phases, phases + 4, per_phase_out);
+    return phases[0] + phases[1] + phases[2] + phases[3];
 }

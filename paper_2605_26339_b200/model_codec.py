@@ -237,9 +237,10 @@ class ModelCodec:
         self.distortion_all()
 
     def capture_step(self) -> "torch.cuda.CUDAGraph":
-        """The whole step as one CUDA graph (a node for each of kernel_launches_per_step()): replaying it costs one launch, which is what small models need -- their kernels take a few microseconds
-        each and the per-call overhead of the host dominates otherwise.  The batched phases launch on the
-        current stream and allocate nothing, so they can be captured as they are."""
+        """The whole step as one CUDA graph (a node for each of kernel_launches_per_step()): replaying it costs one
+        launch, which is what small models need -- their kernels take a few microseconds each and the per-call
+        overhead of the host dominates otherwise.  The batched phases launch on the current stream and allocate
+        nothing, so they can be captured as they are."""
         if not (self.use_batch and self.batch is not None):
             raise RuntimeError("capture_step needs the batched phases (finalize() first)")
         self.step()  # first use outside the capture: per-kernel attributes are set once
@@ -266,7 +267,7 @@ class ModelCodec:
 
     def kernel_launches_per_step(self) -> int:
         if self.use_batch and self.batch is not None:
-            return self.batch.launches()
+            return sum(self.batch.launches())
         # per matrix: calibrate 2, encode 1, decode 1, distortion 1 (its memset is not a kernel of ours)
         return 5 * len(self.slots)
 

@@ -197,7 +197,7 @@ def test_argument_errors_are_reported_before_any_launch():
     assert lib.qamw_decode_batch(None, None) == q.ERR_ARG
     assert lib.qamw_distortion_batch(None, None) == q.ERR_ARG
     assert lib.qamw_calibrate_batch(None, ptr, 64, None, None) == q.ERR_ARG
-    assert lib.qamw_batch_workspace_bytes(None) == 0
+    assert lib.qamw_batch_workspace_bytes(None) == 0 and lib.qamw_batch_launches(None, None) == q.ERR_ARG
     h = C.c_void_p()
     cbk = np.zeros((4, 2), np.float32)
     assert lib.qamw_codebook_create(cbk.ctypes.data, 3, 0, C.byref(h)) == q.ERR_SHAPE
