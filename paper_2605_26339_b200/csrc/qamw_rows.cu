@@ -1391,9 +1391,10 @@ extern "C" int qamw_batch_create(const qamw_matrix* items, int n, const qamw_cod
     // a block fills and drains once: with few items one wave is best, with many more and shorter blocks even out what the
     // SMs lose to each other.  us with 5, 16 and 24 blocks per SM, by items per block of one wave: 3.7 (a layer of 1.1B)
     // 40.0, 45.9, 43.6; 14.9 (four of them) 137.9, 140.0, 137.4; 16.8 (a layer of 7B) 157.3, 157.6, 154.9; 26.4 (13B) 241,
-    // 238, 237; 33.6 306, 301, 285; 105 (four layers of 13B) 974, 909, 886; 1055 (forty) 10114, 9322, 9197.  f32 rows and
-    // rows off 16 bytes have no ring and lose what a last partial wave leaves idle: 58.8, 74.9, 66.3 at 3.7; 349, 408, 379
-    // at 26.4; 1365, 1579, 1409 at 105.
+    // 238, 237; 33.6 306, 301, 285; 105 (four layers of 13B) 974, 909, 886; 1055 (forty) 10114, 9322, 9197.  f32 rows
+    // have no ring and lose what a last partial wave leaves idle: 58.8, 74.9, 66.3 at 3.7; 349, 408, 379 at 26.4; 1365,
+    // 1579, 1409 at 105.  bf16 rows off 16 bytes have none either, and 5 and 24 blocks do alike: 209, 224, 214 at 15.3;
+    // 404, 438, 405 at 30.6; 1596, 1686, 1545 at 122.
     if (e == cudaSuccess) {
         std::vector<MatDesc> items_as_rows(b->dec.descs);
         std::vector<int> unit(size_t(n), 1);
