@@ -99,12 +99,13 @@ QAMW_HOST_DEVICE inline uint64_t sample_key(uint64_t seed) { return mix64(seed ^
 // Sign of column j: -1 or 1.
 QAMW_HOST_DEVICE inline int8_t column_sign(uint64_t seed, int j) { return (mix64(seed + kGolden * uint64_t(j + 1)) >> 63) ? int8_t(-1) : int8_t(1); }
 
-// The samples [lo, hi) of a cell as a warp walks them, kStep at a time.  Positions are 64-bit: a call may have up to
+// The samples [lo, hi) of a cell as a warp walks them, STEP at a time.  Positions are 64-bit: a call may have up to
 // 2^31 - 1 samples, so a position of the next step need not fit an int.
-struct CellWalk {
-    static constexpr int kStep = 64;
+template <int STEP>
+struct CellWalkBy {
+    static constexpr int kStep = STEP;
     long long base, hi;
-    QAMW_HOST_DEVICE CellWalk(int lo, int end) : base(lo), hi(end) {}
+    QAMW_HOST_DEVICE CellWalkBy(int lo, int end) : base(lo), hi(end) {}
     QAMW_HOST_DEVICE bool more() const { return base < hi; }
     QAMW_HOST_DEVICE bool full() const { return hi - base >= kStep; }
     QAMW_HOST_DEVICE int left() const { return int(hi - base); }
@@ -112,6 +113,7 @@ struct CellWalk {
     QAMW_HOST_DEVICE long long at(int k) const { return base + k; }
     QAMW_HOST_DEVICE void step() { base += kStep; }
 };
+using CellWalk = CellWalkBy<64>;
 
 void set_cuda_error(const char* what, int code);
 void set_error_text(const char* text);

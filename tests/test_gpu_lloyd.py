@@ -102,6 +102,38 @@ def test_tiles_and_chunks_that_do_not_fill(orc, K, n):
     assert abs(out["mse"] - ref_mse) <= 1e-12 * ref_mse
 
 
+@pytest.mark.parametrize("kind,K,n,iters", [
+    ("plain", 64, 70000, 40),      # cells of more than one chunk of the merge
+    ("plain", 64, 1152 * 64, 12),  # the largest cells that are updated incrementally,
+    ("plain", 64, 1153 * 64, 12),  # and the smallest that are not
+    ("plain", 2048, 60000, 60),    # tiles as wide as many codewords
+    ("plain", 4096, 40000, 30),
+    ("ties", 256, 20000, 40),      # a lattice: equal distances, equal samples, empty cells
+    ("outliers", 512, 30001, 40),  # boxes that hold half of the codebook
+    ("late", 128, 60000, 40),      # codewords that start in one place: cells still move when the incremental passes begin
+    ("point", 64, 3000, 20),       # one sample many times
+])
+def test_incremental_updates(orc, kind, K, n, iters):
+    """Training that goes on after the passes in full: the same codebook, updates and errors as the oracle.  (With a tolerance of zero
+    the rule would compare errors that differ in the order of their sums only.)"""
+    rng = np.random.default_rng(K + n)
+    z = rng.standard_normal((n, 2))
+    if kind == "ties":
+        z = np.round(z * 6) / 6
+    elif kind == "outliers":
+        z[rng.integers(0, n, n // 50)] *= 30.0
+    elif kind == "late":
+        z[:K] = 4.0 + 1e-3 * z[:K]
+    elif kind == "point":
+        z[:] = z[0]
+    ref_cb, ref_mse, ref_iters, ref_trace = orc.train_codebook_on(z, K, iters, 1e-12)
+    out = q.train_codebook_gpu(K, max_iters=iters, rel_tol=1e-12, samples=torch.from_numpy(z).to(DEV))
+    assert out["iters"] == ref_iters and np.array_equal(out["codebook"], ref_cb)
+    assert abs(out["mse"] - ref_mse) <= 1e-12 * ref_mse
+    again = q.train_codebook_gpu(K, max_iters=iters, rel_tol=1e-12, samples=torch.from_numpy(z).to(DEV))
+    assert np.array_equal(again["codebook"], out["codebook"]) and np.array_equal(again["trace"], out["trace"])
+
+
 def test_samples_still_on_their_way_on_another_stream():
     """Samples that a stream of the caller's is still writing when the call is made: the call waits for them."""
     g = torch.Generator(device=DEV)
