@@ -35,6 +35,8 @@ struct PrepParams {
 };
 
 // s_j = clamp(exp(alpha log r_j - mean), 1/16, 16) in double, as qamw_channel_scales; signs as qamw_make_signs.
+// Everything but the stores comes before the wait when the statistics are in the parameters: what follows the wait is on the
+// critical path of a chain of kernels that last two to five microseconds each.
 template <int N>
 __global__ void __cluster_dims__(kPrepBlocks) __launch_bounds__(kPrepThreads) prepare_kernel(const __grid_constant__ PrepParams<N> p) {
     __shared__ double part[kPrepThreads / 32], block_sum;
@@ -43,21 +45,27 @@ __global__ void __cluster_dims__(kPrepBlocks) __launch_bounds__(kPrepThreads) pr
     const int j0 = blockIdx.x * kPrepThreads + threadIdx.x;
     constexpr int kStep = kPrepBlocks * kPrepThreads;
     chain_release();
-    chain_wait();
+    if (a.act) chain_wait();  // the kernel before this one has written them
     double t[kPrepMaxPerThread], sum = 0.0;
 #pragma unroll
     for (int i = 0; i < kPrepMaxPerThread; ++i) {
         const int j = j0 + i * kStep;
         t[i] = 0.0;
         if (j >= a.d_in) break;
-        a.signs[j] = column_sign(a.seed, j);
         if (!a.chan_scale) continue;
         double r = double(a.act ? a.act[j] : p.act[j < N ? j : 0]);
         if (!(r > double(FLT_MIN))) r = double(FLT_MIN);
         t[i] = double(a.alpha) * log(r);
         sum += t[i];
     }
-    if (!a.chan_scale) return;  // the same for all blocks
+    auto store_signs = [&]() {
+        for (int j = j0; j < a.d_in; j += kStep) a.signs[j] = column_sign(a.seed, j);
+    };
+    if (!a.chan_scale) {  // the same for all blocks
+        chain_wait();
+        store_signs();
+        return;
+    }
     sum = warp_sum(sum);
     if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = sum;
     __syncthreads();
@@ -71,11 +79,20 @@ __global__ void __cluster_dims__(kPrepBlocks) __launch_bounds__(kPrepThreads) pr
     for (int b = 0; b < kPrepBlocks; ++b) mean += *cluster.map_shared_rank(&block_sum, b);
     mean /= double(a.d_in);
     cluster.sync();  // nobody leaves while its sum is still read
+    float s[kPrepMaxPerThread];
+#pragma unroll
+    for (int i = 0; i < kPrepMaxPerThread; ++i) {
+        s[i] = 0.f;
+        if (j0 + i * kStep >= a.d_in) break;
+        s[i] = float(fmin(16.0, fmax(1.0 / 16.0, exp(t[i] - mean))));
+    }
+    if (!a.act) chain_wait();
+    store_signs();
 #pragma unroll
     for (int i = 0; i < kPrepMaxPerThread; ++i) {
         const int j = j0 + i * kStep;
         if (j >= a.d_in) break;
-        a.chan_scale[j] = float(fmin(16.0, fmax(1.0 / 16.0, exp(t[i] - mean))));
+        a.chan_scale[j] = s[i];
     }
 }
 

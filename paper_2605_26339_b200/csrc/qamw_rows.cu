@@ -212,6 +212,46 @@ __device__ __forceinline__ int4 block_span(const int4* spans, int d_out_single) 
     return make_int4(0, int(n * blockIdx.x / gridDim.x), 0, int(n * (blockIdx.x + 1) / gridDim.x));
 }
 
+// Per-column constants of a thread's octets, as they lie in memory: scales and signs of octet e[p], pair scales of octet
+// k[p].  All loads are issued before the first is used, and none depends on a test (an octet lies inside the row or outside: d_in
+// is a multiple of 8; one outside reads the first and is masked by its user): loads behind tests of their own came one after the
+// other, 1.0 us for two octets and 4.4 us for four, before the first row was asked for.
+template <int NS, bool SIGMA>
+struct Columns {
+    float4 cs[NS][2], sg[SIGMA ? NS : 1];
+    uint2 sign[NS];
+    __device__ __forceinline__ void load(const float* chan_scale, const int8_t* signs, const float* sigma, const int (&e)[NS], const int (&k)[NS],
+                                         int d_in) {
+#pragma unroll
+        for (int p = 0; p < NS; ++p) {
+            sign[p] = *reinterpret_cast<const uint2*>(signs + (8 * e[p] < d_in ? 8 * e[p] : 0));
+            if (SIGMA) sg[SIGMA ? p : 0] = *reinterpret_cast<const float4*>(sigma + (8 * k[p] < d_in ? 4 * k[p] : 0));
+        }
+        if (chan_scale) {
+#pragma unroll
+            for (int p = 0; p < NS; ++p) {
+                const float4* c = reinterpret_cast<const float4*>(chan_scale + (8 * e[p] < d_in ? 8 * e[p] : 0));
+                cs[p][0] = c[0];
+                cs[p][1] = c[1];
+            }
+        } else {
+#pragma unroll
+            for (int p = 0; p < NS; ++p) cs[p][0] = cs[p][1] = make_float4(1.f, 1.f, 1.f, 1.f);
+        }
+    }
+    // scales (1 outside the row) and signs (0 outside)
+    __device__ __forceinline__ void unpack(int p, bool in, float (&c)[8], float (&s)[8]) const {
+        const float4 a = cs[p][0], b = cs[p][1];
+        const float v[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const uint32_t byte = ((i < 4 ? sign[p].x : sign[p].y) >> (8 * (i & 3))) & 0xffu;
+            c[i] = in ? v[i] : 1.0f;
+            s[i] = in ? __uint_as_float(0x3f800000u | ((byte & 0x80u) << 24)) : 0.f;  // +-1.0f from the byte's sign bit
+        }
+    }
+};
+
 // ---------------------------------------------------------------------------------------------
 // decoder
 // ---------------------------------------------------------------------------------------------
@@ -255,6 +295,8 @@ __global__ void __launch_bounds__(32 * kDecodeWarps, 1) decode2_kernel(const Dec
 
     chain_release();
     fill_codebook_copies(reinterpret_cast<float2*>(smem), a.codebook, a.K, a.log2c, true);
+    // spans and descriptors are written once, before the batch handle exists
+    const int4 span = block_span(a.spans, a.one.d_out);
     __syncthreads();
     chain_wait();
 
@@ -268,7 +310,6 @@ __global__ void __launch_bounds__(32 * kDecodeWarps, 1) decode2_kernel(const Dec
         run_shift[x] = bit0 & 31u;
     }
 
-    const int4 span = block_span(a.spans, a.one.d_out);
     for (int m = span.x; m <= span.z; ++m) {
         const MatDesc& d = a.descs ? a.descs[m] : a.one;
         const int d_in = d.d_in, n_pairs = d_in >> 1;
@@ -317,21 +358,25 @@ __global__ void __launch_bounds__(32 * kDecodeWarps, 1) decode2_kernel(const Dec
         const int oct0 = seg * (WE / 8);  // first octet of the segment
         float sg[NS][4];
         f32x2 mcol[NS][4];
-        int e_out[NS];
+        int e_out[NS], e_oct[NS], k_oct[NS];
 #pragma unroll
         for (int p = 0; p < NS; ++p) {
-            const int k0 = 4 * (oct0 + Lay::octet_before(lane, p));
-            load4f(d.sigma, k0, n_pairs, 1, 0.f, sg[p]);
-            const int e0 = 8 * (oct0 + Lay::octet_after(lane, p));
-            e_out[p] = e0;
-            float cs[8], sgn[8];
-            if (d.chan_scale) {
-                load8f(d.chan_scale, e0, d_in, 1, 1.0f, cs);
-            } else {
+            k_oct[p] = oct0 + Lay::octet_before(lane, p);
+            e_oct[p] = oct0 + Lay::octet_after(lane, p);
+        }
+        Columns<NS, true> cols;
+        cols.load(d.chan_scale, d.signs, d.sigma, e_oct, k_oct, d_in);
 #pragma unroll
-                for (int e = 0; e < 8; ++e) cs[e] = 1.0f;
-            }
-            load8s(d.signs, e0, d_in, 1, sgn);
+        for (int p = 0; p < NS; ++p) {
+            const bool in = 8 * k_oct[p] < d_in;  // a pair beyond the row has scale 0
+            const float4 v = cols.sg[p];
+            sg[p][0] = in ? v.x : 0.f;
+            sg[p][1] = in ? v.y : 0.f;
+            sg[p][2] = in ? v.z : 0.f;
+            sg[p][3] = in ? v.w : 0.f;
+            e_out[p] = 8 * e_oct[p];
+            float cs[8], sgn[8];
+            cols.unpack(p, e_out[p] < d_in, cs, sgn);
             const float fl = Lay::negated(lane, p) ? -1.0f : 1.0f;
 #pragma unroll
             for (int i = 0; i < 4; ++i)
@@ -618,12 +663,14 @@ __global__ void __launch_bounds__(MAXT, 1) encode2_kernel(const Encode2Args a) {
         first[p] = w | ((32 * w - bit0) << 16);
     }
 
-    chain_wait();
+    // the span is written once, before the batch handle exists
     const int4 span = block_span(a.spans, CALIB ? min(a.one.d_out, QAMW_CALIB_MAX_ROWS) : a.one.d_out);
+    chain_wait();
     for (int m = span.x; m <= span.z; ++m) {
         // The warps regroup when the row length changes: nobody may still be inside the previous
         // matrix (its named barriers and partial sums) when the first warp enters the next one.  The
-        // first pass also waits for the tables.
+        // first pass also waits for the tables.  (The first descriptor ahead of the wait: 0.3 us less for one matrix, but the
+        // compiler then spills more in the row loop, 3092 -> 3253 us for four layers of 13B.)
         __syncthreads();
         if (threadIdx.x == 0) {
             cur = a.descs ? a.descs[m] : a.one;
@@ -645,56 +692,9 @@ __global__ void __launch_bounds__(MAXT, 1) encode2_kernel(const Encode2Args a) {
         const int tg = n_seg * 32;
         const int oct0 = seg * (WE / 8);
 
-        // per-column constants: t_j = s_j sign_j of the columns the thread loads; reciprocal pair scales
-        // (with the butterfly's sign pattern folded in) of the pairs it holds after the rotation
-        f32x2 t[NS][4];
-        float q[NS][4];
-        uint32_t live = 0;  // bit p: the octet that ends up in slot p lies inside the row
-        bool risky = false;
-#pragma unroll
-        for (int p = 0; p < NS; ++p) {
-            const int e0 = 8 * (oct0 + Lay::octet_before(lane, p));
-            float cs[8], sgn[8];
-            if (d.chan_scale) {
-                load8f(d.chan_scale, e0, d_in, 1, 1.0f, cs);
-            } else {
-#pragma unroll
-                for (int e = 0; e < 8; ++e) cs[e] = 1.0f;
-            }
-            load8s(d.signs, e0, d_in, 1, sgn);
-#pragma unroll
-            for (int i = 0; i < 4; ++i) t[p][i] = pack2(cs[2 * i] * sgn[2 * i], cs[2 * i + 1] * sgn[2 * i + 1]);
-            const int k0 = 4 * (oct0 + Lay::octet_after(lane, p));
-            const bool in = k0 < n_pairs;
-            live |= in ? 1u << p : 0u;
-            if (!CALIB) {
-                load4f(d.sigma, k0, n_pairs, 1, 1.0f, q[p]);
-                const float fl = Lay::negated(lane, p) ? -1.0f : 1.0f;
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    // q_k = f32(1 / (double)sigma_k): the correctly rounded f32 reciprocal is the same number
-                    const float r = in ? __frcp_rn(q[p][i]) : 0.f;
-                    // |z| <= q (1 + eps) because |y| <= 1 for a unit row: only a huge reciprocal pair scale can
-                    // carry a point beyond the table's reach
-                    risky |= !(r < 15000.0f);
-                    q[p][i] = fl * r;
-                }
-            }
-        }
-        const uint32_t careful = a.brute || __any_sync(kFull, risky) ? 1u : 0u;
-
+        // The first row is asked for together with the constants where registers are left for it.
+        constexpr bool kEarly = MAXT <= 512;
         const int col0 = seg * WE + 8 * NS * lane;  // first column of this thread
-        const int seg_word0 = 4 * NS * B * seg;     // first packed word of this warp's segment (16 NS B bytes per segment)
-        const bool last_seg = seg == n_seg - 1;
-        double* part_base = &ss_part[0][group * n_seg];
-
-        int parity = 0;
-        double acc[NS][4];
-        int used = 0;
-#pragma unroll
-        for (int p = 0; p < NS; ++p)
-#pragma unroll
-            for (int i = 0; i < 4; ++i) acc[p][i] = 0.0;
         // Raw bits of the thread's elements of one row.  The next row is fetched between the searches of the thread's
         // octets: early enough for its latency to hide, and late enough that its registers are those of the points
         // searched already (with both alive, 72 and 80 registers a thread spilled into the row loop: 58
@@ -728,7 +728,60 @@ __global__ void __launch_bounds__(MAXT, 1) encode2_kernel(const Encode2Args a) {
         };
 #pragma unroll
         for (int i = 0; i < kRaw; ++i) raw[i] = 0u;
-        if (row0 < row_end) fetch(row0);
+        if (kEarly && row0 < row_end) fetch(row0);
+        // per-column constants: t_j = s_j sign_j of the columns the thread loads; reciprocal pair scales
+        // (with the butterfly's sign pattern folded in) of the pairs it holds after the rotation
+        f32x2 t[NS][4];
+        float q[NS][4];
+        uint32_t live = 0;  // bit p: the octet that ends up in slot p lies inside the row
+        bool risky = false;
+        {
+            int e_oct[NS], k_oct[NS];
+#pragma unroll
+            for (int p = 0; p < NS; ++p) {
+                e_oct[p] = oct0 + Lay::octet_before(lane, p);
+                k_oct[p] = oct0 + Lay::octet_after(lane, p);
+            }
+            Columns<NS, !CALIB> cols;
+            cols.load(d.chan_scale, d.signs, d.sigma, e_oct, k_oct, d_in);
+#pragma unroll
+            for (int p = 0; p < NS; ++p) {
+                float cs[8], sgn[8];
+                cols.unpack(p, 8 * e_oct[p] < d_in, cs, sgn);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) t[p][i] = pack2(cs[2 * i] * sgn[2 * i], cs[2 * i + 1] * sgn[2 * i + 1]);
+                const bool in = 8 * k_oct[p] < d_in;
+                live |= in ? 1u << p : 0u;
+                if (!CALIB) {
+                    const float4 v = cols.sg[CALIB ? 0 : p];
+                    const float sg[4] = {v.x, v.y, v.z, v.w};
+                    const float fl = Lay::negated(lane, p) ? -1.0f : 1.0f;
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        // q_k = f32(1 / (double)sigma_k): the correctly rounded f32 reciprocal is the same number
+                        const float r = in ? __frcp_rn(sg[i]) : 0.f;
+                        // |z| <= q (1 + eps) because |y| <= 1 for a unit row: only a huge reciprocal pair scale can
+                        // carry a point beyond the table's reach
+                        risky |= !(r < 15000.0f);
+                        q[p][i] = fl * r;
+                    }
+                }
+            }
+        }
+        if (!kEarly && row0 < row_end) fetch(row0);
+        const uint32_t careful = a.brute || __any_sync(kFull, risky) ? 1u : 0u;
+
+        const int seg_word0 = 4 * NS * B * seg;     // first packed word of this warp's segment (16 NS B bytes per segment)
+        const bool last_seg = seg == n_seg - 1;
+        double* part_base = &ss_part[0][group * n_seg];
+
+        int parity = 0;
+        double acc[NS][4];
+        int used = 0;
+#pragma unroll
+        for (int p = 0; p < NS; ++p)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) acc[p][i] = 0.0;
         for (int row = row0; row < row_end; row += row_step, parity ^= 1) {
             f32x2 P[NS][4];
             if (BF16) {
@@ -864,8 +917,7 @@ __global__ void __launch_bounds__(MAXT, 1) encode2_kernel(const Encode2Args a) {
 // sigma_k of every matrix from the slots of partial sums, one per block that the matrix was spread over.  A block
 // owns 32 pair positions of one matrix; its eight warps each add a contiguous slice of the slots in ascending
 // order, and the slice sums are then added in ascending order: the result does not depend on timing.  Bound by the
-// latency of its loads: with a slot per SM, the 19 of a slice come in two
-// steps.  (Sixteen slices: 1 us less for one matrix, 2 to 10 us more for the batches, whose slots are few.)
+// latency of its loads, which come in one step.  (Sixteen slices: 1 us less for one matrix, 2 to 10 us more for the batches, whose slots are few.)
 constexpr int kFinishSlices = 8;
 __global__ void __launch_bounds__(32 * kFinishSlices) calibrate_finish2_kernel(const MatDesc* descs, const MatDesc one,
                                                                              const unsigned char* calib_base) {
@@ -883,7 +935,7 @@ __global__ void __launch_bounds__(32 * kFinishSlices) calibrate_finish2_kernel(c
     double sum = 0.0, used = 0.0;
     for (int slot = s0 + lane; slot < s1; slot += 32) used += ws[size_t(d.calib_slots) * pair_stride + slot];  // whole numbers: any order
     if (k < n_pairs) {
-        constexpr int U = 10;
+        constexpr int U = 20;  // a slot per SM: one step
         for (int slot = s0; slot < s1; slot += U) {
             double v[U];
 #pragma unroll
