@@ -14,6 +14,7 @@
 #include <algorithm>
 #include <cmath>
 #include <mutex>
+#include <type_traits>
 #include <unordered_map>
 
 #include "qamw_device.cuh"
@@ -175,8 +176,15 @@ struct Gemv2Args {
     float inv_sqrt_b;
 };
 
+// One vector: where the rotation has shared memory of its own, or 0: it uses the ring.  (Four vectors carry it too: the compiler's
+// code for 136 bytes of parameters is 2 to 4 % faster there than for 128; for two vectors it is 4 % slower on small matrices.)
+struct Gemv2ArgsRot : Gemv2Args {
+    int rotate_off;
+};
+
 template <int NVEC>
 struct GemvGeom {
+    typedef std::conditional_t<NVEC == 2, Gemv2Args, Gemv2ArgsRot> Args;
     static constexpr int kThreads = NVEC == 4 ? 320 : NVEC == 2 ? 384 : 512;  // 32 activation registers per thread and vector; warps per scheduler set the register cap
     static constexpr int kDepth = 6;       // staged rows per warp, in pairs: about 40 KB in flight per SM
     static constexpr int kTileRows = 32;   // rows per warp between two block barriers
@@ -312,7 +320,7 @@ __global__ void __launch_bounds__(32 * kRotateWarps) gemv_rotate4_kernel(const G
 
 // BT: bits of an index, or 0 for the widths below 6, read from the arguments
 template <int NVEC, int BT>
-__global__ void __launch_bounds__(GemvGeom<NVEC>::kThreads, 1) gemv2_kernel(const Gemv2Args a) {
+__global__ void __launch_bounds__(GemvGeom<NVEC>::kThreads, 1) gemv2_kernel(const typename GemvGeom<NVEC>::Args a) {
     constexpr int R = 2, D = GemvGeom<NVEC>::kDepth;
     constexpr int BMAX = BT ? BT : 5;
     constexpr bool ODD = BT == 0 || BT % 2;                         // a chunk may start in the middle of a word
@@ -357,24 +365,6 @@ __global__ void __launch_bounds__(GemvGeom<NVEC>::kThreads, 1) gemv2_kernel(cons
         const unsigned char* src = a.packed + ((long long)blockIdx.x + (long long)gridDim.x * g) * a.stride + seg_off;
         int off = int(reinterpret_cast<uintptr_t>(src) & 15);  // of the current row from the 16-byte boundary below it
         f32x2 xr[NVEC][16];
-        if (n_rows > 0) {
-            if constexpr (NVEC == 4) {
-                const bool valid = 32 * slice + lane < a.n_chunks;
-#pragma unroll
-                for (int v = 0; v < NVEC; ++v)
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        const float4 q = valid ? __ldcg(a.xt + xt_index(a, slice, v, j, lane)) : make_float4(0.f, 0.f, 0.f, 0.f);
-                        xr[v][2 * j] = pack2(q.x, q.y);
-                        xr[v][2 * j + 1] = pack2(q.z, q.w);
-                    }
-            } else {
-                // the first rows come to the L2 while the ring's memory serves the rotation
-                for (int i = 0; i < min(n_rows, D) && lane * 128 < seg_len + 15; ++i)
-                    asm volatile("prefetch.global.L2 [%0];" ::"l"(src + i * src_step + min(lane * 128, seg_len - 1)));
-                rotate_slice<NVEC>(a, slice, 0, stage, lane, xr);
-            }
-        }
         // the ring of a warp: D staged rows of its slice, one commit group per R rows (empty past the end)
         int issued = 0;
         auto issue = [&]() {
@@ -393,7 +383,35 @@ __global__ void __launch_bounds__(GemvGeom<NVEC>::kThreads, 1) gemv2_kernel(cons
             }
             cp_async_commit();
         };
-        for (int i = 0; i < D / R - 1; ++i) issue();
+        auto fill = [&]() {
+            for (int i = 0; i < D / R - 1; ++i) issue();
+        };
+        bool early = NVEC == 4;  // the ring is free of the rotation: the first rows travel meanwhile
+        unsigned char* turn = stage;
+        if constexpr (NVEC == 1) {
+            early = a.rotate_off > 0;
+            if (early) turn = smem + a.rotate_off + warp * kRotateStage;
+        }
+        if (early) fill();
+        if (n_rows > 0) {
+            if constexpr (NVEC == 4) {
+                const bool valid = 32 * slice + lane < a.n_chunks;
+#pragma unroll
+                for (int v = 0; v < NVEC; ++v)
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        const float4 q = valid ? __ldcg(a.xt + xt_index(a, slice, v, j, lane)) : make_float4(0.f, 0.f, 0.f, 0.f);
+                        xr[v][2 * j] = pack2(q.x, q.y);
+                        xr[v][2 * j + 1] = pack2(q.z, q.w);
+                    }
+            } else {
+                if (!early)  // the first rows come to the L2 while the ring's memory serves the rotation
+                    for (int i = 0; i < min(n_rows, D) && lane * 128 < seg_len + 15; ++i)
+                        asm volatile("prefetch.global.L2 [%0];" ::"l"(src + i * src_step + min(lane * 128, seg_len - 1)));
+                rotate_slice<NVEC>(a, slice, 0, turn, lane, xr);
+            }
+        }
+        if (!early) fill();
 
         for (int tile = 0; tile < n_tiles; ++tile) {
             float* ps = ps_base + (tile & 1) * (S_par * TI * NVEC);  // [slice][row of the tile][vector]
@@ -518,7 +536,7 @@ int gemv_raise_smem(const void* kernel) {
 }
 
 template <int NVEC, int BT>
-int launch_gemv2_b(const Gemv2Args& a, int blocks, int threads, size_t smem, cudaStream_t st) {
+int launch_gemv2_b(const typename GemvGeom<NVEC>::Args& a, int blocks, int threads, size_t smem, cudaStream_t st) {
     int rc = gemv_raise_smem(reinterpret_cast<const void*>(&gemv2_kernel<NVEC, BT>));
     if (rc) return rc;
     return gemv_check("gemv2_kernel", launch_chained(gemv2_kernel<NVEC, BT>, blocks, threads, smem, st, a));
@@ -533,13 +551,23 @@ int launch_gemv2(const Gemv2Args& a, int sms, cudaStream_t st) {
     const int blocks = std::max(1, std::min(sms, a.d_out));
     const int n_b = (a.d_out + blocks - 1) / blocks;  // rows of a block
     const int G = std::max(1, std::min(kWarps / S_par, n_b));
-    Gemv2Args b = a;
+    typename GemvGeom<NVEC>::Args b{};
+    static_cast<Gemv2Args&>(b) = a;
     b.s_par = S_par;
     b.log2c = pick_copies(a.K, (long long)n_b * (a.d_in / 64), size_t(128) * 1024);
     const int threads = 32 * S_par * G;
     const size_t sums = size_t(2) * S_par * GemvGeom<NVEC>::kTileRows * G * NVEC * sizeof(float);
-    const size_t smem = (size_t(a.K) * 8 << b.log2c) + size_t(S_par * G) * GemvGeom<NVEC>::kDepth * a.stage_bytes + sums;
+    size_t smem = (size_t(a.K) * 8 << b.log2c) + size_t(S_par * G) * GemvGeom<NVEC>::kDepth * a.stage_bytes + sums;
     if (smem > kSmemLimit) return QAMW_ERR_NOMEM;
+    // One vector: where there is room beside the ring (a small matrix keeps few copies of the codebook) the rotation leaves the
+    // ring alone: 2048 x 5632 10.40 -> 10.33 us.  Two vectors lose by it (11.96 -> 12.47), four are rotated elsewhere.
+    const size_t rotate_at = (smem + 15) & ~size_t(15), rotate = size_t(S_par * G) * kRotateStage;
+    if constexpr (NVEC == 1) {
+        if (rotate_at + rotate <= kSmemLimit) {
+            b.rotate_off = int(rotate_at);
+            smem = rotate_at + rotate;
+        }
+    }
     switch (a.B) {
         case 6: return launch_gemv2_b<NVEC, 6>(b, blocks, threads, smem, st);
         case 7: return launch_gemv2_b<NVEC, 7>(b, blocks, threads, smem, st);
