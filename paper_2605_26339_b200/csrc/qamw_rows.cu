@@ -366,6 +366,7 @@ __global__ void __launch_bounds__(32 * kDecodeWarps, 1) decode2_kernel(const Dec
         }
         Columns<NS, true> cols;
         cols.load(d.chan_scale, d.signs, d.sigma, e_oct, k_oct, d_in);
+        const f32x2 c2 = pack2(a.inv_sqrt_b, a.inv_sqrt_b);
 #pragma unroll
         for (int p = 0; p < NS; ++p) {
             const bool in = 8 * k_oct[p] < d_in;  // a pair beyond the row has scale 0
@@ -378,10 +379,15 @@ __global__ void __launch_bounds__(32 * kDecodeWarps, 1) decode2_kernel(const Dec
             float cs[8], sgn[8];
             cols.unpack(p, e_out[p] < d_in, cs, sgn);
             const float fl = Lay::negated(lane, p) ? -1.0f : 1.0f;
+            uint32_t off = 0;  // a scale that quotient2 does not take
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
-                mcol[p][i] = pack2(fl * __fdiv_rn(sgn[2 * i] * a.inv_sqrt_b, cs[2 * i]),
-                                   fl * __fdiv_rn(sgn[2 * i + 1] * a.inv_sqrt_b, cs[2 * i + 1]));
+            for (int i = 0; i < 8; ++i) off |= uint32_t(__float_as_uint(cs[i]) - 0x21800000u >= 0x3c000000u);  // [2^-60, 2^60)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                f32x2 v = quotient2(c2, cs[2 * i], cs[2 * i + 1]);
+                if (off) v = pack2(library_quotient(a.inv_sqrt_b, cs[2 * i]), library_quotient(a.inv_sqrt_b, cs[2 * i + 1]));
+                mcol[p][i] = mul2(pack2(fl * sgn[2 * i], fl * sgn[2 * i + 1]), v);
+            }
         }
         __nv_bfloat16* orow = static_cast<__nv_bfloat16*>(d.w_hat) + (long long)row0 * d_in;
         const long long out_step = (long long)row_step * d_in;

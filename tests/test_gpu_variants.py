@@ -280,3 +280,59 @@ def test_outputs_that_share_memory_until_they_are_written(orc):
     packed, norm = torch.zeros_like(e["packed"]), torch.zeros_like(e["norm"])
     q.encode(e["W"], e["p"], e["s"], e["signs"], e["sigma"], e["cb"], torch._lazy_clone(packed), torch._lazy_clone(norm))
     assert not packed.any() and not norm.any()
+
+
+def test_quotients_of_the_column_factors(tmp_path):
+    """quotient2 equals the correctly rounded division for every significand of the divisor, at both ends of the range that it is
+    used for and in its middle, and for the numerator of every block size."""
+    import os
+    import subprocess
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    src = tmp_path / "quotient.cu"
+    src.write_text(r'''
+#include <cmath>
+#include <cstdio>
+#include "qamw_device.cuh"
+__global__ void check(float a, int exponent, unsigned long long* wrong) {
+    const unsigned m = 2u * (blockIdx.x * blockDim.x + threadIdx.x);  // 2^23 significands, two at a time
+    const float b0 = __uint_as_float((unsigned(exponent + 127) << 23) | m), b1 = __uint_as_float((unsigned(exponent + 127) << 23) | (m + 1u));
+    float q0, q1;
+    unpack2(quotient2(pack2(a, a), b0, b1), q0, q1);
+    if (q0 != __fdiv_rn(a, b0) || q1 != __fdiv_rn(a, b1)) atomicAdd(wrong, 1ull);
+}
+int main() {
+    unsigned long long* wrong;
+    if (cudaMallocManaged(&wrong, 8) != cudaSuccess) return 1;
+    *wrong = 0;
+    for (int log2b = 1; log2b <= 10; ++log2b)
+        for (int e : {-60, -5, -1, 0, 1, 4, 59}) check<<<(1 << 22) / 256, 256>>>(float(1.0 / std::sqrt(double(1 << log2b))), e, wrong);
+    if (cudaDeviceSynchronize() != cudaSuccess) return 1;
+    std::printf("%llu", *wrong);
+}
+''')
+    exe = tmp_path / "quotient"
+    from paper_2605_26339_b200 import build
+    subprocess.run([build._nvcc(), "-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-std=c++17", "-I",
+                    os.path.join(root, "paper_2605_26339_b200", "csrc"), "-o", str(exe), str(src)], check=True)
+    assert subprocess.run([str(exe)], check=True, capture_output=True, text=True).stdout == "0"
+
+
+@pytest.mark.parametrize("scale", [1.0, 2.0 ** -61, 2.0 ** 61])
+def test_decode_with_channel_scales_off_the_usual_range(scale):
+    """Channel scales below and above the range of quotient2, alone and among usual ones: as the general kernels, bit for bit."""
+    d_out, d_in, K = 37, 1056, 64
+    g = torch.Generator(device=DEV)
+    g.manual_seed(3)
+    cb = q.Codebook(q.train_codebook(K, n_samples=4096, seed=1, max_iters=3)[0])
+    s = torch.rand(d_in, generator=g, device=DEV) + 0.5
+    s[::7] *= scale
+    signs = torch.from_numpy(q.make_signs(q.DEFAULT_SIGN_SEED, d_in)).to(DEV)
+    sigma = torch.rand(d_in // 2, generator=g, device=DEV) + 0.1
+    p = q.make_params(torch.empty((d_out, d_in), dtype=torch.bfloat16, device=DEV), d_out, d_in, 32, K)
+    packed = torch.randint(0, 256, (d_out, p.packed_row_stride), generator=g, device=DEV, dtype=torch.uint8)
+    norm = torch.rand(d_out, generator=g, device=DEV)
+    out = [torch.empty((d_out, d_in), dtype=torch.bfloat16, device=DEV) for _ in range(2)]
+    for o, flags in zip(out, (0, q.FLAG_GENERAL_KERNELS)):
+        p.flags = flags
+        q.decode(packed, norm, s, signs, sigma, cb, p, o)
+    assert torch.equal(out[0].view(torch.int16), out[1].view(torch.int16))
