@@ -295,10 +295,9 @@ __global__ void __launch_bounds__(32 * kDecodeWarps, 1) decode2_kernel(const Dec
 
     chain_release();
     fill_codebook_copies(reinterpret_cast<float2*>(smem), a.codebook, a.K, a.log2c, true);
-    // spans and descriptors are written once, before the batch handle exists
+    // spans and descriptors are written once, before the batch handle exists: what follows from them comes before the wait
     const int4 span = block_span(a.spans, a.one.d_out);
     __syncthreads();
-    chain_wait();
 
     // where this thread's index bits sit inside a staged segment: two runs (the lower and the upper
     // physical slots), each 4 B TOP bits long
@@ -310,6 +309,7 @@ __global__ void __launch_bounds__(32 * kDecodeWarps, 1) decode2_kernel(const Dec
         run_shift[x] = bit0 & 31u;
     }
 
+    bool waited = false;
     for (int m = span.x; m <= span.z; ++m) {
         const MatDesc& d = a.descs ? a.descs[m] : a.one;
         const int d_in = d.d_in, n_pairs = d_in >> 1;
@@ -332,6 +332,8 @@ __global__ void __launch_bounds__(32 * kDecodeWarps, 1) decode2_kernel(const Dec
         uint32_t off = ALIGNED ? 0u : uint32_t(reinterpret_cast<uintptr_t>(src) & 15);  // of the row decoded next from the boundary below it
         const uint32_t off_step = ALIGNED ? 0u : uint32_t(src_step & 15);
         const bool copy0 = (lane << 4) < seg_len, copy1 = (lane << 4) + 512 < seg_len;  // two pieces of 16 bytes per lane, no loop
+        if (!waited) chain_wait();
+        waited = true;
         int issued = 0;
         auto issue_row = [&]() {  // one commit group per row, empty past the end
             if (issued < n_rows) {
