@@ -1044,6 +1044,13 @@ __device__ __forceinline__ void dist_cursor_open(DistCursor& c, int d_out, int d
     c.row = chunk * kDistRows;
     c.r1 = min(d_out, c.row + kDistRows);
 }
+// A bf16 number (in the upper half of `bits`) times 2^-896 as a double, for finite ones exactly, subnormal ones included: sign and
+// exponent field moved to their places.  The factor goes into the fused multiply-add that subtracts it.  The conversion from
+// f32 runs on a pipe of 16 lanes a clock, which two per element kept busy to 61 %; one of the two is done with two integer instructions
+// now.  An infinity or a NaN comes out as 2^128 or more: kDistWild is there to see it.
+__device__ __forceinline__ double dist_scaled(uint32_t bits) { return __hiloint2double((int(bits) >> 3) & int(0x8fffffffu), 0); }
+constexpr double kDistScale = 0x1p896;
+constexpr double kDistWild = 0x1p249;  // a column sum this large, or not a number, is taken again with ordinary conversions
 __device__ __forceinline__ void dist_items_stream(const __nv_bfloat16* W, long long w_row_stride, const __nv_bfloat16* What,
                                                   const float* act_rms, int d_out, int d_in, long long first,
                                                   long long last, long long step, double& s0, double& s1, double& s2,
@@ -1090,8 +1097,8 @@ __device__ __forceinline__ void dist_items_stream(const __nv_bfloat16* W, long l
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 const double w0 = double(__uint_as_float(ww[i] << 16)), w1 = double(__uint_as_float(ww[i] & 0xffff0000u));
-                const double d0 = w0 - double(__uint_as_float(hw[i] << 16));
-                const double d1 = w1 - double(__uint_as_float(hw[i] & 0xffff0000u));
+                const double d0 = fma(dist_scaled(hw[i] << 16), -kDistScale, w0);
+                const double d1 = fma(dist_scaled(hw[i] & 0xffff0000u), -kDistScale, w1);
                 E[2 * i] = fma(d0, d0, E[2 * i]);
                 Q[2 * i] = fma(w0, w0, Q[2 * i]);
                 E[2 * i + 1] = fma(d1, d1, E[2 * i + 1]);
@@ -1099,6 +1106,24 @@ __device__ __forceinline__ void dist_items_stream(const __nv_bfloat16* W, long l
             }
         }
         if (++cons.row == cons.r1) {  // end of the item: weight the column sums and start over
+            bool wild = false;
+#pragma unroll
+            for (int e = 0; e < 8; ++e) wild = wild || !(E[e] < kDistWild) || !(Q[e] < kDistWild);
+            if (wild) {  // the same additions; a reconstruction that is not finite makes |d| at least 2^127 or |w| at least 2^125
+#pragma unroll
+                for (int e = 0; e < 8; ++e) E[e] = Q[e] = 0.0;
+#pragma unroll 1
+                for (int row = (cons.r1 - 1) / kDistRows * kDistRows; row < cons.r1; ++row) {
+                    float w[8], h[8];
+                    dist_load<true>(W, w_row_stride, What, row, cons.j0, d_in, 1, w, h);
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) {
+                        const double wd = double(w[e]), d = wd - double(h[e]);
+                        E[e] = fma(d, d, E[e]);
+                        Q[e] = fma(wd, wd, Q[e]);
+                    }
+                }
+            }
 #pragma unroll
             for (int e = 0; e < 8; ++e) {
                 const double r2 = double(rj[e]) * double(rj[e]);

@@ -336,3 +336,42 @@ def test_decode_with_channel_scales_off_the_usual_range(scale):
         p.flags = flags
         q.decode(packed, norm, s, signs, sigma, cb, p, o)
     assert torch.equal(out[0].view(torch.int16), out[1].view(torch.int16))
+
+
+@pytest.mark.parametrize("kind", ["ordinary", "subnormal", "huge", "inf", "nan", "inf and huge"])
+@pytest.mark.parametrize("batched", [False, True])
+def test_distortion_of_numbers_at_the_ends_of_the_range(kind, batched):
+    """The four sums against doubles for reconstructions with subnormal, huge and non-finite entries, also beside weights as large."""
+    d_out, d_in = 37, 1048
+    g = torch.Generator(device=DEV)
+    g.manual_seed(4)
+    W = torch.randn((d_out, d_in), generator=g, device=DEV).to(torch.bfloat16)
+    h = (W.float() * (1 + 0.1 * torch.randn((d_out, d_in), generator=g, device=DEV))).to(torch.bfloat16)
+    act = torch.rand(d_in, generator=g, device=DEV) + 0.5
+    big = 3.3895313892515355e38  # the largest bf16
+    if kind == "subnormal":
+        W, h = (W.float() * 2.0 ** -130).to(torch.bfloat16), (h.float() * 2.0 ** -130).to(torch.bfloat16)
+        assert (h != 0).any() and h.float().abs().max() < 2.0 ** -126
+    elif kind == "huge":
+        W[5, 7], h[5, 7], h[20, 100], W[36, 1047] = big, -big, big, -big
+    elif kind == "inf":
+        h[3, 9], h[30, 1040] = float("inf"), -float("inf")
+    elif kind == "nan":
+        h[17, 511] = float("nan")
+    elif kind == "inf and huge":
+        W[3, 9], h[3, 9] = big, float("inf")
+    p = q.make_params(W, d_out, d_in, 8, 64)
+    out = torch.zeros(4, dtype=torch.float64, device=DEV)
+    if batched:
+        cb = q.Codebook(q.train_codebook(64, n_samples=4096, seed=1, max_iters=3)[0])
+        signs = torch.from_numpy(q.make_signs(q.DEFAULT_SIGN_SEED, d_in)).to(DEV)
+        sigma = torch.ones(d_in // 2, device=DEV)
+        packed = torch.zeros((d_out, p.packed_row_stride), dtype=torch.uint8, device=DEV)
+        norm = torch.ones(d_out, device=DEV)
+        q.Batch([q.make_matrix(p, W, None, signs, sigma, act, packed, norm, h, out)], cb).distortion()
+    else:
+        q.distortion(W, h, act, p, out)
+    w, r2 = W.double(), act.double() ** 2
+    e2 = (w - h.double()) ** 2
+    want = torch.stack([e2.sum(), (w * w).sum(), (r2 * e2).sum(), (r2 * w * w).sum()])
+    assert torch.allclose(out, want, rtol=1e-12, atol=0.0, equal_nan=True), (out, want)
