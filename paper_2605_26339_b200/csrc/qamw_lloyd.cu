@@ -1327,29 +1327,55 @@ extern "C" int qamw_train_codebook_gpu(int K, uint64_t n_samples, uint64_t seed,
     const int chunk = std::min(kMaxChunk, std::max(kMinChunk, int(((n + kManyChunks - 1) / kManyChunks + 31) / 32 * 32)));
     const int n_chunks = int((n + chunk - 1) / chunk), n_tiles = int((n + kTile - 1) / kTile);
     const int bins = std::max(K, 256);
-    // one allocation, cut into pieces
-    size_t bytes = 0;
-    auto piece = [&](size_t b) {
-        const size_t at = bytes;
-        bytes += (b + 255) & ~size_t(255);
-        return at;
-    };
-    const bool incremental = K >= kIncrementalK && n <= kIncrementalSamples && n / K <= 1024 + 2 * unsigned(K);
+    // One allocation, cut into pieces.  Incremental updates need about twice as much again: where that much is not to be had the
+    // passes in full remain, which give the same bits.
+    bool incremental = K >= kIncrementalK && n <= kIncrementalSamples && n / K <= 1024 + 2 * unsigned(K);
     const int room = 64 + int(n / unsigned(K) / 4);
-    const size_t slots = incremental ? n + n / 4 + size_t(room) * (size_t(K) + 1) : 0, tiles = incremental ? size_t(n_tiles) : 0, cells = incremental ? size_t(K) : 0;
-    const size_t o_gen = piece(samples_dev ? 0 : sizeof(double2) * n), o_sorted = piece(sizeof(double2) * n),
-                 o_cell = piece(sizeof(double2) * std::max<size_t>(n, slots)), o_values = piece(sizeof(double2) * slots), o_ids = piece(sizeof(int) * n), o_assign = piece(sizeof(int) * n),
-                 o_hist = piece(sizeof(int) * size_t(bins) * n_chunks), o_start = piece(sizeof(int) * (size_t(bins) + 1)),
-                 o_cb = piece(2 * sizeof(double2) * K), o_cb32 = piece(2 * sizeof(float2) * K), o_err = piece(sizeof(double) * n_tiles),
-                 o_box = piece(sizeof(TileBox) * n_tiles * kBoxes), o_state = piece(sizeof(TrainState)), o_scale = piece(sizeof(float));
-    const size_t o_cur = piece(2 * (incremental ? n : 0)), o_near = piece(2 * tiles * kNearMost), o_near_n = piece(4 * tiles), o_gap = piece(4 * tiles),
-                 o_members = piece(4 * 2 * slots), o_cells = piece(4 * (7 * cells + 1)), o_changes = piece(4 * 2 * cells * kChanges);
+    size_t bytes, slots, o_gen, o_sorted, o_cell, o_values, o_ids, o_assign, o_hist, o_start, o_cb, o_cb32, o_err, o_box, o_state, o_scale;
+    size_t o_cur, o_near, o_near_n, o_gap, o_members, o_cells, o_changes;
+    auto lay_out = [&]() {
+        bytes = 0;
+        auto piece = [&](size_t b) {
+            const size_t at = bytes;
+            bytes += (b + 255) & ~size_t(255);
+            return at;
+        };
+        slots = incremental ? n + n / 4 + size_t(room) * (size_t(K) + 1) : 0;
+        const size_t tiles = incremental ? size_t(n_tiles) : 0, cells = incremental ? size_t(K) : 0;
+        o_gen = piece(samples_dev ? 0 : sizeof(double2) * n);
+        o_sorted = piece(sizeof(double2) * n);
+        o_cell = piece(sizeof(double2) * std::max<size_t>(n, slots));
+        o_values = piece(sizeof(double2) * slots);
+        o_ids = piece(sizeof(int) * n);
+        o_assign = piece(sizeof(int) * n);
+        o_hist = piece(sizeof(int) * size_t(bins) * n_chunks);
+        o_start = piece(sizeof(int) * (size_t(bins) + 1));
+        o_cb = piece(2 * sizeof(double2) * K);
+        o_cb32 = piece(2 * sizeof(float2) * K);
+        o_err = piece(sizeof(double) * n_tiles);
+        o_box = piece(sizeof(TileBox) * n_tiles * kBoxes);
+        o_state = piece(sizeof(TrainState));
+        o_scale = piece(sizeof(float));
+        o_cur = piece(2 * (incremental ? n : 0));
+        o_near = piece(2 * tiles * kNearMost);
+        o_near_n = piece(4 * tiles);
+        o_gap = piece(4 * tiles);
+        o_members = piece(4 * 2 * slots);
+        o_cells = piece(4 * (7 * cells + 1));
+        o_changes = piece(4 * 2 * cells * kChanges);
+    };
     unsigned char* base = nullptr;
-    cudaError_t e = cudaSuccess;
-    if (cudaMemPool_t pool = scratch_pool(true)) {
-        e = cudaMallocFromPoolAsync(reinterpret_cast<void**>(&base), bytes, pool, nullptr);
-    } else {
-        e = cudaMallocAsync(reinterpret_cast<void**>(&base), bytes, nullptr);
+    const cudaMemPool_t pool = scratch_pool(true);
+    auto take = [&]() {
+        lay_out();
+        void** const to = reinterpret_cast<void**>(&base);
+        return pool ? cudaMallocFromPoolAsync(to, bytes, pool, nullptr) : cudaMallocAsync(to, bytes, nullptr);
+    };
+    cudaError_t e = take();
+    if (e == cudaErrorMemoryAllocation && incremental) {
+        cudaGetLastError();
+        incremental = false;
+        e = take();
     }
     if (e != cudaSuccess) {
         set_cuda_error("qamw_train_codebook_gpu: cudaMallocAsync", int(e));

@@ -167,3 +167,23 @@ def test_scratch_kept_between_calls_is_bounded_and_given_back():
     q.release_scratch()
     assert np.array_equal(q.train_codebook_gpu(256, 1 << 20, 0, 2)["codebook"], first["codebook"])
     q.release_scratch()
+
+
+def test_little_device_memory():
+    """A call with memory for the passes in full but not for incremental updates: the same result, and the next one as before."""
+    K, n = 2048, 1 << 22  # 190 MB, or 420
+    g = torch.Generator(device=DEV)
+    g.manual_seed(7)
+    z = torch.randn((n, 2), generator=g, device=DEV, dtype=torch.float64)
+    want = q.train_codebook_gpu(K, max_iters=12, rel_tol=0.0, samples=z)
+    q.release_scratch()
+    torch.cuda.empty_cache()
+    hold = torch.empty(torch.cuda.mem_get_info()[0] - (300 << 20), dtype=torch.uint8, device=DEV)
+    try:
+        got = q.train_codebook_gpu(K, max_iters=12, rel_tol=0.0, samples=z)
+    finally:
+        del hold
+        torch.cuda.empty_cache()
+    for out in (got, q.train_codebook_gpu(K, max_iters=12, rel_tol=0.0, samples=z)):
+        assert np.array_equal(out["codebook"], want["codebook"]) and np.array_equal(out["trace"], want["trace"])
+    q.release_scratch()
