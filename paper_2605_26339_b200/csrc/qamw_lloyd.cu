@@ -1329,7 +1329,7 @@ extern "C" int qamw_train_codebook_gpu(int K, uint64_t n_samples, uint64_t seed,
     const int bins = std::max(K, 256);
     // One allocation, cut into pieces.  Incremental updates need about twice as much again: where that much is not to be had the
     // passes in full remain, which give the same bits.
-    bool incremental = K >= kIncrementalK && n <= kIncrementalSamples && n / K <= 1024 + 2 * unsigned(K);
+    bool incremental = K >= kIncrementalK && n <= kIncrementalSamples && n / K <= 1024 + 2 * unsigned(K) && max_iters >= kFullFirst;
     const int room = 64 + int(n / unsigned(K) / 4);
     size_t bytes, slots, o_gen, o_sorted, o_cell, o_values, o_ids, o_assign, o_hist, o_start, o_cb, o_cb32, o_err, o_box, o_state, o_scale;
     size_t o_cur, o_near, o_near_n, o_gap, o_members, o_cells, o_changes;

@@ -187,3 +187,19 @@ def test_little_device_memory():
     for out in (got, q.train_codebook_gpu(K, max_iters=12, rel_tol=0.0, samples=z)):
         assert np.array_equal(out["codebook"], want["codebook"]) and np.array_equal(out["trace"], want["trace"])
     q.release_scratch()
+
+
+@pytest.mark.parametrize("iters,needed", [(7, 43), (8, 110)])
+def test_scratch_of_a_call_without_incremental_updates(orc, iters, needed):
+    """Eight passes in full come first: a call of up to seven updates (and the last assignment) takes memory for these alone,
+    43 MB at 2^20 samples and K = 2048; one that goes on takes 110.  (A pool grows by 32 MB at a time.)"""
+    K, n = 2048, 1 << 20
+    z = torch.from_numpy(orc.gauss_pairs(4, n)).to(DEV)
+    q.train_codebook_gpu(K, max_iters=9, rel_tol=0.0, samples=z[: 1 << 14])
+    q.release_scratch()
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    q.train_codebook_gpu(K, max_iters=iters, rel_tol=0.0, samples=z)
+    kept = free - torch.cuda.mem_get_info()[0]
+    q.release_scratch()
+    assert needed <= kept >> 20 <= needed + 32
