@@ -113,7 +113,8 @@ int qamw_train_codebook(int K, uint64_t n_samples, uint64_t seed, int max_iters,
  * mean squared distance before every update; seconds_out: wall time of the call.
  * Synchronous; allocates its device scratch itself (about 45 bytes per sample, 16 more for generated samples; for
  * K >= 64, up to 1024 + 2 K samples per codeword and max_iters >= 8 about 100 per sample, or 45 where that is not to
- * be had), from a pool that keeps up to 256 MB of it on the device for the next call: qamw_release_scratch gives that back.
+ * be had), from a pool that keeps up to 256 MB of it on the device for the next call (640 MB once a call with the larger
+ * amount has needed more than 256): qamw_release_scratch gives that back.
  * n_samples < 2^31. */
 int qamw_train_codebook_gpu(int K, uint64_t n_samples, uint64_t seed, const double* samples_dev, int max_iters,
                             double rel_tol, float* codebook_out, double* train_mse_out, int* iters_out,

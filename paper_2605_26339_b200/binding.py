@@ -180,7 +180,7 @@ def train_codebook_gpu(K: int, n_samples: int = 1 << 20, seed: int = 0, max_iter
 
 
 def release_scratch():
-    """Gives the device memory that training keeps for its next call (up to 256 MB per device) back to the driver."""
+    """Gives the device memory that training keeps for its next call (up to 256 or 640 MB per device, see qamw.h) back to the driver."""
     _check("qamw_release_scratch", lib().qamw_release_scratch())
 
 

@@ -1274,11 +1274,15 @@ __global__ void init_kernel(const double2* samples, int K, double2* codebook, fl
     codebook32[c] = make_float2(float(root2 * z.x), float(root2 * z.y));
 }
 
-// Where the scratch memory of a call comes from: a pool per device that keeps up to 256 MB between calls (the
-// default size takes 115 MB; with cudaMalloc and cudaFree a call cost 3 ms more) until qamw_release_scratch gives it
-// back.  NULL if the device has no pools of its own, or, without `create`, if there is none yet.
+// Where the scratch memory of a call comes from: a pool per device that keeps up to 256 MB between calls until
+// qamw_release_scratch gives them back.  NULL if the device has no pools of its own, or, without `create`, if there is
+// none yet.  256 MB are passes in full on 6 million samples; incremental updates on as many take 600, and a call that makes them and
+// needs more than 256 raises the limit to 640.  What a call takes from the driver and gives back costs it time: K = 2048, 100
+// updates, 3, 4 and 6 million samples 13.6, 18.3 and 28.7 ms with 256 MB kept, 12.7, 16.2 and 24.1 with all (quiet host; up to 0.8 s a
+// call where others keep the driver busy).  Beyond that incremental updates still win (8 million: 35.5 against 52.7 in full).
 constexpr int kMaxDevices = 64;
-constexpr size_t kKeepBytes = size_t(256) << 20;
+constexpr size_t kKeepBytes = size_t(256) << 20, kKeepMore = size_t(640) << 20;
+void keep_at_most(cudaMemPool_t pool, uint64_t bytes) { cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &bytes); }
 cudaMemPool_t scratch_pool(bool create) {
     static std::mutex mu;
     static cudaMemPool_t pools[kMaxDevices] = {};
@@ -1295,8 +1299,7 @@ cudaMemPool_t scratch_pool(bool create) {
             cudaGetLastError();
             return nullptr;
         }
-        uint64_t keep = kKeepBytes;
-        cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep);
+        keep_at_most(p, kKeepBytes);
         pools[dev] = p;
     }
     return pools[dev];
@@ -1307,6 +1310,7 @@ cudaMemPool_t scratch_pool(bool create) {
 extern "C" int qamw_release_scratch(void) {
     cudaMemPool_t pool = scratch_pool(false);
     if (!pool) return QAMW_OK;
+    keep_at_most(pool, kKeepBytes);
     cudaError_t e = cudaStreamSynchronize(nullptr);  // the last call's scratch is freed in the order of this stream
     if (e == cudaSuccess) e = cudaMemPoolTrimTo(pool, 0);
     if (e != cudaSuccess) {
@@ -1381,6 +1385,7 @@ extern "C" int qamw_train_codebook_gpu(int K, uint64_t n_samples, uint64_t seed,
         set_cuda_error("qamw_train_codebook_gpu: cudaMallocAsync", int(e));
         return QAMW_ERR_CUDA;
     }
+    if (pool && incremental && bytes > kKeepBytes) keep_at_most(pool, kKeepMore);
     struct Free {
         void* p;
         size_t bytes;

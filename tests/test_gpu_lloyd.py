@@ -150,7 +150,7 @@ def test_samples_still_on_their_way_on_another_stream():
 
 
 def test_scratch_kept_between_calls_is_bounded_and_given_back():
-    """Device memory that training holds on to: at most 256 MB whatever a call needed, none after release_scratch, and
+    """Device memory that training with passes in full holds on to: at most 256 MB whatever a call needed, none after release_scratch, and
     the next call works as before."""
     q.train_codebook_gpu(16, 1 << 12, 0, 1)  # contexts, modules
     q.release_scratch()
@@ -203,3 +203,27 @@ def test_scratch_of_a_call_without_incremental_updates(orc, iters, needed):
     kept = free - torch.cuda.mem_get_info()[0]
     q.release_scratch()
     assert needed <= kept >> 20 <= needed + 32
+
+
+def test_scratch_of_incremental_updates_is_kept():
+    """Calls of up to some 6 million samples find their scratch memory in the pool the next time; larger ones leave at most 640 MB
+    there, and after release_scratch the limit of passes in full holds again."""
+    K, n = 2048, 1 << 22  # 401 MB
+    g = torch.Generator(device=DEV)
+    g.manual_seed(7)
+    z = torch.randn((9 << 20, 2), generator=g, device=DEV, dtype=torch.float64)  # 9 million: 880 MB
+    q.train_codebook_gpu(K, max_iters=9, rel_tol=0.0, samples=z[: 1 << 14])
+    q.release_scratch()
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+
+    def kept(K, n, iters):
+        q.train_codebook_gpu(K, max_iters=iters, rel_tol=0.0, samples=z[:n])
+        return (free - torch.cuda.mem_get_info()[0]) >> 20
+
+    assert 401 <= kept(K, n, 9) <= 640 and 401 <= kept(K, n, 9) <= 640
+    assert kept(K, 9 << 20, 9) <= 644
+    q.release_scratch()
+    assert kept(256, 8 << 20, 1) <= 260
+    q.release_scratch()
+    assert (free - torch.cuda.mem_get_info()[0]) >> 20 <= 4
