@@ -780,11 +780,10 @@ constexpr int kNear = 64;      // codewords in a neighbourhood, if its box is no
 constexpr int kNearMost = 1024;  // such a box has up to this many
 // Neighbourhoods are listed anew every so many updates (5 and 11 full passes at the start, 8 or 16 updates to a list: within 2 %).
 constexpr int kEarly = 24, kNearEarly = 4, kNearLate = 8;
-// Cells of up to 1024 + 2 K samples on average, from 64 cells on: larger and fewer cells leave the merge to a few blocks, and their chains take
+// Cells of up to 1024 + 2 K samples on average (37.7 million at K = 4096: slots are numbered in 32 bits), from 64 cells on: larger and fewer cells leave the merge to a few blocks, and their chains take
 // the time either way.  ms a call in full and incremental: K = 64 on 70001 samples 3.9, 3.2; 128 on 70001 3.7, 2.5, on 2^18 5.2, 5.7 (5.2 in full
 // is kept); 256 on 2^18 4.9, 3.7, on 2^20 10.6, 12.3; 512 on 2^20 9.5, 7.6; 2048 on 2^20 8.6, 5.2; 4096 on 2^20 10.9, 6.9.
 constexpr int kIncrementalK = 64;
-constexpr unsigned long long kIncrementalSamples = 1ull << 26;
 constexpr int kChanges = 512;  // arrivals, and departures, of a cell in one pass
 
 // Cells as the full pass left them: members and room to grow by a quarter and `room`.
@@ -1333,7 +1332,7 @@ extern "C" int qamw_train_codebook_gpu(int K, uint64_t n_samples, uint64_t seed,
     const int bins = std::max(K, 256);
     // One allocation, cut into pieces.  Incremental updates need about twice as much again: where that much is not to be had the
     // passes in full remain, which give the same bits.
-    bool incremental = K >= kIncrementalK && n <= kIncrementalSamples && n / K <= 1024 + 2 * unsigned(K) && max_iters >= kFullFirst;
+    bool incremental = K >= kIncrementalK && n / K <= 1024 + 2 * unsigned(K) && max_iters >= kFullFirst;
     const int room = 64 + int(n / unsigned(K) / 4);
     size_t bytes, slots, o_gen, o_sorted, o_cell, o_values, o_ids, o_assign, o_hist, o_start, o_cb, o_cb32, o_err, o_box, o_state, o_scale;
     size_t o_cur, o_near, o_near_n, o_gap, o_members, o_cells, o_changes;
