@@ -134,6 +134,59 @@ def test_incremental_updates(orc, kind, K, n, iters):
     assert np.array_equal(again["codebook"], out["codebook"]) and np.array_equal(again["trace"], out["trace"])
 
 
+def _repeated_passes(orc, z, K, iters, rel_tol):
+    """Which incremental passes run out of room, by the oracle's assignments and the library's limits: (pass, limit that it meets,
+    incremental updates before it in its batch)."""
+    import os
+    import re
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    src = open(os.path.join(root, "paper_2605_26339_b200", "csrc", "qamw_lloyd.cu")).read()
+    first, again, batch, most = (int(re.search(rf"constexpr int {c} = (\d+);", src)[1])
+                                 for c in ("kFullFirst", "kFullAgain", "kBatch", "kChanges"))
+    n, cb, found = len(z), np.sqrt(2.0) * z[:K], []
+    full, before, in_batch, changes_in_batch, updates, last = first, None, 0, 0, 0, None
+    while True:
+        cell, err = orc.lloyd_assign(z, cb)
+        count = np.bincount(cell, minlength=K)
+        if full == 0:
+            moved = cell != before
+            came, left = np.bincount(cell[moved], minlength=K), np.bincount(before[moved], minlength=K)
+            what = "changes" if max(came.max(), left.max()) > most else "slots" if (size + came > slots)[came > 0].any() else None
+            if what:
+                found.append((updates, what, changes_in_batch))
+                full, in_batch, changes_in_batch = again, 0, 0
+                continue
+            changes_in_batch += 1
+        if last is not None and last - err <= rel_tol * last or updates >= iters:
+            return found
+        last, before, size = err, cell, count
+        updates, in_batch = updates + 1, (in_batch + 1) % batch
+        if in_batch == 0:
+            changes_in_batch = 0
+        total = np.zeros((K, 2))
+        np.add.at(total, cell, z)
+        cb = np.where(count[:, None] > 0, total / np.maximum(count, 1)[:, None], cb)
+        if full and (full := full - 1) == 0:
+            start = np.concatenate([[0], np.cumsum(count)])  # a quarter, and 64 and a quarter of the mean, to grow by
+            slots = np.diff(start + start // 4 + (64 + n // K // 4) * np.arange(K + 1))
+
+
+@pytest.mark.parametrize("K,n,iters,limits", [(128, 60000, 40, {"changes", "slots"}), (64, 20000, 40, {"changes", "slots"}),
+                                              (128, 10000, 60, {"slots"}), (256, 60000, 60, {"changes", "slots"})])
+def test_incremental_passes_that_run_out_of_room(orc, K, n, iters, limits):
+    """Codewords that start in one place: passes in which more samples change cells than a pass may report, or cells outgrow
+    their slots, are repeated in full, once and again: the same codebook, updates and errors as the oracle."""
+    z = np.random.default_rng(K + n).standard_normal((n, 2))
+    z[:K] = 4.0 + 1e-3 * z[:K]
+    repeated = _repeated_passes(orc, z, K, iters, 1e-12)
+    assert len(repeated) > 1 and {what for _, what, _ in repeated} == limits
+    ref_cb, ref_mse, ref_iters, ref_trace = orc.train_codebook_on(z, K, iters, 1e-12)
+    out = q.train_codebook_gpu(K, max_iters=iters, rel_tol=1e-12, samples=torch.from_numpy(z).to(DEV))
+    assert out["iters"] == ref_iters and np.array_equal(out["codebook"], ref_cb)
+    np.testing.assert_allclose(out["trace"], ref_trace, rtol=1e-12)
+    assert abs(out["mse"] - ref_mse) <= 1e-12 * ref_mse
+
+
 def test_samples_still_on_their_way_on_another_stream():
     """Samples that a stream of the caller's is still writing when the call is made: the call waits for them."""
     g = torch.Generator(device=DEV)
