@@ -176,15 +176,14 @@ struct Gemv2Args {
     float inv_sqrt_b;
 };
 
-// One vector: where the rotation has shared memory of its own, or 0: it uses the ring.  (Four vectors carry it too: the compiler's
-// code for 136 bytes of parameters is 2 to 4 % faster there than for 128; for two vectors it is 4 % slower on small matrices.)
+// One vector: where the rotation has shared memory of its own, or 0: it uses the ring.
 struct Gemv2ArgsRot : Gemv2Args {
     int rotate_off;
 };
 
 template <int NVEC>
 struct GemvGeom {
-    typedef std::conditional_t<NVEC == 2, Gemv2Args, Gemv2ArgsRot> Args;
+    typedef std::conditional_t<NVEC == 1, Gemv2ArgsRot, Gemv2Args> Args;
     static constexpr int kThreads = NVEC == 4 ? 320 : NVEC == 2 ? 384 : 512;  // 32 activation registers per thread and vector; warps per scheduler set the register cap
     static constexpr int kDepth = 6;       // staged rows per warp, in pairs: about 40 KB in flight per SM
     static constexpr int kTileRows = 32;   // rows per warp between two block barriers
@@ -320,7 +319,7 @@ __global__ void __launch_bounds__(32 * kRotateWarps) gemv_rotate4_kernel(const G
 
 // BT: bits of an index, or 0 for the widths below 6, read from the arguments
 template <int NVEC, int BT>
-__global__ void __launch_bounds__(GemvGeom<NVEC>::kThreads, 1) gemv2_kernel(const typename GemvGeom<NVEC>::Args a) {
+__device__ __forceinline__ void gemv2_rows(const typename GemvGeom<NVEC>::Args& a) {
     constexpr int R = 2, D = GemvGeom<NVEC>::kDepth;
     constexpr int BMAX = BT ? BT : 5;
     constexpr bool ODD = BT == 0 || BT % 2;                         // a chunk may start in the middle of a word
@@ -498,6 +497,19 @@ __global__ void __launch_bounds__(GemvGeom<NVEC>::kThreads, 1) gemv2_kernel(cons
     }
 }
 
+// The arguments are read where they lie, in constant memory (__grid_constant__), instead of being copied to registers first: at four
+// vectors, whose activations take 128 registers, that is 1 to 7 % faster (eleven shapes at K = 64, 256, 2048 and 4096;
+// 13824 x 5120, K = 2048: 39.8 -> 38.9 us).  At two vectors the copy stays: without it blocks of few rows take longer (2048 x 5632: 12.0 ->
+// 12.5 us), if blocks of many take less (13824 x 5120: 34.2 -> 33.3).
+template <int NVEC, int BT>
+__global__ void __launch_bounds__(GemvGeom<NVEC>::kThreads, 1) gemv2_kernel(const __grid_constant__ typename GemvGeom<NVEC>::Args a) {
+    gemv2_rows<NVEC, BT>(a);
+}
+template <int BT>
+__global__ void __launch_bounds__(GemvGeom<2>::kThreads, 1) gemv2_two_kernel(const GemvGeom<2>::Args a) {
+    gemv2_rows<2, BT>(a);
+}
+
 int gemv_check(const char* what, cudaError_t e) {
     if (e != cudaSuccess) {
         set_cuda_error(what, int(e));
@@ -537,9 +549,12 @@ int gemv_raise_smem(const void* kernel) {
 
 template <int NVEC, int BT>
 int launch_gemv2_b(const typename GemvGeom<NVEC>::Args& a, int blocks, int threads, size_t smem, cudaStream_t st) {
-    int rc = gemv_raise_smem(reinterpret_cast<const void*>(&gemv2_kernel<NVEC, BT>));
-    if (rc) return rc;
-    return gemv_check("gemv2_kernel", launch_chained(gemv2_kernel<NVEC, BT>, blocks, threads, smem, st, a));
+    auto go = [&](auto* kernel) {
+        int rc = gemv_raise_smem(reinterpret_cast<const void*>(kernel));
+        return rc ? rc : gemv_check("gemv2_kernel", launch_chained(kernel, blocks, threads, smem, st, a));
+    };
+    if constexpr (NVEC == 2) return go(&gemv2_two_kernel<BT>);
+    else return go(&gemv2_kernel<NVEC, BT>);
 }
 
 template <int NVEC>
