@@ -14,7 +14,6 @@
 #include <algorithm>
 #include <cmath>
 #include <mutex>
-#include <type_traits>
 #include <unordered_map>
 
 #include "qamw_device.cuh"
@@ -176,14 +175,8 @@ struct Gemv2Args {
     float inv_sqrt_b;
 };
 
-// One vector: where the rotation has shared memory of its own, or 0: it uses the ring.
-struct Gemv2ArgsRot : Gemv2Args {
-    int rotate_off;
-};
-
 template <int NVEC>
 struct GemvGeom {
-    typedef std::conditional_t<NVEC == 1, Gemv2ArgsRot, Gemv2Args> Args;
     static constexpr int kThreads = NVEC == 4 ? 320 : NVEC == 2 ? 384 : 512;  // 32 activation registers per thread and vector; warps per scheduler set the register cap
     static constexpr int kDepth = 6;       // staged rows per warp, in pairs: about 40 KB in flight per SM
     static constexpr int kTileRows = 32;   // rows per warp between two block barriers
@@ -319,7 +312,7 @@ __global__ void __launch_bounds__(32 * kRotateWarps) gemv_rotate4_kernel(const G
 
 // BT: bits of an index, or 0 for the widths below 6, read from the arguments
 template <int NVEC, int BT>
-__device__ __forceinline__ void gemv2_rows(const typename GemvGeom<NVEC>::Args& a) {
+__device__ __forceinline__ void gemv2_rows(const Gemv2Args& a) {
     constexpr int R = 2, D = GemvGeom<NVEC>::kDepth;
     constexpr int BMAX = BT ? BT : 5;
     constexpr bool ODD = BT == 0 || BT % 2;                         // a chunk may start in the middle of a word
@@ -385,13 +378,7 @@ __device__ __forceinline__ void gemv2_rows(const typename GemvGeom<NVEC>::Args& 
         auto fill = [&]() {
             for (int i = 0; i < D / R - 1; ++i) issue();
         };
-        bool early = NVEC == 4;  // the ring is free of the rotation: the first rows travel meanwhile
-        unsigned char* turn = stage;
-        if constexpr (NVEC == 1) {
-            early = a.rotate_off > 0;
-            if (early) turn = smem + a.rotate_off + warp * kRotateStage;
-        }
-        if (early) fill();
+        if (NVEC == 4) fill();  // the ring is free of the rotation: the first rows travel meanwhile
         if (n_rows > 0) {
             if constexpr (NVEC == 4) {
                 const bool valid = 32 * slice + lane < a.n_chunks;
@@ -404,13 +391,13 @@ __device__ __forceinline__ void gemv2_rows(const typename GemvGeom<NVEC>::Args& 
                         xr[v][2 * j + 1] = pack2(q.z, q.w);
                     }
             } else {
-                if (!early)  // the first rows come to the L2 while the ring's memory serves the rotation
-                    for (int i = 0; i < min(n_rows, D) && lane * 128 < seg_len + 15; ++i)
-                        asm volatile("prefetch.global.L2 [%0];" ::"l"(src + i * src_step + min(lane * 128, seg_len - 1)));
-                rotate_slice<NVEC>(a, slice, 0, turn, lane, xr);
+                // the first rows come to the L2 while the ring's memory serves the rotation
+                for (int i = 0; i < min(n_rows, D) && lane * 128 < seg_len + 15; ++i)
+                    asm volatile("prefetch.global.L2 [%0];" ::"l"(src + i * src_step + min(lane * 128, seg_len - 1)));
+                rotate_slice<NVEC>(a, slice, 0, stage, lane, xr);
             }
         }
-        if (!early) fill();
+        if (NVEC != 4) fill();
 
         for (int tile = 0; tile < n_tiles; ++tile) {
             float* ps = ps_base + (tile & 1) * (S_par * TI * NVEC);  // [slice][row of the tile][vector]
@@ -502,11 +489,11 @@ __device__ __forceinline__ void gemv2_rows(const typename GemvGeom<NVEC>::Args& 
 // 13824 x 5120, K = 2048: 39.8 -> 38.9 us).  At two vectors the copy stays: without it blocks of few rows take longer (2048 x 5632: 12.0 ->
 // 12.5 us), if blocks of many take less (13824 x 5120: 34.2 -> 33.3).
 template <int NVEC, int BT>
-__global__ void __launch_bounds__(GemvGeom<NVEC>::kThreads, 1) gemv2_kernel(const __grid_constant__ typename GemvGeom<NVEC>::Args a) {
+__global__ void __launch_bounds__(GemvGeom<NVEC>::kThreads, 1) gemv2_kernel(const __grid_constant__ Gemv2Args a) {
     gemv2_rows<NVEC, BT>(a);
 }
 template <int BT>
-__global__ void __launch_bounds__(GemvGeom<2>::kThreads, 1) gemv2_two_kernel(const GemvGeom<2>::Args a) {
+__global__ void __launch_bounds__(GemvGeom<2>::kThreads, 1) gemv2_two_kernel(const Gemv2Args a) {
     gemv2_rows<2, BT>(a);
 }
 
@@ -548,7 +535,7 @@ int gemv_raise_smem(const void* kernel) {
 }
 
 template <int NVEC, int BT>
-int launch_gemv2_b(const typename GemvGeom<NVEC>::Args& a, int blocks, int threads, size_t smem, cudaStream_t st) {
+int launch_gemv2_b(const Gemv2Args& a, int blocks, int threads, size_t smem, cudaStream_t st) {
     auto go = [&](auto* kernel) {
         int rc = gemv_raise_smem(reinterpret_cast<const void*>(kernel));
         return rc ? rc : gemv_check("gemv2_kernel", launch_chained(kernel, blocks, threads, smem, st, a));
@@ -566,23 +553,13 @@ int launch_gemv2(const Gemv2Args& a, int sms, cudaStream_t st) {
     const int blocks = std::max(1, std::min(sms, a.d_out));
     const int n_b = (a.d_out + blocks - 1) / blocks;  // rows of a block
     const int G = std::max(1, std::min(kWarps / S_par, n_b));
-    typename GemvGeom<NVEC>::Args b{};
-    static_cast<Gemv2Args&>(b) = a;
+    Gemv2Args b = a;
     b.s_par = S_par;
     b.log2c = pick_copies(a.K, (long long)n_b * (a.d_in / 64), size_t(128) * 1024);
     const int threads = 32 * S_par * G;
     const size_t sums = size_t(2) * S_par * GemvGeom<NVEC>::kTileRows * G * NVEC * sizeof(float);
-    size_t smem = (size_t(a.K) * 8 << b.log2c) + size_t(S_par * G) * GemvGeom<NVEC>::kDepth * a.stage_bytes + sums;
+    const size_t smem = (size_t(a.K) * 8 << b.log2c) + size_t(S_par * G) * GemvGeom<NVEC>::kDepth * a.stage_bytes + sums;
     if (smem > kSmemLimit) return QAMW_ERR_NOMEM;
-    // One vector: where there is room beside the ring (a small matrix keeps few copies of the codebook) the rotation leaves the
-    // ring alone: 2048 x 5632 10.40 -> 10.33 us.  Two vectors lose by it (11.96 -> 12.47), four are rotated elsewhere.
-    const size_t rotate_at = (smem + 15) & ~size_t(15), rotate = size_t(S_par * G) * kRotateStage;
-    if constexpr (NVEC == 1) {
-        if (rotate_at + rotate <= kSmemLimit) {
-            b.rotate_off = int(rotate_at);
-            smem = rotate_at + rotate;
-        }
-    }
     switch (a.B) {
         case 6: return launch_gemv2_b<NVEC, 6>(b, blocks, threads, smem, st);
         case 7: return launch_gemv2_b<NVEC, 7>(b, blocks, threads, smem, st);
