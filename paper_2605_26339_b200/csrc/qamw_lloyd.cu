@@ -24,7 +24,7 @@
 // after the last wanted update return at once, and the host reads the errors once per batch.
 //
 // K = 2048 on 2^20 samples, 100 updates on a B200: 235 ms with the exhaustive scan, a serial scan of the histograms
-// and one host round trip per update; 8.6 with five kernels for every update; 5.2 with incremental ones (ms).
+// and one host round trip per update; 8.6 with five kernels for every update; 5.3 with incremental ones (ms).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -782,7 +782,7 @@ constexpr int kNearMost = 1024;  // such a box has up to this many
 constexpr int kEarly = 24, kNearEarly = 4, kNearLate = 8;
 // Cells of up to 1024 + 2 K samples on average (37.7 million at K = 4096: slots are numbered in 32 bits), from 64 cells on: larger and fewer cells leave the merge to a few blocks, and their chains take
 // the time either way.  ms a call in full and incremental: K = 64 on 70001 samples 3.9, 3.2; 128 on 70001 3.7, 2.5, on 2^18 5.2, 5.7 (5.2 in full
-// is kept); 256 on 2^18 4.9, 3.7, on 2^20 10.6, 12.3; 512 on 2^20 9.5, 7.6; 2048 on 2^20 8.6, 5.2; 4096 on 2^20 10.9, 6.9.
+// is kept); 256 on 2^18 4.9, 3.7, on 2^20 10.6, 12.3; 512 on 2^20 9.5, 7.6; 2048 on 2^20 8.6, 5.3; 4096 on 2^20 10.9, 6.9.
 constexpr int kIncrementalK = 64;
 constexpr int kChanges = 512;  // arrivals, and departures, of a cell in one pass
 

@@ -602,10 +602,11 @@ __device__ __forceinline__ void store_indices(const uint2 (&u)[NS], const uint32
 // row's warps -- a named barrier for the norm -- searches its pairs and writes its 16 NS B bytes of the packed
 // row.  W is read once.
 //
-// Bound by the shared-memory pipe and by issue slots, both at 60 %, with too few warps to hide what depends on what: 27.5
+// Bound by the shared-memory pipe and by issue slots, both at 60 %, with too few warps to hide what depends on what: 26.7
 // wavefronts per 32 points (a cell record, 8 random bytes, takes 5.6, the candidate codewords 14: 4 per read from
-// eight copies, the fourth only where there is one; rotation shuffles 3) and 117 instructions.  Four layers of 13B,
-// K = 2048: 4.01 ms with 33.7 wavefronts per 32 points, 3.14 ms now.
+// eight copies, the fourth only where there is one; rotation shuffles 3) and 106 instructions with the default codebook of
+// 2048; 27.5 and 116 with one of 12 updates on 2^15 samples, of whose cells more overflow.  Four layers of 13B with the
+// latter: 4.01 ms with 33.7 wavefronts per 32 points, 3.09 ms now.
 // QUANT: 0 = nearest codeword through the cell table, 1 = polar quantiser, 2 = no quantiser at all:
 // the kernel then is the calibration pass of Section 3.4, which visits n = min(d_out, 1024) rows
 // floor(t d_out / n) and adds up the pair moduli |(y_2k, y_2k+1)| per pair position.  The row groups of a
